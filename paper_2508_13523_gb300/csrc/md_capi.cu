@@ -16,6 +16,7 @@
 #include "md_integrate.cuh"
 #include "md_internal.cuh"
 #include "md_pair.cuh"
+#include "md_pair_fx.cuh"
 #include "md_pair_q.cuh"
 
 // md_step_fused.cu
@@ -101,6 +102,7 @@ int setup_geometry(md_ctx* c, const double* boxes) {
   for (int k = 0; k < 3 * c->nrep; k++) lmax = boxes[k] > lmax ? boxes[k] : lmax;
   int pe = 0;
   frexp(1.25 * lmax, &pe);
+  c->lmax = lmax;
   const double P = ldexp(1.0, pe);
   c->xgrid.k = pe - 24;
   for (int r = 0; r < c->nrep; r++) {
@@ -127,6 +129,17 @@ int setup_geometry(md_ctx* c, const double* boxes) {
         int E = 0;
         frexp(lm, &E);  // lm < 2^E
         g.xfix = 61 - E;
+      }
+      if (a == 2) {
+        for (int k = 0; k < 3; k++) {
+          // ldexp is exact; Lx < 2^61
+          const double L = g.L[k], lim = ldexp(1.0, c->fxR + g.xfix);
+          g.Lx[k] = (long long)floor(ldexp(L, g.xfix));
+          g.hx[k] = (long long)floor(ldexp(L, g.xfix - 1));
+          const double h = lim < (double)g.hx[k] ? lim : (double)g.hx[k];
+          const int gh = (int)floor(ldexp(h, -32));
+          if (k == 0 || gh < g.gh) g.gh = gh;
+        }
       }
       g.lo[a] = g.nc[a] >= 3 ? -1 : 0;
       g.hi[a] = g.nc[a] >= 3 ? 1 : 0;
@@ -205,6 +218,135 @@ void md_set_coef(PairCoef& pc, double eps, double sigma, double rc, double qq,
   pc.lj4f = (float)pc.lj4;
 }
 
+namespace {
+
+// A number as the unevaluated sum of two doubles (106 bits), for coefficients
+// of more than 53 bits.  The product's error term is exact (one FMA).
+struct Dd {
+  double h, l;
+};
+Dd dd_mul(Dd a, Dd b) {
+  const double p = a.h * b.h;
+  const double e = fma(a.h, b.h, -p) + (a.h * b.l + a.l * b.h);
+  const double h = p + e;
+  return {h, e - (h - p)};
+}
+Dd dd_div(Dd a, Dd b) {
+  const double q = a.h / b.h;
+  const double r = fma(-q, b.h, a.h) + (a.l - q * b.l);
+  const double e = r / b.h;
+  const double h = q + e;
+  return {h, e - (h - q)};
+}
+// a 2^s rounded to an integer
+long long dd_fixed(Dd a, int s) {
+  const double h = ldexp(a.h, s), f = floor(h);
+  return (long long)f + llrint((h - f) + ldexp(a.l, s));
+}
+
+}  // namespace
+
+// Eq. 1's fixed-point coefficients of one type pair (md_fx.cuh).
+static void set_fx(PairFx& p, double eps, double sigma, double rc, int R, double lmax) {
+  memset(&p, 0, sizeof(p));
+  // exact sigma^2 as m 2^e, m < 2^106
+  int es = 0;
+  const unsigned __int128 ms = (unsigned long long)ldexp(frexp(sigma, &es), 53);
+  const unsigned __int128 m = ms * ms;
+  const int e = 2 * (es - 53);
+  // m 2^(e + s), rounded, for results below 2^63
+  auto scaled = [&](int s) {
+    const int sh = -(e + s);
+    if (sh <= 0) return (unsigned long long)(m << -sh);
+    if (sh > 110) return 0ULL;
+    return (unsigned long long)((m + ((unsigned __int128)1 << (sh - 1))) >> sh);
+  };
+  const double ratio = ldexp(1.0, 2 * R) / (sigma * sigma);  // 4^R / sigma^2
+  p.e2 = 2.0 * eps;
+  p.smin = ~0u;  // nothing in fixed point
+  // cutoff band: r^2 here (4 units, positions within 2^-53), fma(dz,dz,
+  // fma(dy,dy, dx*dx)) on FP64 separations of coordinates up to 1.25 lmax
+  const double su = ldexp(1.0, 62 - 2 * R), sc = rc * rc * su;
+  const double band = ldexp(sc, -44) + rc * lmax * ldexp(su, -47) + 64.0;
+  p.cut_lo = sc - band > 0.0 ? (unsigned int)floor(ldexp(sc - band, -32)) : 0u;
+  p.cut_hi = sc + band < ldexp(1.0, 63) ? (unsigned int)ceil(ldexp(sc + band, -32)) : ~0u;
+  if (!(ratio < ldexp(1.0, 40)) || !(ratio > ldexp(1.0, -2)) || !(band < 0.25 * sc)) return;
+  // largest tau with |F| below the accumulators' range for every smaller one
+  // (|F| = 24 eps / sigma tau^3.5 |2 tau^3 - 1|, largest of the attractive
+  // branch 2.397 eps / sigma at tau^3 = 7 / 26)
+  const double fs = 24.0 * eps / sigma, flim = ldexp(1.0 - ldexp(1.0, -10), MD_FIX_EMAX + 1);
+  auto force = [&](double t) { return fs * pow(t, 3.5) * fabs(2.0 * t * t * t - 1.0); };
+  const double ta = pow(7.0 / 26.0, 1.0 / 3.0);
+  double lo = 0.0, hi = MD_FX_TAU_MAX;
+  if (force(ta) > flim) {
+    hi = ta;
+  } else if (force(hi) <= flim) {
+    lo = hi;
+  } else {
+    lo = ta;
+  }
+  for (int k = 0; k < 60 && lo < hi; k++) {
+    const double mid = 0.5 * (lo + hi);
+    (force(mid) <= flim ? lo : hi) = mid;
+  }
+  const double tl = lo * (1.0 - 1e-9);
+  if (!(tl > 1e-3)) return;
+  // z = tau^4 (2 tau^3 - 1) over tau < tl: smallest -0.0806 at tau^3 = 2 / 7
+  const double tm = pow(2.0 / 7.0, 1.0 / 3.0);
+  auto zabs = [](double t) { return t * t * t * t * fabs(2.0 * t * t * t - 1.0); };
+  double zmax = zabs(tl);
+  if (tl > tm && zabs(tm) > zmax) zmax = zabs(tm);
+  int ze = 0;
+  frexp(zmax * 1.001, &ze);  // zmax < 2^ze
+  p.zsh = 7 - ze < 0 ? 0 : 7 - ze;
+  const Dd s2 = dd_mul({sigma, 0.0}, {sigma, 0.0}), s6 = dd_mul(s2, dd_mul(s2, s2));
+  const Dd c6 = dd_mul(dd_mul({24.0, 0.0}, {eps, 0.0}), s6);
+  const Dd cc = dd_div(dd_mul({24.0, 0.0}, {eps, 0.0}), s2);  // C
+  int ce = 0;
+  frexp(cc.h, &ce);
+  const int cx = 62 - ce;
+  p.cm = dd_fixed(cc, cx);
+  p.sh = cx - 8 + p.zsh - 45 - R;
+  if (p.sh > 12) {  // small forces: more bits than the counts can use
+    const int d = p.sh - 12;
+    p.cm = d < 62 ? p.cm >> d : 0;
+    p.sh = 12;
+  }
+  if (p.sh < 1) return;
+  p.B = 0;
+  while (ldexp(1.0, p.B) < 1.001 * MD_FX_TAU_MAX * ratio) p.B++;
+  if (p.B <= MD_FX_BMAX) {
+    const double q = ldexp(1.0, p.B) / ratio;  // s 2^B, in (1.5, 3.1)
+    // C q^4 = 24 eps sigma^6 2^(4B - 8R) = kf 2^ke; k2 in [2^55, 2^56], k1 = 4 k2 q^3
+    int ke = 0;
+    frexp(ldexp(c6.h, 4 * p.B - 8 * R), &ke);
+    p.k2 = dd_fixed(c6, 4 * p.B - 8 * R + 56 - ke);
+    p.k1 = dd_fixed(dd_mul(c6, s6), 4 * p.B - 8 * R + 56 - ke + 2 + 3 * p.B - 6 * R);
+    // |w| = 4 k2 (tau / q)^3 |2 tau^3 - 1| < 2^58 wmax
+    double wmax = 0.0;
+    for (int k = 1; k <= 256; k++) {
+      const double t = tl * k / 256.0, x = t / q;
+      wmax = fmax(wmax, x * x * x * fabs(2.0 * t * t * t - 1.0));
+    }
+    int we = 0;
+    frexp(wmax * 1.02, &we);
+    p.zsh1 = 5 - we < 0 ? 0 : 5 - we;  // |w 2^zsh1| < 2^63
+    p.sh1 = 57 + p.zsh1 - ke - 45 - R;  // P = fpair 2^(57 + zsh1 - ke)
+    if (p.sh1 > 12) {
+      const int d = p.sh1 - 12;
+      p.k1 = d < 62 ? p.k1 >> d : 0;
+      p.k2 = d < 62 ? p.k2 >> d : 0;
+      p.sh1 = 12;
+    }
+    if (p.sh1 < 1) p.B = MD_FX_BMAX + 1;  // the general form
+  }
+  int c = 0;
+  while (scaled(c + 1 - 2 * R) < (1ULL << 63)) c++;  // sigma^2 / 4^R 2^c in [2^62, 2^63)
+  p.csign = scaled(c - 2 * R);
+  p.tsh = c - 62;
+  p.smin = (unsigned int)ceil(ldexp(1.0, 30) / (ratio * tl)) + 1;
+}
+
 // Coefficient table (device), the single-type copy, and the FP32 cutoff
 // bounds (device copy for the compacted kernel).  Synchronizes: the host
 // table must outlive the copies.
@@ -213,13 +355,18 @@ int md_upload_coef(md_ctx* c) {
   set_cut_bounds(c);
   PairCoef tab[MD_MAX_TYPES * MD_MAX_TYPES];
   memset(tab, 0, sizeof(tab));
+  PairFx fx[MD_MAX_TYPES * MD_MAX_TYPES];
+  memset(fx, 0, sizeof(fx));
   for (int a = 0; a < nt; a++)
     for (int b = 0; b < nt; b++) {
       const int k = a * nt + b;
+      set_fx(fx[k], c->eps[k], c->sigma[k], c->rc[k], c->fxR, c->lmax);
       const double qq = c->coul ? c->qqrd2e * c->qtype[a] * c->qtype[b] : 0.0;
       md_set_coef(tab[k], c->eps[k], c->sigma[k], c->rc[k], qq, c->coul ? c->rc_coul : 0.0);
     }
   c->coef1 = tab[0];
+  c->fx1 = fx[0];
+  MD_CUDA(cudaMemcpyAsync(c->fxt, fx, sizeof(fx), cudaMemcpyHostToDevice, c->stream));
   MD_CUDA(cudaMemcpyAsync(c->coef, tab, sizeof(tab), cudaMemcpyHostToDevice, c->stream));
   MD_CUDA(cudaMemcpyAsync(c->cut_hi_dev, c->geo.cut_hi, sizeof(c->geo.cut_hi),
                           cudaMemcpyHostToDevice, c->stream));
@@ -284,7 +431,7 @@ void free_ctx(md_ctx* c) {
                   c->scan_tmp, c->numneigh, c->nbr,  c->ev,       c->dmax,    c->i64_tmp,
                   c->stage,  c->rep,     c->vcoef,    c->adj_c,    c->adj_xbar, c->adj_vbar,
                   c->adj_carry, c->seg_x, c->gbar,     c->fmax_bits, c->cut_hi_dev,
-                  c->tile_ctr, c->fix,   c->xq,       c->evs};
+                  c->tile_ctr, c->fix,   c->xq,       c->evs,       c->fxt};
   for (void* b : bufs)
     if (b) cudaFree(b);
   if (c->pair_ev) {
@@ -332,12 +479,19 @@ int md_fresh_start(md_ctx* c) {
 
 namespace {
 
-// One cooperative launch: K21 (or K1) of every atom, a grid barrier, the
-// forces (md_step_fused.cu).
-int launch_fused(md_ctx* c, int mode) {
-  const IntArgs ia = md_int_args(c, md_pair_fixed(c), md_pair_accumulates(c));
+// The fixed-point kernel keeps contributions below 2^(MD_FIX_EMAX + 1); an
+// atom that may receive k >= 2^11 of them needs contributions below 2^(63 -
+// MD_FIX_BITS) / k.  Returns log2 of the factor (the force falls at least as
+// r^-7, so a larger smin by that factor does it).
+int fx_dense(const md_ctx* c) {
+  int kb = 0;
+  while (kb < 31 && ((unsigned)c->kmax >> kb)) kb++;
+  const int d = kb - (63 - MD_FIX_BITS - (MD_FIX_EMAX + 1));
+  return d > 0 ? d : 0;
+}
+
+PairArgs pair_args(md_ctx* c) {
   PairArgs a;
-  memset(&a, 0, sizeof(a));
   a.x4 = c->x4;
   a.xs = c->xs;
   a.xq = c->xq;
@@ -347,6 +501,16 @@ int launch_fused(md_ctx* c, int mode) {
   a.fix = c->fix;
   a.kmax = c->dmax + 2;
   a.coef = c->coef;
+  a.fxt = c->fxt;
+  a.fx1 = c->fx1;
+  a.fxR = c->fxR;
+  a.fx_dense = fx_dense(c);
+  if (a.fx_dense)
+    a.fx1.smin = a.fx_dense < __builtin_clz(a.fx1.smin) ? a.fx1.smin << a.fx_dense : ~0u;
+  a.nrep = c->nrep;
+  // one type: at most maxneigh + 64 terms x^3 2^62 < 2^62 in 64 bits
+  a.ev_shift = 0;
+  while (a.ev_shift < 32 && (int64_t)c->maxneigh + 64 > (4LL << a.ev_shift)) a.ev_shift++;
   a.c1 = c->coef1;
   a.rep = c->rep;
   a.ev = c->evs;
@@ -355,8 +519,28 @@ int launch_fused(md_ctx* c, int mode) {
   a.nt = c->nt;
   a.maxneigh = c->maxneigh;
   a.nslots = c->nsm;
+  a.tile_ctr = nullptr;
+  return a;
+}
+
+// The fixed-point kernel's one-type form: its range of 4^R / sigma^2.
+bool fx_single(const md_ctx* c) { return c->nt == 1 && c->fx1.B <= MD_FX_BMAX; }
+
+// Lanes per atom of the fixed-point kernel.  Few atoms: more lanes shorten
+// each lane's chain of dependent loads and fill the SMs; many atoms: two lanes
+// share a row's tail (1, 2, 4 and 8 lanes, force-only half list: 4,000 atoms
+// 38, 24, 17 and 14 us; 32,000 atoms 42, 31, 27 and 27 us; 108,000 atoms 68,
+// 62, 60 and 64 us; 256,000 atoms 134, 117, 122 and 138 us; 4,000,000 atoms
+// 1.470, 1.464, 1.70 and 2.00 ms).
+int fx_lanes(const md_ctx* c) { return c->n < 16000 ? 8 : c->n < 160000 ? 4 : 2; }
+
+// One cooperative launch: K21 (or K1) of every atom, a grid barrier, the
+// forces (md_step_fused.cu).
+int launch_fused(md_ctx* c, int mode) {
+  const IntArgs ia = md_int_args(c, md_pair_fixed(c), md_pair_accumulates(c));
+  PairArgs a = pair_args(c);
   a.tile_ctr = c->tile_ctr;
-  cudaError_t e = md_step_fused_launch(ia, a, mode, c->list_kind == MD_LIST_HALF, c->nt == 1,
+  cudaError_t e = md_step_fused_launch(ia, a, mode, c->list_kind == MD_LIST_HALF, fx_single(c),
                                        c->geo.cut_hi[0], c->cut_hi_dev, c->dmax + 6,
                                        c->dmax + 5, c->stream);
   c->launches++;
@@ -495,6 +679,7 @@ int create_impl(const md_params* p, int nrep, const int64_t* rep_off, const doub
     c->dtf[t] = 0.5 * c->dt / c->mass[t];
   }
   c->rlist = rcmax + c->skin;
+  if (frexp(rcmax, &c->fxR) == 0.5) c->fxR--;  // rcmax <= 2^fxR
   c->rep_host = new (std::nothrow) RepGeo[nrep];
   c->rep_off_host = new (std::nothrow) int64_t[nrep + 1];
   c->graphs = new (std::nothrow) std::map<GraphKey, std::pair<cudaGraphExec_t, int>>();
@@ -525,6 +710,7 @@ int create_impl(const md_params* p, int nrep, const int64_t* rep_off, const doub
   if (rc == MD_OK) rc = dalloc(&c->tag0, n);
   if (rc == MD_OK) rc = dalloc(&c->coef, MD_MAX_TYPES * MD_MAX_TYPES);
   if (rc == MD_OK) rc = dalloc(&c->cut_hi_dev, MD_MAX_TYPES * MD_MAX_TYPES);
+  if (rc == MD_OK) rc = dalloc(&c->fxt, MD_MAX_TYPES * MD_MAX_TYPES);
   if (rc == MD_OK) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -606,7 +792,10 @@ int create_impl(const md_params* p, int nrep, const int64_t* rep_off, const doub
 // -(lj4 / 2) r^-6 and leave fpair r^2 / 12 (lj1 = 12 lj3, lj2 = 6 lj4) to
 // the virial: the potential energy is then ev[0] + trace(W) / 12.
 double md_ev_trace_share(const md_ctx* c) {
-  return (c->precision == MD_PREC_FP64 && c->nt == 1 && !c->coul) ? 1.0 / 12.0 : 0.0;
+  return (c->precision == MD_PREC_FP64 && c->nt == 1 && !c->coul &&
+          !(c->compact == 2 && !fx_single(c)))
+             ? 1.0 / 12.0
+             : 0.0;
 }
 
 // Pair energies/virials and kinetic energies per replica into ev_host.
@@ -655,24 +844,7 @@ namespace {
 // forces, so it is only asked for with the fold in this call.
 int launch_pair_impl(md_ctx* c, int ev, int tpa, int prezeroed, int defer_fold) {
   if (ev && defer_fold) return MD_EINVAL;
-  PairArgs a;
-  a.x4 = c->x4;
-  a.xs = c->xs;
-  a.xq = c->xq;
-  a.numneigh = c->numneigh;
-  a.nbr = c->nbr;
-  a.f = c->f;
-  a.fix = c->fix;
-  a.kmax = c->dmax + 2;
-  a.coef = c->coef;
-  a.c1 = c->coef1;
-  a.rep = c->rep;
-  a.ev = c->evs;
-  a.ev_spread = c->ev_spread;
-  a.n = c->n;
-  a.nt = c->nt;
-  a.maxneigh = c->maxneigh;
-  a.nslots = c->nsm;
+  PairArgs a = pair_args(c);
   a.tile_ctr = c->persist ? c->tile_ctr : nullptr;
   if (c->persist)
     MD_CUDA(cudaMemsetAsync(c->tile_ctr, 0, sizeof(int) * c->nsm, c->stream));
@@ -690,9 +862,8 @@ int launch_pair_impl(md_ctx* c, int ev, int tpa, int prezeroed, int defer_fold) 
         c->coul ? md_pair_q_coul_launch(a, fix, half, ev != 0, c->nt == 1, c->geo.cut_hi[0],
                                         c->cut_hi_dev, (unsigned)md_blocks(c->n), c->stream,
                                         c->carve)
-                : fix ? md_pair_q_fix_launch(a, half, ev != 0, c->nt == 1, c->geo.cut_hi[0],
-                                             c->cut_hi_dev, (unsigned)md_blocks(c->n),
-                                             c->stream, c->carve, c->qu)
+                : fix ? md_pair_fx_launch(a, half, ev != 0, fx_single(c), fx_lanes(c), c->qu,
+                                          c->geo.cut_hi[0], c->cut_hi_dev, c->stream, c->carve)
                       : md_pair_q_launch(a, half, ev != 0, c->nt == 1, c->geo.cut_hi[0],
                                          c->cut_hi_dev, (unsigned)md_blocks(c->n), c->stream,
                                          c->carve);

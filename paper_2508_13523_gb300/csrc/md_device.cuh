@@ -230,17 +230,19 @@ __device__ __forceinline__ void md_split(double x, const XGrid& g, float& hi, fl
   lo = __double2float_rn(__dsub_rn(x, md_widen(hi)));
 }
 
-// x as a fixed-point count X = x 2^F when that is exact and |x| < 2^(61 - F)
-// (so |X| < 2^61); false otherwise.  Integer instructions only.  x = M
-// 2^(e - 1075) with M the 53-bit significand: X = M 2^(e - 1075 + F), an
-// integer iff e - 1075 + F >= 0 or the low 1075 - F - e bits of M are zero.
+// x as a fixed-point count X = x 2^F, |x| < 2^(61 - F) (so |X| < 2^61); false
+// beyond that range (and for infinities and NaNs).  Integer instructions only.
+// x = M 2^(e - 1075) with M the 53-bit significand: X = M 2^(e - 1075 + F),
+// an integer for |x| >= 2^(52 - F).  Smaller x are rounded to the nearest
+// multiple of 2^-F where F >= MD_XFIX_ROUND_F (an error of at most 2^-53, no
+// more than FP64's own rounding of a separation above 1); with a coarser
+// grid (boxes of more than 409 length units) they must be exact, else false.
+#define MD_XFIX_ROUND_F 52
 __device__ __forceinline__ bool md_xfix(double x, int F, long long& X) {
   const long long b = __double_as_longlong(x);
   const int e = (int)((b >> 52) & 0x7ff);
-  if (e == 0) {  // zero (subnormals are never positions)
-    X = 0;
-    return (b & 0x7fffffffffffffffLL) == 0;
-  }
+  X = 0;
+  if (e == 0) return true;  // zero (or subnormal: rounds to it)
   if (e - 1023 >= 61 - F) return false;  // |x| >= 2^(61 - F)
   const long long M = (b & 0xfffffffffffffLL) | (1LL << 52);
   const int sh = 1075 - F - e;
@@ -248,8 +250,8 @@ __device__ __forceinline__ bool md_xfix(double x, int F, long long& X) {
   if (sh <= 0) {
     m = M << (-sh);  // -sh <= 8: |x| < 2^(61 - F)
   } else {
-    if (sh > 52 || (M & ((1LL << sh) - 1)) != 0) return false;
-    m = M >> sh;
+    if (F < MD_XFIX_ROUND_F && (sh > 52 || (M & ((1LL << sh) - 1)) != 0)) return false;
+    m = sh > 53 ? 0 : (M + (1LL << (sh - 1))) >> sh;
   }
   X = b < 0 ? -m : m;
   return true;
@@ -257,8 +259,8 @@ __device__ __forceinline__ bool md_xfix(double x, int F, long long& X) {
 
 // Store the position p of atom i into its derived records: the double-float
 // split (md_split; tag in hi.w) and, where xq is given (FP64 contexts), the
-// fixed-point record, with MD_TAG_OFFGRID in the split's tag when some
-// coordinate has no exact fixed-point form.  FP64 contexts keep only the hi
+// fixed-point record, with MD_TAG_OFFGRID in its tag when some coordinate has
+// no fixed-point form.  FP64 contexts keep only the hi
 // parts of the split (lo = 0).  Returns the split.
 __device__ __forceinline__ XSplit md_store_pos(const double4_32a& p, const XGrid& gr,
                                                XSplit* __restrict__ xs, XFix* __restrict__ xq,
@@ -315,16 +317,15 @@ __device__ __forceinline__ XSplit md_store_pos(const double4_32a& p, const XGrid
     md_split(p.z, gr, s.hi.z, s.lo.z);
   }
   const int tag = md_tag_of(p);
-  int stag = tag;
-  if (xq) {  // FP64 contexts: the compacted kernel's fixed-point record
+  if (xq) {  // FP64 contexts: the fixed-point kernel's record
     XFix q;
     const int F = gr.rep[MD_TAG_REP(tag)].xfix;
     const bool on = md_xfix(p.x, F, q.x) & md_xfix(p.y, F, q.y) & md_xfix(p.z, F, q.z);
-    q.w = (long long)(unsigned int)tag | ((long long)F << 32);
+    if (!on) q.x = q.y = q.z = 1LL << 62;  // farther than 2^61 from every position
+    q.w = (long long)(unsigned int)(on ? tag : tag | MD_TAG_OFFGRID) | ((long long)F << 32);
     xq[i] = q;
-    if (!on) stag |= MD_TAG_OFFGRID;
   }
-  s.hi.w = __int_as_float(stag);
+  s.hi.w = __int_as_float(tag);
   s.lo.w = 0.f;
   xs[i] = s;
   if (xb) xb[i] = s;
@@ -347,80 +348,6 @@ __device__ __forceinline__ float md_disp2(const XSplit& s, const XSplit& b, cons
   const float step = __int_as_float((gr.k + 127) << 23);  // 2^k
   const float d = __fmaf_rn(sqrtf(d2), 1.f + 0x1p-20f, 4.f * step);
   return d * d;
-}
-
-// ---- the compacted FP64 kernel's integer path (XFix positions) --------------
-//
-// A pair's separation is D = X_j - X_i per axis (units 2^-F, |D| < 2^60
-// for pairs closer than half the box).  The three |D| share one left shift
-// sh that puts the largest at bit 60: A = |D| 2^sh < 2^61.  Products are
-// then taken as the high 64 bits of 64 x 64-bit products (__umul64hi), whose
-// truncation is below one unit of a result of 56 to 61 significant bits.
-
-// |d| of a separation count.
-__device__ __forceinline__ unsigned long long md_uabs(long long d) {
-  return d < 0 ? (unsigned long long)(-d) : (unsigned long long)d;
-}
-
-// The common shift sh (>= 0) and the shifted magnitudes A = |D| 2^sh, and
-// r^2 = (Dx^2 + Dy^2 + Dz^2) 2^-2F as a double, truncated: the sum of the
-// three high products S is within 3 units below the exact sum 2^(2 sh - 64)
-// (S ~ 2^56 or more for pairs near the cutoff), and S is truncated once
-// more to 53 bits, so the result lies within 1.1 ulps below the exact r^2.
-// Integer instructions only.
-__device__ __forceinline__ double md_sep_r2(long long Dx, long long Dy, long long Dz, int F,
-                                            unsigned long long& Ax, unsigned long long& Ay,
-                                            unsigned long long& Az, int& sh) {
-  Ax = md_uabs(Dx);
-  Ay = md_uabs(Dy);
-  Az = md_uabs(Dz);
-  const unsigned long long am = Ax | Ay | Az;
-  if (am == 0) {  // coincident atoms
-    sh = 0;
-    return 0.0;
-  }
-  sh = __clzll((long long)am) - 3;  // am < 2^61: sh >= 0, leading one to bit 60
-  Ax <<= sh;
-  Ay <<= sh;
-  Az <<= sh;
-  const unsigned long long S = __umul64hi(Ax, Ax) + __umul64hi(Ay, Ay) + __umul64hi(Az, Az);
-  // r^2 = S 2^(64 - 2 sh - 2 F); S > 0 (its largest term is >= 2^56)
-  const int lz = __clzll((long long)S);
-  const unsigned long long m = (S << lz) >> 11;  // 53 bits, leading one at bit 52
-  const long long e = 1150 - 2 * F - lz - 2 * sh;  // biased exponent of the result
-  return __longlong_as_double(((e - 1) << 52) + (long long)m);
-}
-
-// The fixed-point count (units 2^-MD_FIX_BITS) of the contribution f d, with
-// d = +-A 2^(-F - sh) (A and sh from md_sep_r2, neg: d < 0): the high 64
-// bits H of the product of f's significand (at bit 63) and A, rounded to the
-// nearest count.  Within one count of the exact f d 2^44 (the truncated low
-// bits weigh below 2^-7 counts for any count in range).  False, leaving q
-// unset, when |q| >= 2^qbits (the accumulators' range) or f is not finite.
-// Integer instructions only.
-__device__ __forceinline__ bool md_fix_prod(double f, unsigned long long A, bool neg, int sh,
-                                            int F, int qbits, long long& q) {
-  static_assert(MD_FIX_BITS == 44, "the exponent 978 below");
-  const long long b = __double_as_longlong(f);
-  const int e = (int)((b >> 52) & 0x7ff);
-  if (e == 0x7ff) return false;
-  if (e == 0) {
-    q = 0;
-    return true;
-  }
-  const unsigned long long Mn = ((unsigned long long)b << 11) | (1ULL << 63);
-  const unsigned long long H = __umul64hi(Mn, A);  // < 2^61
-  // |f d| 2^44 = Mn A 2^(e - 1042 - F - sh) = H 2^(e - 978 - F - sh) (+ the
-  // low half)
-  const int s = 978 + F + sh - e;
-  if (s <= 0) return false;
-  unsigned long long r = 0;
-  if (s < 64) {
-    r = (H + (1ULL << (s - 1))) >> s;
-    if ((r >> qbits) != 0) return false;
-  }
-  q = ((b < 0) != neg) ? -(long long)r : (long long)r;
-  return true;
 }
 
 // r^2 in FP64 from the position splits: the hi parts' difference and image

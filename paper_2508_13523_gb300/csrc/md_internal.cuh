@@ -13,6 +13,7 @@
 #include <utility>
 
 #include "../../include/md.h"
+#include "md_fx.cuh"
 
 #define MD_BLOCK 128     // threads per block of every per-atom kernel
 #define MD_EV_STRIDE 16  // doubles per replica in the energy accumulators
@@ -72,6 +73,10 @@ struct RepGeo {
   int cell_base;            // first global cell of this replica
   int xfix;                 // fixed-point scale F of its positions (XFix): 61 - E
                             // with 2^E >= 1.25 x the largest edge
+  // fixed-point kernel (md_pair_fx.cuh), all in units of 2^-xfix:
+  long long Lx[3], hx[3];   // L and L / 2, rounded down
+  int gh;                   // min(2^R, L / 2 over the axes) >> 32: separations whose
+                            // high words are below it need no image
 };
 
 // Linear cell index: cells are ordered brick by brick (4 x 4 x 4 cells,
@@ -178,6 +183,10 @@ struct md_ctx {
   double qqrd2e, rc_coul;
   double dtf[MD_MAX_TYPES];  // 0.5 dt / m per type
   PairCoef coef1;            // coefficients when nt == 1
+  PairFx fx1;                // fixed-point coefficients when nt == 1
+  PairFx* fxt;               // nt*nt fixed-point coefficients (device)
+  int fxR;                   // largest rc <= 2^fxR
+  double lmax;               // largest box edge
   Geo geo;
   int nrep;                  // replicas
   RepGeo* rep;               // device, nrep
@@ -259,6 +268,7 @@ struct md_ctx {
   // counters
   int64_t step, builds, dangerous, launches;
   int32_t max_count;
+  uint32_t kmax;           // dmax[2] of the last build
   int64_t pairs_in_range;  // at the last md_energy
 };
 

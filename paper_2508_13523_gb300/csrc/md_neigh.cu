@@ -498,13 +498,19 @@ int md_rebuild(md_ctx* c) {
   MD_CUDA(cudaMemsetAsync(c->dmax, 0, sizeof(unsigned int), s));
   for (int attempt = 0; attempt < 4; attempt++) {
     MD_TRY(launch_build(c));
-    MD_CUDA(cudaMemcpyAsync(c->h_pinned + 9, c->dmax + 1, sizeof(unsigned int),
+    MD_CUDA(cudaMemcpyAsync(c->h_pinned + 9, c->dmax + 1, 2 * sizeof(unsigned int),
                             cudaMemcpyDeviceToHost, s));
     MD_CUDA(cudaStreamSynchronize(s));
     MD_TRY(md_barrier_status(c));
     unsigned int mc;
     memcpy(&mc, (const char*)(c->h_pinned + 9), sizeof(mc));
     c->max_count = (int32_t)mc;
+    uint32_t kmax;
+    memcpy(&kmax, (const char*)(c->h_pinned + 9) + sizeof(mc), sizeof(kmax));
+    // captured graphs hold the range that follows from it (fx_dense)
+    if ((kmax | c->kmax) >= (1u << (63 - MD_FIX_BITS - (MD_FIX_EMAX + 1))) && kmax != c->kmax)
+      md_drop_graphs(c);
+    c->kmax = kmax;
     if ((int)mc <= c->maxneigh) {
       unsigned int disp_bits;
       memcpy(&disp_bits, (const char*)(c->h_pinned + 8), sizeof(disp_bits));

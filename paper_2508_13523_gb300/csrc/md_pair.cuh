@@ -44,12 +44,13 @@
 #include <type_traits>
 
 #include "md_device.cuh"
+#include "md_fx.cuh"
 #include "md_internal.cuh"
 
 struct PairArgs {
   const double4_32a* x4;
   const XSplit* xs;
-  const XFix* xq;        // fixed-point positions (compacted FP64 kernel's integer path)
+  const XFix* xq;        // fixed-point positions (FP64 contexts' fixed-point kernel)
   const int32_t* numneigh;
   const int32_t* nbr;
   double* f;            // SoA fx[n], fy[n], fz[n]
@@ -57,6 +58,12 @@ struct PairArgs {
                              // k_pair); zero at entry of a half-list launch
   const unsigned int* kmax;  // bound on the contributions one atom receives
   const PairCoef* coef;  // nt*nt table (multi-type)
+  const PairFx* fxt;     // the fixed-point kernel's nt*nt table
+  PairFx fx1;            // and its only entry when nt == 1
+  int fxR;               // largest cutoff <= 2^fxR
+  int fx_dense;          // smin of the table is scaled by 2^fx_dense
+  int nrep;
+  int ev_shift;          // one type: sums of x^3 (md_fx_force1) in units of 2^(ev_shift - 62)
   PairCoef c1;           // the only coefficients when nt == 1
   const RepGeo* rep;     // box of each replica
   double* ev;            // per-replica accumulators: ev_spread rows of MD_EV_STRIDE

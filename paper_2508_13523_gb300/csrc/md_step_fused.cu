@@ -1,7 +1,7 @@
 // md_step_fused.cu -- one launch per velocity-Verlet step: the integrator's
 // kick-drift (K1 or K21) of every atom, a grid-wide barrier, then the pair
-// forces of every tile at the new positions (the compacted FP64 kernel with
-// fixed-point sums, persistent tile scheduling).  For a batch of replicas
+// forces of every tile at the new positions (the fixed-point kernel,
+// persistent tile scheduling).  For a batch of replicas
 // the launch covers all of them: uneven boxes share one grid.
 //
 // The launch is cooperative (all blocks resident at once), so the barrier
@@ -20,7 +20,7 @@
 #include "md_integrate.cuh"
 #include "md_internal.cuh"
 #include "md_pair.cuh"
-#include "md_pair_q.cuh"
+#include "md_pair_fx.cuh"
 
 namespace {
 
@@ -86,8 +86,8 @@ __device__ __noinline__ void integrate_all(const IntArgs& ia) {
 }
 
 template <int MODE, bool HALF, bool SINGLE>
-__global__ void __launch_bounds__(MD_BLOCK, md_pair_q_minb(true, false, true, false, 1))
-    k_step_fused(const IntArgs ia, const PairArgs a, const float cut_hi1,
+__global__ void __launch_bounds__(MD_BLOCK, MD_FX_MINB)
+    k_step_fused(const IntArgs ia, const __grid_constant__ PairArgs a, const float cut_hi1,
                  const float* __restrict__ cut_hi_tab, unsigned int* bar, unsigned int* err) {
   integrate_all<MODE>(ia);
   if (blockIdx.x == 0)  // the pair phase's tile counters start at zero
@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(MD_BLOCK, md_pair_q_minb(true, false, true, fa
   __threadfence();
   if (!grid_barrier(bar, err, gridDim.x, BARRIER_LIMIT_NS)) return;
   // phase 2: the forces at the new positions
-  md_pair_q_tiles<HALF, false, SINGLE, true, false, 1>(a, cut_hi1, cut_hi_tab);
+  md_pair_fx_tiles<HALF, false, SINGLE, 1, 1>(a, cut_hi1, cut_hi_tab);
 }
 
 template <int MODE, bool HALF, bool SINGLE>
