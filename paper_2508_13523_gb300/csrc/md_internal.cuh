@@ -193,6 +193,7 @@ struct md_ctx {
   RepGeo* rep_host;          // host copy
   int64_t* rep_off_host;     // host, nrep + 1 atom offsets
   int64_t ncell;
+  int64_t occ_max;           // atoms per cell of the fullest box, on average
   cudaStream_t stream;
   int own_stream;  // the context created the stream (caller passed NULL)
 

@@ -9,19 +9,22 @@
 //                 histogram with atomics (rank of each atom in its cell)
 //   scan          exclusive prefix sum of the histogram -> cell starts
 //   k_scatter     perm[start[c] + rank] = atom
-//   k_cell_sort   sort each cell's slice of perm ascending: a stable,
-//                 deterministic counting sort
-//   k_gather      permuted copies of x, v, f, id, cell; copied back so that
-//                 every pointer stays fixed (CUDA graphs capture them)
-//   k_split_snapshot  double-float split of x (xs, md_split) and the build
-//                 snapshot (xb)
-//   k_build       27-cell stencil (one cell along an axis with < 3 cells);
-//                 FP32 test with certified bounds, FP64 only inside the
-//                 band where FP32 cannot decide; writes tiled lists
+//   k_sort_gather permuted copies of x, v, f, id, cell; an atom's place in its
+//                 cell is the number of the cell's atoms with a smaller
+//                 index: a stable, deterministic counting sort
+//   k_restore     the copies back, so that every pointer stays fixed (CUDA
+//                 graphs capture them), with the position records (xs,
+//                 md_split; xq) and the build snapshot (xb)
+//   k_build_cell  27-cell stencil (one cell along an axis with < 3 cells), one
+//                 block per cell; sparse boxes: k_build, one thread per atom.
+//                 FP32 test with certified bounds, FP64 only inside the band
+//                 where FP32 cannot decide; writes tiled lists
 // The host then reads the largest count; if it exceeds the capacity the
 // list storage grows and k_build runs again.
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <type_traits>
 
 #include "md_device.cuh"
 #include "md_internal.cuh"
@@ -33,8 +36,12 @@ constexpr int SCAN_ITEMS = 8;
 constexpr int SCAN_TILE = SCAN_THREADS * SCAN_ITEMS;
 
 // x - L*floor(x/L) with correctly rounded division and product (no
-// contraction); a result equal to L becomes 0.
+// contraction); a result equal to L becomes 0.  For 0 <= x < L the rounded
+// quotient is below 1 (x <= L - ulp(L) / 2, and 1 - 2^-53 is a double) and x
+// stays: an integer test instead of the division.
 __device__ __forceinline__ double wrap1(double x, double L) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  if (b < (unsigned long long)__double_as_longlong(L)) return x;
   double q = floor(__ddiv_rn(x, L));
   double w = __dsub_rn(x, __dmul_rn(L, q));
   return (w == L) ? 0.0 : w;
@@ -117,7 +124,10 @@ __global__ void k_scan_tiles(const int32_t* __restrict__ in, TOUT* __restrict__ 
                              int64_t n, int64_t* __restrict__ tile_sums) {
   int64_t t;
   block_scan_tile<int32_t, TOUT>(in, out, n, (int64_t)blockIdx.x * SCAN_TILE, (TOUT)0, &t);
-  if (threadIdx.x == 0) tile_sums[blockIdx.x] = t;
+  if (threadIdx.x == 0) {
+    tile_sums[blockIdx.x] = t;
+    if (gridDim.x == 1) out[n] = (TOUT)t;  // one tile: the scan is complete
+  }
 }
 
 // One block: exclusive scan of the tile sums in place, any count.
@@ -154,49 +164,57 @@ __global__ void k_scatter(const int32_t* __restrict__ cell, const int32_t* __res
   perm[start[cell[i]] + rank[i]] = (int32_t)i;
 }
 
-// Insertion sort of each cell's slice (cells hold tens of atoms).
-__global__ void k_cell_sort(int32_t* __restrict__ perm, const int32_t* __restrict__ start,
-                            int64_t ncell) {
-  int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= ncell) return;
-  int b = start[c], e = start[c + 1];
-  for (int k = b + 1; k < e; k++) {
-    int32_t key = perm[k];
-    int q = k - 1;
-    while (q >= b && perm[q] > key) {
-      perm[q + 1] = perm[q];
-      q--;
-    }
-    perm[q + 1] = key;
-  }
+__global__ void k_sort_gather(const int32_t* __restrict__ perm,
+                              const int32_t* __restrict__ start, int64_t n,
+                              const double4_32a* __restrict__ x4, const double* __restrict__ v,
+                              const double* __restrict__ f, const int32_t* __restrict__ id,
+                              const int32_t* __restrict__ cell, double4_32a* __restrict__ x4n,
+                              double* __restrict__ vn, double* __restrict__ fn,
+                              int32_t* __restrict__ idn, int32_t* __restrict__ celln) {
+  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= n) return;
+  const int o = perm[s];
+  const double4_32a x = x4[o];
+  const double vx = v[o], vy = v[n + o], vz = v[2 * n + o];
+  const double fx = f[o], fy = f[n + o], fz = f[2 * n + o];
+  const int ido = id[o], c = cell[o];
+  const int b = start[c], e = start[c + 1];
+  int64_t p = b;
+  for (int q = b; q < e; q++) p += perm[q] < o;
+  x4n[p] = x;
+  vn[p] = vx;
+  vn[n + p] = vy;
+  vn[2 * n + p] = vz;
+  fn[p] = fx;
+  fn[n + p] = fy;
+  fn[2 * n + p] = fz;
+  idn[p] = ido;
+  celln[p] = c;
 }
 
-__global__ void k_gather(const int32_t* __restrict__ perm, int64_t n,
-                         const double4_32a* __restrict__ x4, const double* __restrict__ v,
-                         const double* __restrict__ f, const int32_t* __restrict__ id,
-                         const int32_t* __restrict__ cell, double4_32a* __restrict__ x4n,
-                         double* __restrict__ vn, double* __restrict__ fn,
-                         int32_t* __restrict__ idn, int32_t* __restrict__ celln) {
-  int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n) return;
-  int64_t o = perm[p];
-  x4n[p] = x4[o];
-  vn[p] = v[o];
-  vn[n + p] = v[n + o];
-  vn[2 * n + p] = v[2 * n + o];
-  fn[p] = f[o];
-  fn[n + p] = f[n + o];
-  fn[2 * n + p] = f[2 * n + o];
-  idn[p] = id[o];
-  celln[p] = cell[o];
-}
-
-__global__ void k_split_snapshot(const double4_32a* __restrict__ x4, XSplit* __restrict__ xs,
-                                 XSplit* __restrict__ xb, XFix* __restrict__ xq, int64_t n,
-                                 const XGrid gr) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void k_restore(const double4_32a* __restrict__ x4n, const double* __restrict__ vn,
+                          const double* __restrict__ fn, const int32_t* __restrict__ idn,
+                          const int32_t* __restrict__ celln, int64_t n,
+                          double4_32a* __restrict__ x4, double* __restrict__ v,
+                          double* __restrict__ f, int32_t* __restrict__ id,
+                          int32_t* __restrict__ cell, XSplit* __restrict__ xs,
+                          XSplit* __restrict__ xb, XFix* __restrict__ xq, const XGrid gr) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  md_store_pos(x4[i], gr, xs, xq, i, xb);
+  const double4_32a p = x4n[i];
+  const double vx = vn[i], vy = vn[n + i], vz = vn[2 * n + i];
+  const double fx = fn[i], fy = fn[n + i], fz = fn[2 * n + i];
+  const int32_t k = idn[i], c = celln[i];
+  x4[i] = p;
+  v[i] = vx;
+  v[n + i] = vy;
+  v[2 * n + i] = vz;
+  f[i] = fx;
+  f[n + i] = fy;
+  f[2 * n + i] = fz;
+  id[i] = k;
+  cell[i] = c;
+  md_store_pos(p, gr, xs, xq, i, xb);
 }
 
 // FP32 minimum image of one component (float positions in [0, L]).
@@ -365,6 +383,259 @@ __global__ void __launch_bounds__(MD_BLOCK)
   atomicMax(maxcount + 1, (unsigned int)cand);
 }
 
+// Neighbor build, one block per cell: the cell's stencil atoms (FP32 hi
+// parts, image shift added) are staged in shared memory, a warp tests 32 of
+// them (one per lane) against each atom of the cell in turn and keeps the
+// ballots, and then lane a writes atom a's row from its ballots, so that the
+// rows of consecutive atoms are written together.  Membership and row parts
+// are those of k_build: FP32 decides outside [lo2f, hi2f], the exact FP64 test
+// inside.  Row order: stencil cells in order, ascending index in a cell.
+// Half list: the atoms that an even i owns (md_owns) are the even j of later
+// cells and the odd j of earlier ones, and the reverse for an odd i; so the
+// candidates are staged as two lists, each tested against the cell's atoms of
+// one parity only (the own cell's atoms are in both and tested one by one).
+constexpr int BC_WARPS = MD_BLOCK / 32;
+constexpr int BC_CAP = 768;           // staged candidates (half list: two lists of half as many)
+constexpr int BC_CHUNKS = BC_CAP / 32;
+constexpr int BC_OWN = 0;             // the own cell comes first among the 27
+
+template <bool HALF, bool SINGLE>
+__global__ void __launch_bounds__(MD_BLOCK)
+    k_build_cell(const double4_32a* __restrict__ x4, const XSplit* __restrict__ xs,
+                 const int32_t* __restrict__ start, int64_t n, const Geo gg,
+                 const RepGeo* __restrict__ rep, int32_t* __restrict__ numneigh,
+                 int32_t* __restrict__ nbr, int maxneigh, unsigned int* __restrict__ maxcount) {
+  constexpr int NL = HALF ? 2 : 1;                // candidate lists
+  constexpr int LCAP = BC_CAP / NL;               // slots of a list
+  constexpr int LCH = BC_CHUNKS / NL;             // its chunks of 32
+  __shared__ float4 cx[BC_CAP];                   // x, y, z, tag
+  __shared__ int cj[BC_CAP];
+  __shared__ float4 own[32];
+  __shared__ uint2 mask[LCH][32];  // ballots: kept, kept and inside rc
+  __shared__ int s_b[27], s_e[27], s_off[NL][28];
+  __shared__ float s_sh[27][3];
+  __shared__ float scut[MD_MAX_TYPES * MD_MAX_TYPES];
+  __shared__ int part_in[BC_WARPS][32], part_sk[BC_WARPS][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int ob = start[blockIdx.x], oe = start[blockIdx.x + 1];
+  if (ob + (int)blockIdx.y * 32 >= oe) return;
+  const RepGeo& g = rep[MD_TAG_REP(__float_as_int(xs[ob].hi.w))];
+  const bool img = g.nc[0] < 3 || g.nc[1] < 3 || g.nc[2] < 3;  // minimum image per pair
+  if (threadIdx.x < gg.nt * gg.nt) scut[threadIdx.x] = gg.cutsqf[threadIdx.x];
+  const float cut1 = gg.cutsqf[0];
+  // the stencil's cells: their atoms, image shifts and places in the lists
+  int cand = 0;
+  if (w == 0) {
+    int b = 0, e = 0;
+    if (lane < 27) {
+      int c0[3];
+      md_cell_coords(g, (int)blockIdx.x, c0[0], c0[1], c0[2]);
+      const int q27 = lane == BC_OWN ? 13 : (lane <= 13 ? lane - 1 : lane);
+      const int o[3] = {q27 / 9 - 1, q27 / 3 % 3 - 1, q27 % 3 - 1};
+      bool in = true;
+      for (int a = 0; a < 3; a++) {
+        in = in && o[a] >= g.lo[a] && o[a] <= g.hi[a];
+        int q = c0[a] + o[a];
+        float s = 0.f;
+        if (q < 0) {
+          q += g.nc[a];
+          s = -g.Lf[a];
+        } else if (q >= g.nc[a]) {
+          q -= g.nc[a];
+          s = g.Lf[a];
+        }
+        c0[a] = q;
+        s_sh[lane][a] = img ? 0.f : s;
+      }
+      if (in) {
+        const int q = md_cell_index(g, c0[0], c0[1], c0[2]);
+        b = start[q];
+        e = start[q + 1];
+      }
+      s_b[lane] = b;
+      s_e[lane] = e;
+    }
+    cand = e - b;
+#pragma unroll
+    for (int l = 0; l < NL; l++) {
+      // list l holds what atoms of parity l need
+      int k = e - b;
+      if (HALF && lane != BC_OWN) {
+        const int par = b >= oe ? l : 1 - l;  // later cell: own parity
+        k = ((e + 1 - par) >> 1) - ((b + 1 - par) >> 1);
+      }
+      int s = k;
+      for (int d = 1; d < 32; d <<= 1) {
+        const int up = __shfl_up_sync(0xffffffffu, s, d);
+        if (lane >= d) s += up;
+      }
+      if (lane < 27) s_off[l][lane] = s - k;
+      if (lane == 26) s_off[l][27] = s;
+    }
+    cand = __reduce_add_sync(0xffffffffu, cand);
+  }
+  __syncthreads();
+  int most = 0;
+  int len = s_off[0][27];
+  if (HALF) len = max(len, s_off[NL - 1][27]);
+  for (int i0 = ob + (int)blockIdx.y * 32; i0 < oe; i0 += 32 * (int)gridDim.y) {
+    const int na = min(32, oe - i0);
+    int nin = 0, nsk = 0;  // lane a: entries of atom i0 + a found so far (all warps alike)
+    const int i = i0 + lane;
+    int32_t* out = nbr + (int64_t)(i >> 5) * maxneigh * 32 + (i & 31);
+    __syncthreads();
+    if (threadIdx.x < na) own[threadIdx.x] = xs[i0 + threadIdx.x].hi;
+    for (int p0 = 0; p0 < len; p0 += LCAP) {
+      // stage the candidates of slots p0 .. p0 + LCAP - 1 of each list
+      for (int c = w; c < 27; c += BC_WARPS) {
+        const int b = s_b[c], e = s_e[c];
+        const float s0 = s_sh[c][0], s1 = s_sh[c][1], s2 = s_sh[c][2];
+        for (int j = b + lane; j < e; j += 32) {
+          float4 h = __ldg(&xs[j].hi);
+          h.x += s0;
+          h.y += s1;
+          h.z += s2;
+          auto put = [&](int l, int slot) {
+            slot -= p0;
+            if (slot >= 0 && slot < LCAP) {
+              cx[l * LCAP + slot] = h;
+              cj[l * LCAP + slot] = j;
+            }
+          };
+          if (!HALF) {
+            put(0, s_off[0][c] + (j - b));
+          } else if (c == BC_OWN) {
+            put(0, s_off[0][c] + (j - b));
+            put(NL - 1, s_off[NL - 1][c] + (j - b));
+          } else {
+            const int l = b >= oe ? (j & 1) : 1 - (j & 1);
+            put(l, s_off[l][c] + ((j - b) >> 1));
+          }
+        }
+      }
+      __syncthreads();
+      // chunks of 32 candidates, one per lane, against the atoms
+      for (int ch = w; ch < BC_CHUNKS; ch += BC_WARPS) {
+        const int l = HALF ? ch / LCH : 0, c = ch - l * LCH;
+        const int left = s_off[l][27] - p0 - 32 * c;  // candidates from this chunk on
+        if (left <= 0) continue;
+        float4 h = cx[l * LCAP + 32 * c + lane];
+        const int j = cj[l * LCAP + 32 * c + lane];
+        if (lane >= left) h.x = 3.0e38f;  // no candidate
+        const int tj = MD_TAG_TYPE(__float_as_int(h.w));
+        const int a0 = HALF ? ((i0 ^ l) & 1) : 0, da = HALF ? 2 : 1;
+        // IMG: minimum image per pair; OWN: the chunk holds own-cell atoms (each
+        // pair's ownership is tested); EXACT: FP64 where FP32 cannot decide.
+        // Returns whether some lane met such a pair.
+        auto chunk = [&](auto img_, auto own_, auto exact_) {
+          constexpr bool IMG = decltype(img_)::value, OWN = decltype(own_)::value,
+                         EXACT = decltype(exact_)::value;
+          bool und = false;
+#pragma unroll 2
+          for (int a = a0; a < na; a += da) {
+            const float4 o = own[a];
+            float dx = h.x - o.x, dy = h.y - o.y, dz = h.z - o.z;
+            if (IMG) {
+              dx = min_image_f(dx, g.Lf[0], g.halfLf[0]);
+              dy = min_image_f(dy, g.Lf[1], g.halfLf[1]);
+              dz = min_image_f(dz, g.Lf[2], g.halfLf[2]);
+            }
+            const float r2f = __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, dx * dx));
+            bool keep = r2f < gg.lo2f;
+            if (EXACT) {
+              if (!keep && r2f <= gg.hi2f) {
+                const double4_32a xi = x4[i0 + a], xj = x4[j];
+                const double ex = md_min_image(__dsub_rn(xj.x, xi.x), g.L[0], g.halfL_bits[0]);
+                const double ey = md_min_image(__dsub_rn(xj.y, xi.y), g.L[1], g.halfL_bits[1]);
+                const double ez = md_min_image(__dsub_rn(xj.z, xi.z), g.L[2], g.halfL_bits[2]);
+                keep = md_lt_pos(md_r2(ex, ey, ez), gg.rlist2_bits);
+              }
+            } else {
+              und |= !keep & (r2f <= gg.hi2f);
+            }
+            if (OWN) {
+              const int ii = i0 + a;
+              keep = keep && j != ii;
+              if (HALF && j >= ob && j < oe) keep = keep && md_owns(ii, j);
+            }
+            const float cut =
+                SINGLE ? cut1 : scut[MD_TAG_TYPE(__float_as_int(o.w)) * gg.nt + tj];
+            const unsigned int bk = __ballot_sync(0xffffffffu, keep);
+            const unsigned int bi = __ballot_sync(0xffffffffu, keep & (r2f < cut));
+            if (lane == 0) mask[c][a] = make_uint2(bk, bi);
+          }
+          return und;
+        };
+        const std::true_type yes{};
+        const std::false_type no{};
+        if (img) {
+          chunk(yes, yes, yes);
+        } else {
+          const bool mixed = 32 * c + p0 < s_off[l][BC_OWN + 1];  // own-cell slots come first
+          const bool und = mixed ? chunk(no, yes, no) : chunk(no, no, no);
+          if (__any_sync(0xffffffffu, und)) chunk(no, yes, yes);
+        }
+      }
+      __syncthreads();
+      // each warp writes the entries of a quarter of the chunks
+      const int l = HALF ? (i & 1) : 0;
+      const int nch = min(LCH, (s_off[l][27] - p0 + 31) >> 5);
+      const int c0 = w * nch / BC_WARPS, c1 = (w + 1) * nch / BC_WARPS;
+      int pi = 0, ps = 0;
+      if (lane < na) {
+        for (int c = c0; c < c1; c++) {
+          const uint2 m = mask[c][lane];
+          pi += __popc(m.y);
+          ps += __popc(m.x & ~m.y);
+        }
+      }
+      part_in[w][lane] = pi;
+      part_sk[w][lane] = ps;
+      __syncthreads();
+      int ki = nin, ks = nsk;
+#pragma unroll
+      for (int q = 0; q < BC_WARPS; q++) {
+        const int qi = part_in[q][lane], qs = part_sk[q][lane];
+        if (q < w) {
+          ki += qi;
+          ks += qs;
+        }
+        nin += qi;
+        nsk += qs;
+      }
+      if (lane < na && nin + nsk <= maxneigh) {
+        int32_t* fi = out + (int64_t)ki * 32;
+        int32_t* fs = out + (int64_t)(maxneigh - 1 - ks) * 32;
+        for (int c = c0; c < c1; c++) {
+          const uint2 m = mask[c][lane];
+          const int* jt = cj + l * LCAP + 32 * c;
+          for (unsigned int k = m.y; k; k &= k - 1, fi += 32) *fi = jt[__ffs(k) - 1];
+          for (unsigned int k = m.x & ~m.y; k; k &= k - 1, fs -= 32) *fs = jt[__ffs(k) - 1];
+        }
+      }
+      __syncthreads();
+    }
+    // on overflow the rows are incomplete (but in bounds); the host sees
+    // total > maxneigh, grows the list and rebuilds
+    if (w == 0 && lane < na) {
+      const int a = min(nin, maxneigh);
+      numneigh[i] = a;
+      numneigh[n + i] = min(nsk, maxneigh - a);
+      most = max(most, nin + nsk);
+    }
+  }
+  if (w == 0) {
+    most = __reduce_max_sync(0xffffffffu, most);
+    if (lane == 0) {
+      atomicMax(maxcount, (unsigned int)most);
+      // every pair of an atom in any list built now joins it to a stencil
+      // candidate, so their number bounds the force contributions an atom
+      // receives in one pair launch (the range of the fixed-point accumulators)
+      atomicMax(maxcount + 1, (unsigned int)cand);
+    }
+  }
+}
+
 __global__ void k_sum_counts(const int32_t* __restrict__ numneigh, int64_t n,
                              unsigned long long* __restrict__ total) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -417,6 +688,10 @@ static int scan_impl(md_ctx* c, const int32_t* in, TOUT* out, int64_t n) {
     k_scan_tiles<TOUT><<<(unsigned)tiles, SCAN_THREADS, 0, c->stream>>>(in, out, n, c->scan_tmp);
     c->launches++;
   }
+  if (tiles == 1) {
+    MD_CUDA(cudaGetLastError());
+    return MD_OK;
+  }
   k_scan_top<<<1, SCAN_THREADS, 0, c->stream>>>(c->scan_tmp, tiles);
   k_scan_add<TOUT><<<(unsigned)md_blocks(n > 0 ? n : 1), MD_BLOCK, 0, c->stream>>>(out, n,
                                                                                    c->scan_tmp);
@@ -454,16 +729,30 @@ void md_drop_graphs(md_ctx* c) {
 }
 
 static int launch_build(md_ctx* c) {
-  MD_CUDA(cudaMemsetAsync(c->dmax + 1, 0, 2 * sizeof(unsigned int), c->stream));
   unsigned nb = (unsigned)md_blocks(c->n);
-  if (c->list_kind == MD_LIST_HALF)
+  const bool half = c->list_kind == MD_LIST_HALF;
+  // sparse boxes (mostly empty cells) keep one thread per atom: a block per cell
+  // would launch mostly empty blocks
+  if (c->ncell <= c->n) {
+    // one block per cell and 32 of its atoms; further groups are looped over
+    // unless the grid is small (boxes with few, full cells)
+    const int64_t occ = c->occ_max < 1 ? 1 : c->occ_max;
+    int64_t gy = (occ + 31) / 32;
+    if (c->ncell * gy > 8192) gy = 1;
+    const dim3 grid((unsigned)c->ncell, (unsigned)(gy < 64 ? gy : 64));
+    auto kern = half ? (c->nt == 1 ? k_build_cell<true, true> : k_build_cell<true, false>)
+                     : (c->nt == 1 ? k_build_cell<false, true> : k_build_cell<false, false>);
+    kern<<<grid, MD_BLOCK, 0, c->stream>>>(c->x4, c->xs, c->start, c->n, c->geo, c->rep,
+                                           c->numneigh, c->nbr, c->maxneigh, c->dmax + 1);
+  } else if (half) {
     k_build<true><<<nb, MD_BLOCK, 0, c->stream>>>(c->x4, c->xs, c->cell, c->start, c->n,
                                                   c->geo, c->rep, c->numneigh, c->nbr,
                                                   c->maxneigh, c->dmax + 1);
-  else
+  } else {
     k_build<false><<<nb, MD_BLOCK, 0, c->stream>>>(c->x4, c->xs, c->cell, c->start, c->n,
                                                    c->geo, c->rep, c->numneigh, c->nbr,
                                                    c->maxneigh, c->dmax + 1);
+  }
   c->launches++;
   MD_CUDA(cudaGetLastError());
   return MD_OK;
@@ -473,35 +762,32 @@ int md_rebuild(md_ctx* c) {
   const int64_t n = c->n;
   const unsigned nb = (unsigned)md_blocks(n);
   cudaStream_t s = c->stream;
-  // displacement since the previous build: dangerous if > skin/2
-  MD_CUDA(cudaMemcpyAsync(c->h_pinned + 8, c->dmax, sizeof(unsigned int), cudaMemcpyDeviceToHost, s));
-  MD_CUDA(cudaMemcpyAsync(c->h_pinned + 14, c->dmax + 5, sizeof(unsigned int),
+  // dmax[0]: displacement since the previous build, dangerous if > skin/2;
+  // dmax[5]: a fused step's barrier gave up
+  MD_CUDA(cudaMemcpyAsync(c->h_pinned + 12, c->dmax, 6 * sizeof(unsigned int),
                           cudaMemcpyDeviceToHost, s));
   MD_CUDA(cudaMemsetAsync(c->cnt, 0, sizeof(int32_t) * c->ncell, s));
   k_wrap_bin<<<nb, MD_BLOCK, 0, s>>>(c->x4, n, c->rep, c->cell, c->cnt, c->rank);
   c->launches++;
   MD_TRY(md_scan_i32(c, c->cnt, c->start, c->ncell));
   k_scatter<<<nb, MD_BLOCK, 0, s>>>(c->cell, c->rank, c->start, c->perm, n);
-  k_cell_sort<<<(unsigned)md_blocks(c->ncell), MD_BLOCK, 0, s>>>(c->perm, c->start, c->ncell);
-  k_gather<<<nb, MD_BLOCK, 0, s>>>(c->perm, n, c->x4, c->v, c->f, c->id, c->cell, c->x4_alt,
-                                   c->v_alt, c->f_alt, c->id_alt, c->cell_alt);
+  k_sort_gather<<<nb, MD_BLOCK, 0, s>>>(c->perm, c->start, n, c->x4, c->v, c->f, c->id, c->cell,
+                                        c->x4_alt, c->v_alt, c->f_alt, c->id_alt, c->cell_alt);
+  k_restore<<<nb, MD_BLOCK, 0, s>>>(c->x4_alt, c->v_alt, c->f_alt, c->id_alt, c->cell_alt, n,
+                                    c->x4, c->v, c->f, c->id, c->cell, c->xs, c->xb, c->xq,
+                                    c->xgrid);
   c->launches += 3;
   MD_CUDA(cudaGetLastError());
-  MD_CUDA(cudaMemcpyAsync(c->x4, c->x4_alt, sizeof(double4_32a) * n, cudaMemcpyDeviceToDevice, s));
-  MD_CUDA(cudaMemcpyAsync(c->v, c->v_alt, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, s));
-  MD_CUDA(cudaMemcpyAsync(c->f, c->f_alt, sizeof(double) * 3 * n, cudaMemcpyDeviceToDevice, s));
-  MD_CUDA(cudaMemcpyAsync(c->id, c->id_alt, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
-  MD_CUDA(cudaMemcpyAsync(c->cell, c->cell_alt, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
-  k_split_snapshot<<<nb, MD_BLOCK, 0, s>>>(c->x4, c->xs, c->xb, c->xq, n, c->xgrid);
-  c->launches++;
-  MD_CUDA(cudaGetLastError());
-  MD_CUDA(cudaMemsetAsync(c->dmax, 0, sizeof(unsigned int), s));
   for (int attempt = 0; attempt < 4; attempt++) {
+    // displacement, largest count, largest number of stencil candidates
+    MD_CUDA(cudaMemsetAsync(c->dmax, 0, 3 * sizeof(unsigned int), s));
     MD_TRY(launch_build(c));
     MD_CUDA(cudaMemcpyAsync(c->h_pinned + 9, c->dmax + 1, 2 * sizeof(unsigned int),
                             cudaMemcpyDeviceToHost, s));
     MD_CUDA(cudaStreamSynchronize(s));
-    MD_TRY(md_barrier_status(c));
+    unsigned int before[6];
+    memcpy(before, (const char*)(c->h_pinned + 12), sizeof(before));
+    if (before[5]) return MD_ETIMEOUT;
     unsigned int mc;
     memcpy(&mc, (const char*)(c->h_pinned + 9), sizeof(mc));
     c->max_count = (int32_t)mc;
@@ -512,10 +798,8 @@ int md_rebuild(md_ctx* c) {
       md_drop_graphs(c);
     c->kmax = kmax;
     if ((int)mc <= c->maxneigh) {
-      unsigned int disp_bits;
-      memcpy(&disp_bits, (const char*)(c->h_pinned + 8), sizeof(disp_bits));
       float disp2;
-      memcpy(&disp2, &disp_bits, sizeof(disp2));
+      memcpy(&disp2, &before[0], sizeof(disp2));
       double half = 0.5 * c->skin;
       // with check_disp the list is rebuilt before any force evaluation at
       // positions beyond skin/2, so no build is dangerous
