@@ -250,7 +250,9 @@ long long dd_fixed(Dd a, int s) {
 }  // namespace
 
 // Eq. 1's fixed-point coefficients of one type pair (md_fx.cuh).
-static void set_fx(PairFx& p, double eps, double sigma, double rc, int R, double lmax) {
+// qq, rc_coul: the Coulomb term (rc_coul <= 0: none).
+static void set_fx(PairFx& p, double eps, double sigma, double rc, int R, double lmax, double qq,
+                   double rc_coul) {
   memset(&p, 0, sizeof(p));
   // exact sigma^2 as m 2^e, m < 2^106
   int es = 0;
@@ -267,17 +269,25 @@ static void set_fx(PairFx& p, double eps, double sigma, double rc, int R, double
   const double ratio = ldexp(1.0, 2 * R) / (sigma * sigma);  // 4^R / sigma^2
   p.e2 = 2.0 * eps;
   p.smin = ~0u;  // nothing in fixed point
-  // cutoff band: r^2 here (4 units, positions within 2^-53), fma(dz,dz,
+  // cutoff band: r^2 here (3 units, positions within 2^-53), fma(dz,dz,
   // fma(dy,dy, dx*dx)) on FP64 separations of coordinates up to 1.25 lmax
-  const double su = ldexp(1.0, 62 - 2 * R), sc = rc * rc * su;
-  const double band = ldexp(sc, -44) + rc * lmax * ldexp(su, -47) + 64.0;
-  p.cut_lo = sc - band > 0.0 ? (unsigned int)floor(ldexp(sc - band, -32)) : 0u;
-  p.cut_hi = sc + band < ldexp(1.0, 63) ? (unsigned int)ceil(ldexp(sc + band, -32)) : ~0u;
-  if (!(ratio < ldexp(1.0, 40)) || !(ratio > ldexp(1.0, -2)) || !(band < 0.25 * sc)) return;
+  const double su = ldexp(1.0, 62 - 2 * R);
+  bool narrow = true;
+  auto bounds = [&](double r, unsigned int& lo, unsigned int& hi) {
+    const double sc = r * r * su, band = ldexp(sc, -44) + r * lmax * ldexp(su, -47) + 64.0;
+    lo = sc - band > 0.0 ? (unsigned int)floor(ldexp(sc - band, -32)) : 0u;
+    hi = sc + band < ldexp(1.0, 63) ? (unsigned int)ceil(ldexp(sc + band, -32)) : ~0u;
+    narrow = narrow && band < 0.25 * sc;
+  };
+  bounds(rc, p.cut_lo, p.cut_hi);
+  if (rc_coul > 0.0) bounds(rc_coul, p.cc_lo, p.cc_hi);
+  if (!(ratio < ldexp(1.0, 40)) || !(ratio > ldexp(1.0, -2)) || !narrow) return;
   // largest tau with |F| below the accumulators' range for every smaller one
   // (|F| = 24 eps / sigma tau^3.5 |2 tau^3 - 1|, largest of the attractive
   // branch 2.397 eps / sigma at tau^3 = 7 / 26)
-  const double fs = 24.0 * eps / sigma, flim = ldexp(1.0 - ldexp(1.0, -10), MD_FIX_EMAX + 1);
+  const double fs = 24.0 * eps / sigma, flim0 = ldexp(1.0 - ldexp(1.0, -10), MD_FIX_EMAX + 1);
+  const bool coul = rc_coul > 0.0 && qq != 0.0;  // each term then gets half the range
+  const double flim = coul ? 0.5 * flim0 : flim0;
   auto force = [&](double t) { return fs * pow(t, 3.5) * fabs(2.0 * t * t * t - 1.0); };
   const double ta = pow(7.0 / 26.0, 1.0 / 3.0);
   double lo = 0.0, hi = MD_FX_TAU_MAX;
@@ -292,7 +302,8 @@ static void set_fx(PairFx& p, double eps, double sigma, double rc, int R, double
     const double mid = 0.5 * (lo + hi);
     (force(mid) <= flim ? lo : hi) = mid;
   }
-  const double tl = lo * (1.0 - 1e-9);
+  double tl = lo * (1.0 - 1e-9);
+  if (coul && fabs(qq) * tl > flim * sigma * sigma) tl = flim * sigma * sigma / fabs(qq);
   if (!(tl > 1e-3)) return;
   // z = tau^4 (2 tau^3 - 1) over tau < tl: smallest -0.0806 at tau^3 = 2 / 7
   const double tm = pow(2.0 / 7.0, 1.0 / 3.0);
@@ -314,6 +325,23 @@ static void set_fx(PairFx& p, double eps, double sigma, double rc, int R, double
     const int d = p.sh - 12;
     p.cm = d < 62 ? p.cm >> d : 0;
     p.sh = 12;
+  }
+  if (coul) {
+    // |fpair| <= |F| / r: keep both terms below 2^61 in units of 2^-p
+    const int pm = (int)floor(61.0 - log2(flim * sqrt(tl) / sigma)), pp = p.sh + 45 + R;
+    if (pp > pm) {
+      p.cm >>= pp - pm < 62 ? pp - pm : 62;
+      p.sh -= pp - pm;
+    }
+    int qe = 0;
+    frexp(qq, &qe);
+    p.cq = dd_fixed({qq, 0.0}, 62 - qe);
+    p.csh = 62 - qe - 9 + 3 * R - (p.sh + 45 + R);
+    if (p.csh < -24) return;
+    if (p.csh > 62) {  // the term is far below P's unit
+      p.cq = 0;
+      p.csh = 62;
+    }
   }
   if (p.sh < 1) return;
   p.B = 0;
@@ -363,9 +391,10 @@ int md_upload_coef(md_ctx* c) {
   for (int a = 0; a < nt; a++)
     for (int b = 0; b < nt; b++) {
       const int k = a * nt + b;
-      set_fx(fx[k], c->eps[k], c->sigma[k], c->rc[k], c->fxR, c->lmax);
       const double qq = c->coul ? c->qqrd2e * c->qtype[a] * c->qtype[b] : 0.0;
       md_set_coef(tab[k], c->eps[k], c->sigma[k], c->rc[k], qq, c->coul ? c->rc_coul : 0.0);
+      set_fx(fx[k], c->eps[k], c->sigma[k], c->rc[k], c->fxR, c->lmax, qq,
+             c->coul ? c->rc_coul : 0.0);
     }
   c->coef1 = tab[0];
   c->fx1 = fx[0];
@@ -861,15 +890,19 @@ int launch_pair_impl(md_ctx* c, int ev, int tpa, int prezeroed, int defer_fold) 
     MD_CUDA(cudaMemsetAsync(c->f, 0, sizeof(double) * 3 * c->n, c->stream));
   if (compact) {
     const bool fix = c->compact == 2;
+    const unsigned qb = (unsigned)md_blocks(c->n);
+    const bool single = c->nt == 1;
+    const float cut1 = c->geo.cut_hi[0];
+    const float* cut = c->cut_hi_dev;
+    cudaStream_t s = c->stream;
+    const int t = fx_lanes(c);
     cudaError_t e =
-        c->coul ? md_pair_q_coul_launch(a, fix, half, ev != 0, c->nt == 1, c->geo.cut_hi[0],
-                                        c->cut_hi_dev, (unsigned)md_blocks(c->n), c->stream,
-                                        c->carve)
-                : fix ? md_pair_fx_launch(a, half, ev != 0, fx_single(c), fx_lanes(c), c->qu,
-                                          c->geo.cut_hi[0], c->cut_hi_dev, c->stream, c->carve)
-                      : md_pair_q_launch(a, half, ev != 0, c->nt == 1, c->geo.cut_hi[0],
-                                         c->cut_hi_dev, (unsigned)md_blocks(c->n), c->stream,
-                                         c->carve);
+        fix ? (c->coul ? md_pair_fx_coul_launch(a, half, ev != 0, t, 2, cut1, cut, s, c->carve)
+                       : md_pair_fx_launch(a, half, ev != 0, fx_single(c), t, c->qu, cut1, cut, s,
+                                           c->carve))
+            : (c->coul
+                   ? md_pair_q_coul_launch(a, half, ev != 0, single, cut1, cut, qb, s, c->carve)
+                   : md_pair_q_launch(a, half, ev != 0, single, cut1, cut, qb, s, c->carve));
     c->launches++;
     MD_CUDA(e);
     if (fix && !defer_fold) MD_TRY(md_launch_fix_finalize(c));

@@ -47,6 +47,11 @@ struct PairFx {
   unsigned long long csign;   // sigma^2 / 4^R 2^c, in [2^62, 2^63)
   long long cm;               // C = cm 2^-(p + 8 - zsh), in [2^61, 2^62)
   double e2;                  // 2 eps
+  // lj/cut/coul/cut (general form): rc_coul's bounds as cut_lo, cut_hi, and
+  // qq = cq 2^-x in 62 bits with csh = x - 9 + 3R - p
+  unsigned int cc_lo, cc_hi;
+  long long cq;
+  int csh;
 };
 
 #define MD_FX_BMAX 7
@@ -119,6 +124,27 @@ MD_HD unsigned long long md_fx_rcp(unsigned long long S, unsigned int Y0, int B)
   c += (h * h + (1 << 20)) >> 21;
   return ((unsigned long long)Y0 << 32) +
          (unsigned long long)(((long long)(int)Y0 * c) >> 21);
+}
+
+// rho 2^60 with rho = (2^62 / S)^(1/2) for 2^58 <= S < 2^62 (rho <= 4), from
+// Y0 = rho 2^28 within 2^-22 relative: e = 1 - S Y0^2 / 2^118 and the series
+// (1 - e)^(-1/2) ~ 1 + e / 2 + 3 e^2 / 8; within 2^-53 relative.
+MD_HD unsigned long long md_fx_rsqrt(unsigned long long S, unsigned int Y0) {
+  const unsigned long long Q = (unsigned long long)Y0 * Y0;  // <= 2^60
+  const long long e = (long long)((1ULL << 56) - md_mulhi_u(S, Q << 2));
+  int c = (int)((e + 8) >> 4);  // e 2^52
+  const int h = c >> 16;
+  c += (3 * h * h + (1 << 21)) >> 22;
+  return ((unsigned long long)Y0 << 32) +
+         (unsigned long long)(((long long)(int)Y0 * c) >> 21);
+}
+
+// P of the Coulomb term: qq rho t 8^(k - R) 2^p with rho t 2^55 in v.
+MD_HD long long md_fx_coul(unsigned long long rho, unsigned long long T, const PairFx& c, int k) {
+  const unsigned long long v = md_mulhi_u(rho, T << 1);
+  const long long f = md_mulhi_s(c.cq, (long long)v);
+  const int s = c.csh - 3 * k;
+  return s > 0 ? (f + (1LL << (s - 1))) >> s : f << -s;
 }
 
 // P of the one-type form, five products.  With x = T 2^-63 (tau = q x):

@@ -1,17 +1,25 @@
 // md_pair_coul.cu -- the second pair style, lj/cut/coul/cut (Eq. 1 plus a
 // cut Coulomb term with per-type charges; the paper's pair styles share one
-// two-body base, Sec. 4): the warp-compacted FP64 kernel with either force
-// summation, and the mixed-precision per-atom kernel at 1, 2 or 4 threads
-// per atom.
+// two-body base, Sec. 4): the fixed-point kernel, the warp-compacted FP64
+// kernel, and the mixed-precision per-atom kernel at 1, 2 or 4 threads per
+// atom.
 #include "md_pair.cuh"
+#include "md_pair_fx.cuh"
 #include "md_pair_q.cuh"
 
-cudaError_t md_pair_q_coul_launch(const PairArgs& a, bool fix, bool half, bool ev, bool single,
+cudaError_t md_pair_q_coul_launch(const PairArgs& a, bool half, bool ev, bool single,
                                   float cut1, const float* cut_tab, unsigned blocks,
                                   cudaStream_t s, int carve) {
-  return fix ? md_pair_q_launch_t<true, true>(a, half, ev, single, cut1, cut_tab, blocks, s, carve)
-             : md_pair_q_launch_t<false, true>(a, half, ev, single, cut1, cut_tab, blocks, s,
-                                               carve);
+  return md_pair_q_launch_t<true>(a, half, ev, single, cut1, cut_tab, blocks, s, carve);
+}
+
+cudaError_t md_pair_fx_coul_launch(const PairArgs& a, bool half, bool ev, int t, int u,
+                                   float cut1, const float* cut_tab, cudaStream_t s, int carve) {
+  if (half)
+    return ev ? md_pair_fx_launch_t<true, true, false, true>(a, t, u, cut1, cut_tab, s, carve)
+              : md_pair_fx_launch_t<true, false, false, true>(a, t, u, cut1, cut_tab, s, carve);
+  return ev ? md_pair_fx_launch_t<false, true, false, true>(a, t, u, cut1, cut_tab, s, carve)
+            : md_pair_fx_launch_t<false, false, false, true>(a, t, u, cut1, cut_tab, s, carve);
 }
 
 template <bool HALF, bool EV, bool SINGLE>

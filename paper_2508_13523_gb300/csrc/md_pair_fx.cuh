@@ -46,7 +46,7 @@
 // Sums of one pair taken in FP64.
 struct FxSlow {
   long long q[3];  // counts for atom j (owner: minus these)
-  double e;        // energy, or r^-6 with one type
+  double e;        // energy, or r^-6 with one type (Eq. 1 alone)
   double s[3];     // image shift taken off d
   double g[3];     // fpair d
   int in;
@@ -54,7 +54,7 @@ struct FxSlow {
 
 // The pair (i, j) in FP64, as the oracle evaluates it.  Contributions beyond
 // the accumulators' range are added to f here; the others are returned.
-template <bool HALF, bool EV, bool SINGLE>
+template <bool HALF, bool EV, bool SINGLE, bool COUL>
 __device__ __noinline__ void md_pair_fx_slow(const PairArgs& a, const PairCoef* coef, int64_t i,
                                              int j, FxSlow& o) {
   const int64_t n = a.n;
@@ -71,11 +71,21 @@ __device__ __noinline__ void md_pair_fx_slow(const PairArgs& a, const PairCoef* 
   const double dz = md_min_image(ez, g->L[2], g->halfL_bits[2]);
   const double r2 = md_r2(dx, dy, dz);
   o.q[0] = o.q[1] = o.q[2] = 0;
-  o.in = md_lt_pos(r2, c.cutsq_bits);
+  o.in = md_lt_pos(r2, COUL ? c.cutmax_bits : c.cutsq_bits);
   if (!o.in) return;
-  const double r2inv = md_rcp(r2);
-  const double r6inv = r2inv * r2inv * r2inv;
-  const double fpair = r6inv * (c.lj1 * r6inv - c.lj2) * r2inv;
+  double r2inv, r6inv, fpair, qr = 0.0;
+  if (COUL) {  // Eq. 1 below rc, plus qq / r below rc_coul
+    const double rinv = md_rsqrt(r2);
+    r2inv = rinv * rinv;
+    r6inv = r2inv * r2inv * r2inv;
+    const double flj = r6inv * (c.lj1 * r6inv - c.lj2) * r2inv;
+    qr = md_lt_pos(r2, c.cutsq_coul_bits) ? c.qq * rinv : 0.0;
+    fpair = __fma_rn(qr, r2inv, md_lt_pos(r2, c.cutsq_bits) ? flj : 0.0);
+  } else {
+    r2inv = md_rcp(r2);
+    r6inv = r2inv * r2inv * r2inv;
+    fpair = r6inv * (c.lj1 * r6inv - c.lj2) * r2inv;
+  }
   const double gx = fpair * dx, gy = fpair * dy, gz = fpair * dz;
   if (!(md_fix(gx, ex_lim, o.q[0]) & md_fix(gy, ex_lim, o.q[1]) & md_fix(gz, ex_lim, o.q[2]))) {
     o.q[0] = o.q[1] = o.q[2] = 0;
@@ -90,6 +100,7 @@ __device__ __noinline__ void md_pair_fx_slow(const PairArgs& a, const PairCoef* 
   }
   if (EV) {
     o.e = SINGLE ? r6inv : r6inv * (c.lj3 * r6inv - c.lj4);
+    if (COUL) o.e = (md_lt_pos(r2, c.cutsq_bits) ? o.e : 0.0) + qr;
     o.s[0] = md_abs_gt(ex, g->halfL_bits[0]) ? copysign(g->L[0], ex) : 0.0;
     o.s[1] = md_abs_gt(ey, g->halfL_bits[1]) ? copysign(g->L[1], ey) : 0.0;
     o.s[2] = md_abs_gt(ez, g->halfL_bits[2]) ? copysign(g->L[2], ez) : 0.0;
@@ -103,9 +114,11 @@ __device__ __noinline__ void md_pair_fx_slow(const PairArgs& a, const PairCoef* 
 // and the pair phase of k_step_fused).  All threads of the block must call
 // it.  T lanes per atom; U: skin entries per round of the FP32 test, their
 // gathers in flight together.
-template <bool HALF, bool EV, bool SINGLE, int T, int U>
+// COUL: lj/cut/coul/cut, in the general form.
+template <bool HALF, bool EV, bool SINGLE, bool COUL, int T, int U>
 __device__ __forceinline__ void md_pair_fx_tiles(const PairArgs& a, const float cut_hi1,
                                                  const float* __restrict__ cut_hi_tab) {
+  static_assert(!(SINGLE && COUL), "the Coulomb style takes the general form");
   __shared__ PairCoef sc[SINGLE ? 1 : MD_MAX_TYPES * MD_MAX_TYPES];
   __shared__ PairFx sf[SINGLE ? 1 : MD_MAX_TYPES * MD_MAX_TYPES];
   __shared__ float scut[SINGLE ? 1 : MD_MAX_TYPES * MD_MAX_TYPES];
@@ -159,7 +172,7 @@ __device__ __forceinline__ void md_pair_fx_tiles(const PairArgs& a, const float 
     int npair = 0;
     auto slow = [&](int j) {
       FxSlow o;
-      md_pair_fx_slow<HALF, EV, SINGLE>(a, SINGLE ? &a.c1 : sc, ia, j, o);
+      md_pair_fx_slow<HALF, EV, SINGLE, COUL>(a, SINGLE ? &a.c1 : sc, ia, j, o);
       if (o.in) {
         ax += o.q[0];
         ay += o.q[1];
@@ -221,23 +234,39 @@ __device__ __forceinline__ void md_pair_fx_tiles(const PairArgs& a, const float 
       const unsigned long long Sn = md_fx_r2(Ax, Ay, Az);
       const unsigned long long S = SINGLE ? Sn : (2 * k < 64 ? Sn >> (2 * k) : 0);
       const unsigned int S1 = (unsigned int)(S >> 32);
-      if (!(S1 > c.smin & S1 < c.cut_lo)) {
+      const bool in_lj = S1 < c.cut_lo, in_co = COUL && S1 < c.cc_lo;
+      if (COUL) {
+        if ((S1 <= c.smin) | (!in_lj & (S1 <= c.cut_hi)) | (!in_co & (S1 <= c.cc_hi))) {
+          slow(j);
+          return;
+        }
+        if (!(in_lj | in_co)) return;
+      } else if (!(S1 > c.smin & in_lj)) {
         if (S1 <= c.cut_hi) slow(j);
         return;
       }
       const float sfl = __fmaf_rn((float)(unsigned int)Sn, 0x1p-32f,
                                   (float)(unsigned int)(Sn >> 32));
-      float y;
-      asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(sfl));
       const int B = SINGLE ? c.B : 5;  // general: Sn >= 2^58
-      const unsigned int Y0 =
-          __float2uint_rn(y * __int_as_float((127 + 61 - B) << 23));
-      const unsigned long long Tr = md_fx_rcp(Sn, Y0, B);
+      float y;
+      unsigned long long Tr, rho = 0;
+      if (COUL) {
+        asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(sfl));
+        rho = md_fx_rsqrt(Sn, __float2uint_rn(y * 0x1p43f));
+        Tr = md_mulhi_u(rho, rho) << 2;
+      } else {
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(sfl));
+        Tr = md_fx_rcp(Sn, __float2uint_rn(y * __int_as_float((127 + 61 - B) << 23)), B);
+      }
       FxForce fo;  // tau3: one type: x^3 2^62 (md_fx_force1)
       if (SINGLE)
         fo.P = md_fx_force1(Tr, c, fo.tau3);
       else
         fo = md_fx_force(((md_mulhi_u(Tr, c.csign) >> (c.tsh - 2 * k)) << 6) + 32, c.cm, c.zsh);
+      if (COUL) {
+        fo.P = in_lj ? fo.P : 0;
+        fo.P += in_co ? md_fx_coul(rho, Tr, c, k) : 0;
+      }
       const int sh = SINGLE ? c.sh1 : c.sh + k;
       const long long qx = md_fx_count(fo.P, Ax, sh);
       ax += qx;
@@ -252,8 +281,12 @@ __device__ __forceinline__ void md_pair_fx_tiles(const PairArgs& a, const float 
         npair++;
         if (SINGLE)
           s6 += fo.tau3 >> a.ev_shift;
-        else  // 4 eps (tau^6 - tau^3) = 2 eps (w - tau^3)
+        else if (!COUL || in_lj)  // 4 eps (tau^6 - tau^3) = 2 eps (w - tau^3)
           e0 += c.e2 * 0x1p-57 * __ll2double_rn(fo.w - (long long)(fo.tau3 >> 2));
+        if (COUL && in_co)  // qq / r = qq rho 2^(k - R)
+          e0 += sc[MD_TAG_TYPE(tag) * a.nt + MD_TAG_TYPE((int)o.w)].qq *
+                __ull2double_rn(rho) *
+                __longlong_as_double((long long)(1023 - 60 + k - a.fxR) << 52);
         if (shf) {  // rare
           auto shift = [&](int k3) {
             const int b = (shf >> (2 * k3)) & 3;
@@ -373,14 +406,55 @@ __device__ __forceinline__ void md_pair_fx_tiles(const PairArgs& a, const float 
 #define MD_FX_MINB 9
 constexpr int md_pair_fx_minb(bool half, bool ev) { return ev && half ? 8 : MD_FX_MINB; }
 
-template <bool HALF, bool EV, bool SINGLE, int T, int U>
+template <bool HALF, bool EV, bool SINGLE, bool COUL, int T, int U>
 __global__ void __launch_bounds__(MD_BLOCK, md_pair_fx_minb(HALF, EV))
     k_pair_fx(const __grid_constant__ PairArgs a, const float cut_hi1,
               const float* __restrict__ cut_hi_tab) {
-  md_pair_fx_tiles<HALF, EV, SINGLE, T, U>(a, cut_hi1, cut_hi_tab);
+  md_pair_fx_tiles<HALF, EV, SINGLE, COUL, T, U>(a, cut_hi1, cut_hi_tab);
+}
+
+template <bool HALF, bool EV, bool SINGLE, bool COUL, int T, int U>
+cudaError_t md_pair_fx_launch1(const PairArgs& a, float cut1, const float* cut_tab,
+                               cudaStream_t s, int carve) {
+  int occ = 1;
+  cudaError_t e =
+      md_prepare_kernel((const void*)k_pair_fx<HALF, EV, SINGLE, COUL, T, U>, carve, &occ);
+  if (e != cudaSuccess) return e;
+  unsigned blocks = (unsigned)md_blocks(a.n * T);
+  if (a.tile_ctr) {
+    const unsigned cap = (unsigned)(a.nslots * occ);
+    if (blocks > cap) blocks = cap;
+  }
+  k_pair_fx<HALF, EV, SINGLE, COUL, T, U><<<blocks, MD_BLOCK, 0, s>>>(a, cut1, cut_tab);
+  return cudaGetLastError();
+}
+
+template <bool HALF, bool EV, bool SINGLE, bool COUL>
+cudaError_t md_pair_fx_launch_t(const PairArgs& a, int t, int u, float cut1,
+                                const float* cut_tab, cudaStream_t s, int carve) {
+  constexpr int U1 = EV ? 2 : 1;
+  if (u == 1) {
+    switch (t) {
+      case 1: return md_pair_fx_launch1<HALF, EV, SINGLE, COUL, 1, U1>(a, cut1, cut_tab, s, carve);
+      case 2: return md_pair_fx_launch1<HALF, EV, SINGLE, COUL, 2, U1>(a, cut1, cut_tab, s, carve);
+      case 4: return md_pair_fx_launch1<HALF, EV, SINGLE, COUL, 4, U1>(a, cut1, cut_tab, s, carve);
+      case 8: return md_pair_fx_launch1<HALF, EV, SINGLE, COUL, 8, U1>(a, cut1, cut_tab, s, carve);
+      default: return cudaErrorInvalidValue;
+    }
+  }
+  switch (t) {
+    case 1: return md_pair_fx_launch1<HALF, EV, SINGLE, COUL, 1, 2>(a, cut1, cut_tab, s, carve);
+    case 2: return md_pair_fx_launch1<HALF, EV, SINGLE, COUL, 2, 2>(a, cut1, cut_tab, s, carve);
+    case 4: return md_pair_fx_launch1<HALF, EV, SINGLE, COUL, 4, 2>(a, cut1, cut_tab, s, carve);
+    case 8: return md_pair_fx_launch1<HALF, EV, SINGLE, COUL, 8, 2>(a, cut1, cut_tab, s, carve);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 // t: lanes per atom (1, 2, 4 or 8); u: skin entries per round (1 or 2; 2 with
 // energy and virial)
 cudaError_t md_pair_fx_launch(const PairArgs& a, bool half, bool ev, bool single, int t, int u,
                               float cut1, const float* cut_tab, cudaStream_t s, int carve);
+// lj/cut/coul/cut (md_pair_coul.cu)
+cudaError_t md_pair_fx_coul_launch(const PairArgs& a, bool half, bool ev, int t, int u,
+                                   float cut1, const float* cut_tab, cudaStream_t s, int carve);

@@ -24,22 +24,8 @@
 // three unconditional FP64 subtractions, off the ~98 % of pairs (in a large
 // box) that never cross the boundary.
 // The FP64 decisions and arithmetic per pair are those of k_pair; only the
-// summation of the contributions into f_i differs:
-//   FIX = false: FP64 reductions into f (order-dependent rounding);
-//   FIX = true:  each contribution is rounded to a multiple of 2^-44 and
-//                summed exactly in 64-bit integers: the owner's share in a
-//                shared-memory accumulator of its warp (added to fix once
-//                per atom), f_j's by a global reduction into fix;
-//                contributions too large for the accumulators' range go to
-//                f by FP64 reductions; md_launch_fix_finalize then adds fix
-//                to f.  The sum is independent of the order, within
-//                (contributions) x 2^-45 of the exact sum, needs no FP64
-//                instruction (shared-memory FP64 atomics would run on the
-//                FP64 pipe, and the owner's -g costs an FP64 negation when
-//                it feeds an FP64 reduction) and sends one global reduction
-//                per pair to L2 instead of two.
-// The fixed-point form of Eq. 1 alone is md_pair_fx.cuh's kernel; here FIX =
-// true exists for the second pair style.
+// summation of the contributions into f_i differs: FP64 reductions into f
+// (order-dependent rounding).  The fixed-point sums are md_pair_fx.cuh's.
 // COUL adds the second pair style's cut Coulomb term qq / r (1/r from the
 // rsqrt seed and one series round; r^-2 = (1/r)^2 instead of md_rcp).
 #pragma once
@@ -57,25 +43,16 @@
 #define MD_Q_MINB 10
 
 // The tile loop of the compacted kernel; all threads of the block must call it.
-template <bool HALF, bool EV, bool SINGLE, bool FIX, bool COUL>
+template <bool HALF, bool EV, bool SINGLE, bool COUL>
 __device__ __forceinline__ void md_pair_q_tiles(const PairArgs& a, const float cut_hi1,
                                                 const float* __restrict__ cut_hi_tab) {
   constexpr int W = MD_BLOCK / 32;
-  // range of the fixed-point accumulators: a contribution goes there only if
-  // its biased exponent is below ex_lim, so that |q| <= 2^(ex_lim - 1023 + 44)
-  // and the at most kmax < 2^kb contributions to one atom sum below 2^63
-  int ex_lim = 0;
-  if (FIX) {
-    const int kb = 32 - __clz((int)min(*a.kmax, 0x7fffffffu));
-    ex_lim = min(1023 + MD_FIX_EMAX + 1, 1023 + 63 - MD_FIX_BITS - kb);
-  }
   __shared__ PairCoef sc[SINGLE ? 1 : MD_MAX_TYPES * MD_MAX_TYPES];
   __shared__ float scut[SINGLE ? 1 : MD_MAX_TYPES * MD_MAX_TYPES];
   __shared__ int qj[2][W][MD_Q_CAP];            // queue 0: no image, 1: may wrap
   __shared__ unsigned char qo[2][W][MD_Q_CAP];
   __shared__ double4_32a xown[W][32];      // owner positions (x, y, z, tag)
   __shared__ double sev[EV ? W : 1][8][32];  // owner energy/virial accumulators
-  __shared__ unsigned long long sown[FIX ? W : 1][3][32];  // owner fixed-point forces
   if (!SINGLE) {
     for (int k = threadIdx.x; k < a.nt * a.nt; k += blockDim.x) {
       sc[k] = a.coef[k];
@@ -117,10 +94,6 @@ __device__ __forceinline__ void md_pair_q_tiles(const PairArgs& a, const float c
     const float hm0 = hf0 * (1.f - 0x1p-12f), hm1 = hf1 * (1.f - 0x1p-12f),
                 hm2 = hf2 * (1.f - 0x1p-12f);
     xown[w][lane] = xi;
-    if (FIX) {
-  #pragma unroll
-      for (int k = 0; k < 3; k++) sown[w][k][lane] = 0ULL;
-    }
     if (EV) {
   #pragma unroll
       for (int k = 0; k < 8; k++) sev[w][k][lane] = 0.0;
@@ -205,26 +178,13 @@ __device__ __forceinline__ void md_pair_q_tiles(const PairArgs& a, const float c
           }
           const double gx = fpair * dx, gy = fpair * dy, gz = fpair * dz;
           const int64_t io = tile * MD_BLOCK + w * 32 + o;
-          long long qx = 0, qy = 0, qz = 0;
-          if (FIX && (md_fix(gx, ex_lim, qx) & md_fix(gy, ex_lim, qy) &
-                      md_fix(gz, ex_lim, qz))) {
-            atomicAdd(&sown[FIX ? w : 0][0][o], (unsigned long long)(-qx));
-            atomicAdd(&sown[FIX ? w : 0][1][o], (unsigned long long)(-qy));
-            atomicAdd(&sown[FIX ? w : 0][2][o], (unsigned long long)(-qz));
-            if (HALF) {
-              atomicAdd(a.fix + j, (unsigned long long)qx);
-              atomicAdd(a.fix + n + j, (unsigned long long)qy);
-              atomicAdd(a.fix + 2 * n + j, (unsigned long long)qz);
-            }
-          } else {
-            atomicAdd(a.f + io, md_neg(gx));
-            atomicAdd(a.f + n + io, md_neg(gy));
-            atomicAdd(a.f + 2 * n + io, md_neg(gz));
-            if (HALF) {
-              atomicAdd(a.f + j, gx);
-              atomicAdd(a.f + n + j, gy);
-              atomicAdd(a.f + 2 * n + j, gz);
-            }
+          atomicAdd(a.f + io, md_neg(gx));
+          atomicAdd(a.f + n + io, md_neg(gy));
+          atomicAdd(a.f + 2 * n + io, md_neg(gz));
+          if (HALF) {
+            atomicAdd(a.f + j, gx);
+            atomicAdd(a.f + n + j, gy);
+            atomicAdd(a.f + 2 * n + j, gz);
           }
           if (EV) {  // the virial is x (x) F per atom afterwards, less the image terms
             const bool img = (shx != 0.0) | (shy != 0.0) | (shz != 0.0);
@@ -307,14 +267,6 @@ __device__ __forceinline__ void md_pair_q_tiles(const PairArgs& a, const float c
     while (tail[0] != head[0]) drain(q0, tail[0] - head[0] < 32 ? tail[0] - head[0] : 32);
     while (tail[1] != head[1]) drain(q1, tail[1] - head[1] < 32 ? tail[1] - head[1] : 32);
     __syncwarp();
-    if (FIX && active) {  // the owner's share: one reduction per component
-  #pragma unroll
-      for (int k = 0; k < 3; k++) {
-        const unsigned long long q = sown[FIX ? w : 0][k][lane];
-        if (q) atomicAdd(a.fix + k * n + i, q);
-      }
-    }
-
     if (EV) {
       const int slot = (int)(((int64_t)tile * (MD_BLOCK / 32) + w) % a.ev_spread);
       double ev[8];
@@ -341,49 +293,48 @@ __device__ __forceinline__ void md_pair_q_tiles(const PairArgs& a, const float c
 // 3.60 ms per half-list launch and 5.80, 5.60 and 5.38 ms per full-list one.
 constexpr int md_pair_q_minb(bool half, bool ev) { return ev ? (half ? 8 : 10) : MD_Q_MINB; }
 
-template <bool HALF, bool EV, bool SINGLE, bool FIX, bool COUL>
+template <bool HALF, bool EV, bool SINGLE, bool COUL>
 __global__ void __launch_bounds__(MD_BLOCK, md_pair_q_minb(HALF, EV))
     k_pair_q(const PairArgs a, const float cut_hi1, const float* __restrict__ cut_hi_tab) {
-  md_pair_q_tiles<HALF, EV, SINGLE, FIX, COUL>(a, cut_hi1, cut_hi_tab);
+  md_pair_q_tiles<HALF, EV, SINGLE, COUL>(a, cut_hi1, cut_hi_tab);
 }
 
-template <bool HALF, bool EV, bool SINGLE, bool FIX, bool COUL>
+template <bool HALF, bool EV, bool SINGLE, bool COUL>
 cudaError_t md_pair_q_launch5(const PairArgs& a, float cut1, const float* cut_tab,
                               unsigned blocks, cudaStream_t s, int carve) {
   int occ = 1;
   cudaError_t e =
-      md_prepare_kernel((const void*)k_pair_q<HALF, EV, SINGLE, FIX, COUL>, carve, &occ);
+      md_prepare_kernel((const void*)k_pair_q<HALF, EV, SINGLE, COUL>, carve, &occ);
   if (e != cudaSuccess) return e;
   if (a.tile_ctr) {
     const unsigned cap = (unsigned)(a.nslots * occ);
     if (blocks > cap) blocks = cap;
   }
-  k_pair_q<HALF, EV, SINGLE, FIX, COUL><<<blocks, MD_BLOCK, 0, s>>>(a, cut1, cut_tab);
+  k_pair_q<HALF, EV, SINGLE, COUL><<<blocks, MD_BLOCK, 0, s>>>(a, cut1, cut_tab);
   return cudaGetLastError();
 }
 
-template <bool FIX, bool COUL>
+template <bool COUL>
 cudaError_t md_pair_q_launch_t(const PairArgs& a, bool half, bool ev, bool single, float cut1,
                                const float* cut_tab, unsigned blocks, cudaStream_t s,
                                int carve) {
   if (half) {
     if (ev)
-      return single ? md_pair_q_launch5<true, true, true, FIX, COUL>(a, cut1, cut_tab, blocks, s, carve)
-                    : md_pair_q_launch5<true, true, false, FIX, COUL>(a, cut1, cut_tab, blocks, s, carve);
-    return single ? md_pair_q_launch5<true, false, true, FIX, COUL>(a, cut1, cut_tab, blocks, s, carve)
-                  : md_pair_q_launch5<true, false, false, FIX, COUL>(a, cut1, cut_tab, blocks, s, carve);
+      return single ? md_pair_q_launch5<true, true, true, COUL>(a, cut1, cut_tab, blocks, s, carve)
+                    : md_pair_q_launch5<true, true, false, COUL>(a, cut1, cut_tab, blocks, s, carve);
+    return single ? md_pair_q_launch5<true, false, true, COUL>(a, cut1, cut_tab, blocks, s, carve)
+                  : md_pair_q_launch5<true, false, false, COUL>(a, cut1, cut_tab, blocks, s, carve);
   }
   if (ev)
-    return single ? md_pair_q_launch5<false, true, true, FIX, COUL>(a, cut1, cut_tab, blocks, s, carve)
-                  : md_pair_q_launch5<false, true, false, FIX, COUL>(a, cut1, cut_tab, blocks, s, carve);
-  return single ? md_pair_q_launch5<false, false, true, FIX, COUL>(a, cut1, cut_tab, blocks, s, carve)
-                : md_pair_q_launch5<false, false, false, FIX, COUL>(a, cut1, cut_tab, blocks, s, carve);
+    return single ? md_pair_q_launch5<false, true, true, COUL>(a, cut1, cut_tab, blocks, s, carve)
+                  : md_pair_q_launch5<false, true, false, COUL>(a, cut1, cut_tab, blocks, s, carve);
+  return single ? md_pair_q_launch5<false, false, true, COUL>(a, cut1, cut_tab, blocks, s, carve)
+                : md_pair_q_launch5<false, false, false, COUL>(a, cut1, cut_tab, blocks, s, carve);
 }
 
-// FP64 reductions (md_pair_fp64.cu), and the lj/cut/coul/cut style with
-// either summation (md_pair_coul.cu)
+// md_pair_fp64.cu, and the lj/cut/coul/cut style (md_pair_coul.cu)
 cudaError_t md_pair_q_launch(const PairArgs& a, bool half, bool ev, bool single, float cut1,
                              const float* cut_tab, unsigned blocks, cudaStream_t s, int carve);
-cudaError_t md_pair_q_coul_launch(const PairArgs& a, bool fix, bool half, bool ev, bool single,
+cudaError_t md_pair_q_coul_launch(const PairArgs& a, bool half, bool ev, bool single,
                                   float cut1, const float* cut_tab, unsigned blocks,
                                   cudaStream_t s, int carve);

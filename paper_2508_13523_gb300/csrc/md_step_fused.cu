@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(MD_BLOCK, MD_FX_MINB)
   __threadfence();
   if (!grid_barrier(bar, err, gridDim.x, BARRIER_LIMIT_NS)) return;
   // phase 2: the forces at the new positions
-  md_pair_fx_tiles<HALF, false, SINGLE, 1, 1>(a, cut_hi1, cut_hi_tab);
+  md_pair_fx_tiles<HALF, false, SINGLE, false, 1, 1>(a, cut_hi1, cut_hi_tab);
 }
 
 template <int MODE, bool HALF, bool SINGLE>

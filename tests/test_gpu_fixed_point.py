@@ -146,3 +146,50 @@ def test_skin_entries_in_range(kind):
         ctx.set_state(x1, v0, keep_list=True)
         assert ctx.stats()["builds"] == builds
         check(ctx, x1.cpu().numpy(), box, 1.0, 0.5, 2.5, t, 0.0)
+
+
+COUL = {
+    # name: (cells, eps, sigma, rc, q, qqrd2e, rc_coul)
+    "weak, one type": (6, 1.0, 1.0, 2.5, [1e-3], 1.0, 2.5),
+    "strong": (6, np.ones((2, 2)), np.ones((2, 2)), np.full((2, 2), 2.5), [3.0, -2.0], 10.0, 2.5),
+    "one neutral type": (6, np.ones((2, 2)), np.ones((2, 2)), np.full((2, 2), 2.5), [0.5, 0.0],
+                         1.0, 1.7),
+    "beyond rc of a pair": (6, MIX["eps"], MIX["sigma"], MIX["rc"], [0.5, -0.5], 1.0, 2.45),
+    "4 lanes": (17, np.ones((2, 2)), np.ones((2, 2)), np.full((2, 2), 2.5), [0.5, -0.5], 1.0, 2.5),
+}
+
+
+@pytest.mark.parametrize("kind", [md.MD_LIST_FULL, md.MD_LIST_HALF])
+@pytest.mark.parametrize("case", COUL)
+def test_coulomb(case, kind):
+    """lj/cut/coul/cut against the oracle; the bound as above with the
+    Coulomb contributions' magnitudes added (two roundings per contribution:
+    each term has its own)."""
+    cells, eps, sigma, rc, q, qqrd2e, rc_coul = COUL[case]
+    x, box = lattice(cells, 0.8442, 0.3, 80 + cells)
+    nt = len(q)
+    t = (np.arange(len(x)) % 4 >= 2).astype(np.int32) if nt > 1 else np.zeros(len(x), np.int32)
+    with md.LJMD(x, np.zeros_like(x), t, box, eps, sigma, rc, np.ones(nt), list_kind=kind,
+                 threads_per_atom=1) as ctx:
+        ctx.set_coulomb(q, rc_coul, qqrd2e)
+        ctx.set_kernel(1, -1, 2, 0)
+        ctx.compute_forces(0)
+        xw, _, f = (a.cpu().numpy() for a in ctx.get_state())
+        th = ctx.energy()
+    lj = O.LJ(eps, sigma, rc, ntypes=nt, q=q, rc_coul=rc_coul, qqrd2e=qqrd2e)
+    fref, E, W = O.forces(xw, box, lj, type_=t if nt > 1 else None, skin=0.3)
+    cnt, mag = pair_sums(xw, box, eps, sigma, rc, t)
+    i, j = O.pairs_cells(xw, box, rc_coul) if len(x) > 3000 else O.pairs_brute(xw, box, rc_coul)
+    d = xw[j] - xw[i]
+    d -= box * np.round(d / box)
+    r2 = (d * d).sum(1)
+    qt = np.asarray(q)
+    fc = qqrd2e * np.abs(qt[t[i]] * qt[t[j]]) / r2
+    cnt = cnt + np.bincount(i, minlength=len(x)) + np.bincount(j, minlength=len(x))
+    mag = mag + np.bincount(i, fc, len(x)) + np.bincount(j, fc, len(x))
+    bound = (2 * cnt * 2.0 ** -44 + mag * 2.0 ** -46)[:, None]
+    assert np.all(np.abs(f - fref) <= bound)
+    noise = 6 * np.sqrt(2 * cnt.sum()) * 2.0 ** -45 * 0.5 * float(np.max(box))
+    ec = (qqrd2e * np.abs(qt[t[i]] * qt[t[j]]) / np.sqrt(r2)).sum()
+    assert abs(th.pe - E) <= 1e-12 * max(abs(E), np.abs(W).max(), ec) + noise
+    assert np.abs(th.virial - W).max() <= 1e-12 * max(np.abs(W).max(), ec) + noise
