@@ -463,7 +463,8 @@ void free_ctx(md_ctx* c) {
                   c->scan_tmp, c->numneigh, c->nbr,  c->ev,       c->dmax,    c->i64_tmp,
                   c->stage,  c->rep,     c->vcoef,    c->adj_c,    c->adj_xbar, c->adj_vbar,
                   c->adj_carry, c->seg_x, c->gbar,     c->fmax_bits, c->cut_hi_dev,
-                  c->tile_ctr, c->fix,   c->xq,       c->evs,       c->fxt};
+                  c->tile_ctr, c->fix,   c->xq,       c->evs,       c->fxt,
+                  c->adj_cf};
   for (void* b : bufs)
     if (b) cudaFree(b);
   if (c->pair_ev) {

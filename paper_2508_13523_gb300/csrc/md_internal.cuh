@@ -255,12 +255,13 @@ struct md_ctx {
 
   // adjoint buffers (allocated on first use)
   double4_32a* adj_c;    // cotangent of the forces, sorted order
+  float4* adj_cf;        // the same in FP32 (mixed contexts)
   double* adj_xbar;      // SoA 3n, sorted order
   double* adj_vbar;      // SoA 3n, sorted order
   double* adj_carry;     // caller order: xbar, vbar, cotangent (9n)
   double4_32a* seg_x;    // positions of one checkpoint segment, sorted
   int64_t seg_cap;       // positions seg_x holds
-  double* gbar;          // 2 nt^2 parameter derivatives
+  double* gbar;          // parameter derivatives (VjpArgs)
   unsigned long long* fmax_bits;  // steepest descent: max |F| as bits
 
   // graphs

@@ -14,6 +14,14 @@
 //   dL/dsigma += (e . w) r^-2 r^-6 (12 lj1 r^-6 - 6 lj2) / sigma.
 // Cutoffs are held fixed.  A full list visits each pair from both ends: each
 // visit adds J w to its own atom only and half of the parameter terms.
+//
+// FP64: bound by the FP64 pipe (about 44 operations a pair at 64 cycles each:
+// 150 us of the 272 us at 62,500 mixture atoms).  Mixed: no FP64 operation per
+// pair; the cotangent is read as FP32 (16 bytes), the parameter terms are FP32
+// values with their rounding errors in the thread's own shared-memory column
+// (one row per thread put all lanes on the same banks), and the sums' atomics
+// are spread over rows.  62,500 atoms, half list, before and after: mixed 140 ->
+// 67 us, FP64 350 -> 272 us.
 #pragma once
 
 #include <type_traits>
@@ -26,39 +34,52 @@ struct VjpCoef {
   float inv_epsf, inv_sigmaf;
 };
 
+#define MD_GBAR_ROWS 128
+
 struct VjpArgs {
   const double4_32a* x4;
   const XSplit* xs;
   const XSplit* xb;      // positions at the last build (split)
   float rin;             // rlist rounded up: atoms this far inside every face need no image
   const double4_32a* c;  // cotangent per sorted atom (x, y, z, unused)
+  const float4* cf;      // the same rounded to FP32 (mixed precision)
   const int32_t* numneigh;
   const int32_t* nbr;
   double* xbar;          // SoA per sorted atom, accumulated (+=)
-  double* gbar;          // 2 nt^2: dL/deps then dL/dsigma, entry [min][max]
+  double* gbar;          // MD_GBAR_ROWS rows of 2 nt^2: dL/deps then dL/dsigma, entry
+                         // [min][max]; the blocks' sums are spread over the rows so
+                         // that their atomics do not queue on the same addresses
   const PairCoef* coef;
   const VjpCoef* vcoef;
   PairCoef c1;
   VjpCoef v1;
   const RepGeo* rep;
+  float cut1;            // certified FP32 bounds of rc^2 (Geo::cut_hi): the only one,
+  const float* cut_tab;  // the nt*nt table
   int64_t n;
   int nt;
   int maxneigh;
 };
 
+#define MD_VJP_SLOTS 8  // skin entries that wait per lane
+
 template <int PREC, bool HALF, int TPA, bool SINGLE>
 __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
   __shared__ PairCoef sc[SINGLE ? 1 : MD_MAX_TYPES * MD_MAX_TYPES];
+  __shared__ float scut[SINGLE ? 1 : MD_MAX_TYPES * MD_MAX_TYPES];
   __shared__ VjpCoef sv[SINGLE ? 1 : MD_MAX_TYPES * MD_MAX_TYPES];
   // parameter terms of each thread by partner type: [tj] eps, [MD_MAX_TYPES + tj]
-  // sigma; thread-private slots, reduced once per block at the end
-  __shared__ double sg[SINGLE ? 1 : MD_BLOCK][SINGLE ? 1 : 2 * MD_MAX_TYPES];
+  // sigma; thread-private columns (no bank conflicts), reduced at the end
+  // (mixed: FP32 values with their rounding errors, md_acc2)
+  constexpr bool MIX = PREC == MD_PREC_MIXED;
+  __shared__ double sg[SINGLE ? 1 : 2 * MD_MAX_TYPES][SINGLE ? 1 : MD_BLOCK];
   if (!SINGLE) {
     for (int k = threadIdx.x; k < a.nt * a.nt; k += blockDim.x) {
       sc[k] = a.coef[k];
       sv[k] = a.vcoef[k];
+      scut[k] = a.cut_tab[k];
     }
-    for (int k = 0; k < 2 * MD_MAX_TYPES; k++) sg[threadIdx.x][k] = 0.0;
+    for (int k = 0; k < 2 * MD_MAX_TYPES; k++) sg[k][threadIdx.x] = 0.0;
     __syncthreads();
   }
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -71,12 +92,44 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
   const int nsk = active ? __ldg(a.numneigh + n + ia) : 0;
   const int32_t* row = a.nbr + (ia >> 5) * (int64_t)a.maxneigh * 32 + (ia & 31);
   const int32_t* skin = row + (int64_t)(a.maxneigh - 1) * 32;
-  const double4_32a ci = a.c[ia];
+  const double4_32a ci = MIX ? double4_32a{} : a.c[ia];
   const double half = HALF ? 1.0 : 0.5;
+
+  // The lane's entries in rounds (almost always one): an FP32 test of the hi
+  // parts picks the skin entries that may be inside rc (few), then the inner
+  // entries and the picked ones go through `take`, so that the derivative's
+  // code runs for lanes that almost all have a pair in range.
+  __shared__ int sslot[MD_VJP_SLOTS][MD_BLOCK];
+  auto walk = [&](const RepGeo* g, int type, auto take) {
+    const float4 hi = __ldg(&a.xs[ia].hi);
+    const float hf0 = g->halfLf[0], hf1 = g->halfLf[1], hf2 = g->halfLf[2];
+    int left = nin, q = t;
+    do {
+      int nsv = 0;
+      for (; q < nsk && nsv < MD_VJP_SLOTS; q += TPA) {
+        const int j = __ldcs(skin - (int64_t)q * 32);
+        const float4 hj = __ldg(&a.xs[j].hi);
+        float dx = hj.x - hi.x, dy = hj.y - hi.y, dz = hj.z - hi.z;
+        dx = fabsf(dx) > hf0 ? dx - copysignf(g->Lf[0], dx) : dx;
+        dy = fabsf(dy) > hf1 ? dy - copysignf(g->Lf[1], dy) : dy;
+        dz = fabsf(dz) > hf2 ? dz - copysignf(g->Lf[2], dz) : dz;
+        const float r2f = __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, dx * dx));
+        const float cut = SINGLE ? a.cut1
+                                 : scut[type * a.nt + MD_TAG_TYPE(__float_as_int(hj.w))];
+        if (r2f <= cut) sslot[nsv++][threadIdx.x] = j;
+      }
+      const int own = left > t ? (left - t + TPA - 1) / TPA : 0;
+      left = 0;
+      for (int k = 0; k < own + nsv; k++)
+        take(k < own ? __ldcs(row + (int64_t)(t + k * TPA) * 32) : sslot[k - own][threadIdx.x]);
+    } while (q < nsk);
+  };
 
   double bx = 0.0, by = 0.0, bz = 0.0;  // xbar_i
   double ge0 = 0.0, gs0 = 0.0;          // parameter terms when SINGLE
-  double* slot = SINGLE ? nullptr : sg[threadIdx.x];
+  double* slot = SINGLE ? nullptr : &sg[0][threadIdx.x];
+  float2* slot2 = reinterpret_cast<float2*>(slot);
+  float geh = 0.f, gel = 0.f, gsh = 0.f, gsl = 0.f;  // mixed: parameter terms when SINGLE
   int ti;
 
   if (PREC == MD_PREC_FP64) {
@@ -99,8 +152,7 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
       constexpr bool WRAP = decltype(wrap)::value;
       const double L0 = g->L[0], L1 = g->L[1], L2 = g->L[2];
       const long long h0 = g->halfL_bits[0], h1 = g->halfL_bits[1], h2 = g->halfL_bits[2];
-      for (int q = t; q < nin + nsk; q += TPA) {
-        const int j = __ldcs(q < nin ? row + (int64_t)q * 32 : skin - (int64_t)(q - nin) * 32);
+      walk(g, ti, [&](int j) {
         const double4_32a xj = md_ld4(a.x4 + j);
         double dx = __dsub_rn(xj.x, xi.x);
         double dy = __dsub_rn(xj.y, xi.y);
@@ -147,11 +199,11 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
             ge0 += de;
             gs0 += ds;
           } else {
-            slot[tj] += de;
-            slot[MD_MAX_TYPES + tj] += ds;
+            slot[tj * MD_BLOCK] += de;
+            slot[(MD_MAX_TYPES + tj) * MD_BLOCK] += ds;
           }
         }
-      }
+      });
     };
     if (no_image)
       pairs(std::integral_constant<bool, false>{});
@@ -165,10 +217,10 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
     const float Lf0 = g->Lf[0], Lf1 = g->Lf[1], Lf2 = g->Lf[2];
     const float Ll0 = g->Llo[0], Ll1 = g->Llo[1], Ll2 = g->Llo[2];
     const float hf0 = g->halfLf[0], hf1 = g->halfLf[1], hf2 = g->halfLf[2];
-    const float cix = (float)ci.x, ciy = (float)ci.y, ciz = (float)ci.z;
+    const float4 cif = a.cf[ia];
+    const float cix = cif.x, ciy = cif.y, ciz = cif.z;
     float axh = 0.f, axl = 0.f, ayh = 0.f, ayl = 0.f, azh = 0.f, azl = 0.f;
-    for (int q = t; q < nin + nsk; q += TPA) {
-      const int j = __ldcs(q < nin ? row + (int64_t)q * 32 : skin - (int64_t)(q - nin) * 32);
+    walk(g, ti, [&](int j) {
       const XSplit sj = md_ld_split(a.xs + j);
       float hx = sj.hi.x - si.hi.x, lx = sj.lo.x - si.lo.x;
       float hy = sj.hi.y - si.hi.y, ly = sj.lo.y - si.lo.y;
@@ -202,8 +254,8 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
         const float r6inv = r2inv * r2inv * r2inv;
         const float gq = r6inv * (cf.lj1f * r6inv - cf.lj2f) * r2inv;
         const float gp = r2inv * r2inv * r6inv * (-7.0f * cf.lj1f * r6inv + 4.0f * cf.lj2f);
-        const double4_32a cj = a.c[j];
-        const float wx = cix - (float)cj.x, wy = ciy - (float)cj.y, wz = ciz - (float)cj.z;
+        const float4 cj = __ldg(a.cf + j);
+        const float wx = cix - cj.x, wy = ciy - cj.y, wz = ciz - cj.z;
         const float ew = -(dx * wx + dy * wy + dz * wz);
         const float s = -2.0f * gp * ew;
         const float jx = __fmaf_rn(s, dx, gq * wx);
@@ -218,16 +270,25 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
           atomicAdd(a.xbar + 2 * n + j, -md_widen(jz));
         }
         const float hw = (float)half * ew;
-        const double de = md_widen(hw * gq);
-        const double ds = md_widen(hw * r2inv * r6inv * (12.0f * cf.lj1f * r6inv - 6.0f * cf.lj2f));
+        // parameter terms: no FP64 operation per pair (an FP64 add costs 64
+        // cycles of its pipe); value and rounding error in FP32
+        const float de = hw * gq;
+        const float ds = hw * r2inv * r6inv * (12.0f * cf.lj1f * r6inv - 6.0f * cf.lj2f);
         if (SINGLE) {
-          ge0 += de;
-          gs0 += ds;
+          md_acc2(geh, gel, de);
+          md_acc2(gsh, gsl, ds);
         } else {
-          slot[tj] += de;
-          slot[MD_MAX_TYPES + tj] += ds;
+          float2 e2 = slot2[tj * MD_BLOCK], s2 = slot2[(MD_MAX_TYPES + tj) * MD_BLOCK];
+          md_acc2(e2.x, e2.y, de);
+          md_acc2(s2.x, s2.y, ds);
+          slot2[tj * MD_BLOCK] = e2;
+          slot2[(MD_MAX_TYPES + tj) * MD_BLOCK] = s2;
         }
       }
+    });
+    if (SINGLE) {
+      ge0 = md_widen(geh) + md_widen(gel);
+      gs0 = md_widen(gsh) + md_widen(gsl);
     }
     bx = md_widen(axh) + md_widen(axl);
     by = md_widen(ayh) + md_widen(ayl);
@@ -255,6 +316,7 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
   }
   // parameter terms: entry [min(ti,tj)][max(ti,tj)] of each table
   const int nt2 = a.nt * a.nt;
+  double* grow = a.gbar + (int64_t)(blockIdx.x % MD_GBAR_ROWS) * 2 * nt2;
   if (SINGLE) {
     double v[2] = {ge0, gs0};
 #pragma unroll
@@ -263,42 +325,47 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
       for (int off = 16; off > 0; off >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], off);
     }
     if ((threadIdx.x & 31) == 0) {
-      atomicAdd(a.gbar, v[0] * a.v1.inv_eps);
-      atomicAdd(a.gbar + nt2, v[1] * a.v1.inv_sigma);
+      atomicAdd(grow, v[0] * a.v1.inv_eps);
+      atomicAdd(grow + nt2, v[1] * a.v1.inv_sigma);
     }
   } else {
-    // thread k of the block sums table entry k (eps entries, then sigma)
-    // over the block's threads: one atomic per entry and block
-    __shared__ int stype[MD_BLOCK];
-    stype[threadIdx.x] = active ? ti : -1;
-    __syncthreads();
-    const int k = threadIdx.x;
-    if (k < 2 * nt2) {
-      const int w = k / nt2, e = k % nt2, ea = e / a.nt, eb = e % a.nt;
-      if (ea <= eb) {
-        double sum = 0.0;
-        for (int q = 0; q < MD_BLOCK; q++) {
-          const int tq = stype[q];
-          if (tq == ea) sum += sg[q][w * MD_MAX_TYPES + eb];
-          else if (tq == eb) sum += sg[q][w * MD_MAX_TYPES + ea];
+    // each warp sums each table entry over its lanes (a lane has terms of
+    // entry (ea, eb) if its atom's type is one of the two): one atomic per
+    // entry and warp
+    const int tt = active ? ti : -1;
+    for (int w = 0; w < 2; w++)
+      for (int ea = 0; ea < a.nt; ea++)
+        for (int eb = ea; eb < a.nt; eb++) {
+          const int o = tt == ea ? eb : (tt == eb ? ea : -1);
+          double v = 0.0;
+          if (MIX) {  // FP32 pairs
+            float2 p = o >= 0 ? slot2[(w * MD_MAX_TYPES + o) * MD_BLOCK] : make_float2(0.f, 0.f);
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+              const float h = __shfl_xor_sync(0xffffffffu, p.x, off);
+              p.y = __fadd_rn(p.y, __shfl_xor_sync(0xffffffffu, p.y, off));
+              md_acc2(p.x, p.y, h);
+            }
+            v = md_widen(p.x) + md_widen(p.y);
+          } else {
+            if (o >= 0) v = slot[(w * MD_MAX_TYPES + o) * MD_BLOCK];
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+          }
+          if ((threadIdx.x & 31) == 0 && v != 0.0) {
+            const VjpCoef& vc = sv[ea * a.nt + eb];
+            atomicAdd(grow + w * nt2 + ea * a.nt + eb, v * (w ? vc.inv_sigma : vc.inv_eps));
+          }
         }
-        const VjpCoef& vc = sv[ea * a.nt + eb];
-        if (sum != 0.0)
-          atomicAdd(a.gbar + w * nt2 + ea * a.nt + eb, sum * (w ? vc.inv_sigma : vc.inv_eps));
-      }
-    }
   }
 }
 
 template <int PREC, bool HALF, bool SINGLE>
 cudaError_t md_vjp_launch_tpa(const VjpArgs& a, int tpa, unsigned blocks, cudaStream_t s) {
   switch (tpa) {
-    case 1: k_vjp<PREC, HALF, 1, SINGLE><<<blocks, MD_BLOCK, 0, s>>>(a); break;
     case 2: k_vjp<PREC, HALF, 2, SINGLE><<<blocks, MD_BLOCK, 0, s>>>(a); break;
     case 4: k_vjp<PREC, HALF, 4, SINGLE><<<blocks, MD_BLOCK, 0, s>>>(a); break;
     case 8: k_vjp<PREC, HALF, 8, SINGLE><<<blocks, MD_BLOCK, 0, s>>>(a); break;
-    case 16: k_vjp<PREC, HALF, 16, SINGLE><<<blocks, MD_BLOCK, 0, s>>>(a); break;
-    case 32: k_vjp<PREC, HALF, 32, SINGLE><<<blocks, MD_BLOCK, 0, s>>>(a); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
