@@ -80,30 +80,28 @@ __global__ void k_sorted_to_caller(const double* __restrict__ soa,
   }
 }
 
-__global__ void k_resplit(const double4_32a* __restrict__ x4, XSplit* __restrict__ xs,
-                          XFix* __restrict__ xq, int64_t n, const XGrid gr) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  md_store_pos(x4[i], gr, xs, xq, i);
-}
-
 struct DtfArgs {
   double dtf[MD_MAX_TYPES];
 };
 
 // Undo the drift of step e-1 and form the next cotangent:
-// vbar += dt xbar;  c = mult (h/m) vbar.
-__global__ void k_adj_step(const double4_32a* __restrict__ x4, const double* __restrict__ xbar,
-                           double* __restrict__ vbar, double4_32a* __restrict__ c,
-                           float4* __restrict__ cf, int64_t n, double dt, double mult,
-                           DtfArgs d) {
+// vbar += dt xbar;  c = mult (h/m) vbar;  and, where x_prev is given, go back
+// to the positions of that evaluation (x4 and its records).
+__global__ void k_adj_step(const double4_32a* __restrict__ x_prev, double4_32a* __restrict__ x4,
+                           XSplit* __restrict__ xs, XFix* __restrict__ xq, const XGrid gr,
+                           const double* __restrict__ xbar, double* __restrict__ vbar,
+                           double4_32a* __restrict__ c, float4* __restrict__ cf, int64_t n,
+                           double dt, double mult, DtfArgs d) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const double hm = mult * d.dtf[md_type_of(x4[i])];
+  double4_32a p = x_prev ? x_prev[i] : x4[i];
+  const double bx = xbar[i], by = xbar[n + i], bz = xbar[2 * n + i];
+  double vx = vbar[i], vy = vbar[n + i], vz = vbar[2 * n + i];
+  const double hm = mult * d.dtf[md_type_of(p)];
   double4_32a q;
-  double vx = __fma_rn(dt, xbar[i], vbar[i]);
-  double vy = __fma_rn(dt, xbar[n + i], vbar[n + i]);
-  double vz = __fma_rn(dt, xbar[2 * n + i], vbar[2 * n + i]);
+  vx = __fma_rn(dt, bx, vx);
+  vy = __fma_rn(dt, by, vy);
+  vz = __fma_rn(dt, bz, vz);
   vbar[i] = vx;
   vbar[n + i] = vy;
   vbar[2 * n + i] = vz;
@@ -113,15 +111,34 @@ __global__ void k_adj_step(const double4_32a* __restrict__ x4, const double* __r
   q.w = 0.0;
   c[i] = q;
   if (cf) cf[i] = make_float4((float)q.x, (float)q.y, (float)q.z, 0.f);
+  if (x_prev) {
+    x4[i] = p;
+    md_store_pos(p, gr, xs, xq, i);
+  }
 }
 
-// max_i |F_i| as the bits of a non-negative double.
-__global__ void k_fmax(const double* __restrict__ f, int64_t n,
-                       unsigned long long* __restrict__ out) {
+// One steepest-descent step after a pair launch that left its sums unfolded:
+// k_fold_fmax folds the fixed-point sums into f (where fix is given) and takes
+// max_i |F_i| as the bits of a non-negative double; k_sd_step moves the atoms
+// by alpha F / max|F|, refreshes their records, zeroes f for the next pair
+// launch (where it accumulates) and clears the next step's maximum.
+__global__ void k_fold_fmax(double* __restrict__ f, unsigned long long* __restrict__ fix,
+                            int64_t n, unsigned long long* __restrict__ out) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   unsigned long long b = 0;
   if (i < n) {
-    const double fx = f[i], fy = f[n + i], fz = f[2 * n + i];
+    double fx = f[i], fy = f[n + i], fz = f[2 * n + i];
+    if (fix) {
+      fx = md_fold_add(fx, (long long)fix[i]);
+      fy = md_fold_add(fy, (long long)fix[n + i]);
+      fz = md_fold_add(fz, (long long)fix[2 * n + i]);
+      f[i] = fx;
+      f[n + i] = fy;
+      f[2 * n + i] = fz;
+      fix[i] = 0ULL;
+      fix[n + i] = 0ULL;
+      fix[2 * n + i] = 0ULL;
+    }
     b = (unsigned long long)__double_as_longlong(sqrt(fx * fx + fy * fy + fz * fz));
   }
 #pragma unroll
@@ -132,19 +149,28 @@ __global__ void k_fmax(const double* __restrict__ f, int64_t n,
   if ((threadIdx.x & 31) == 0 && b) atomicMax(out, b);
 }
 
-// x <- x + alpha F / max|F|
-__global__ void k_sd_update(double4_32a* __restrict__ x4, const double* __restrict__ f,
-                            int64_t n, double alpha, const unsigned long long* __restrict__ fmax) {
+__global__ void k_sd_step(double4_32a* __restrict__ x4, double* __restrict__ f, int64_t n,
+                          double alpha, const unsigned long long* __restrict__ fmax,
+                          unsigned long long* __restrict__ next, int zero,
+                          XSplit* __restrict__ xs, XFix* __restrict__ xq, const XGrid gr) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) *next = 0ULL;
   if (i >= n) return;
   const double m = __longlong_as_double((long long)*fmax);
+  const double fx = f[i], fy = f[n + i], fz = f[2 * n + i];
+  if (zero) {
+    f[i] = 0.0;
+    f[n + i] = 0.0;
+    f[2 * n + i] = 0.0;
+  }
   if (!(m > 0.0)) return;
   const double s = alpha / m;
   double4_32a p = x4[i];
-  p.x = __fma_rn(s, f[i], p.x);
-  p.y = __fma_rn(s, f[n + i], p.y);
-  p.z = __fma_rn(s, f[2 * n + i], p.z);
+  p.x = __fma_rn(s, fx, p.x);
+  p.y = __fma_rn(s, fy, p.y);
+  p.z = __fma_rn(s, fz, p.z);
   x4[i] = p;
+  md_store_pos(p, gr, xs, xq, i);
 }
 
 int upload_vcoef(md_ctx* c) {
@@ -261,14 +287,6 @@ int to_caller(md_ctx* c, const double* soa, const double4_32a* d4, double* dst) 
   return MD_OK;
 }
 
-int resplit(md_ctx* c) {
-  k_resplit<<<(unsigned)md_blocks(c->n), MD_BLOCK, 0, c->stream>>>(c->x4, c->xs, c->xq, c->n,
-                                                                   c->xgrid);
-  c->launches++;
-  MD_CUDA(cudaGetLastError());
-  return MD_OK;
-}
-
 int64_t n_checkpoints(int64_t nsteps, int every) { return (nsteps + every - 1) / every + 1; }
 
 }  // namespace
@@ -284,6 +302,13 @@ int md_set_lj(md_ctx* c, const double* eps, const double* sigma) {
       if (!(e > 0.0) || !(s > 0.0) || !isfinite(e) || !isfinite(s)) return MD_EINVAL;
       if (e != eps[b * nt + a] || s != sigma[b * nt + a]) return MD_EINVAL;
     }
+  // the coefficients the context holds already: nothing to upload, and the
+  // captured graphs stay (a backward pass sets those of its forward pass)
+  if (!memcmp(c->eps, eps, sizeof(double) * nt * nt) &&
+      !memcmp(c->sigma, sigma, sizeof(double) * nt * nt)) {
+    MD_CUDA(cudaStreamSynchronize(c->stream));
+    return MD_OK;
+  }
   for (int k = 0; k < nt * nt; k++) {
     c->eps[k] = eps[k];
     c->sigma[k] = sigma[k];
@@ -353,8 +378,16 @@ int md_traj_vjp(md_ctx* c, int64_t nsteps, int32_t every, const double* ckpt_x,
     const int64_t npos = e_hi - s0 + 1;
     MD_CUDA(cudaMemcpyAsync(c->seg_x, c->x4, sizeof(double4_32a) * n, cudaMemcpyDeviceToDevice,
                             c->stream));
+    // (no rebuild falls inside: the segment is shorter than the cadence; the
+    // forces at its last position are not needed)
+    const int fold = md_pair_fixed(c), zero = md_pair_accumulates(c);
     for (int64_t k = 1; k < npos; k++) {
-      MD_TRY(md_step(c, 1));
+      if (c->check_disp) {
+        MD_TRY(md_step(c, 1));
+      } else {
+        if (k > 1) MD_TRY(md_launch_pair_step(c));
+        MD_TRY(md_launch_integrate(c, k > 1 ? MD_K21 : MD_K1, k > 1 ? fold : 0, zero));
+      }
       MD_CUDA(cudaMemcpyAsync(c->seg_x + k * n, c->x4, sizeof(double4_32a) * n,
                               cudaMemcpyDeviceToDevice, c->stream));
     }
@@ -362,15 +395,14 @@ int md_traj_vjp(md_ctx* c, int64_t nsteps, int32_t every, const double* ckpt_x,
     MD_TRY(to_sorted(c, XB, c->adj_xbar, nullptr));
     MD_TRY(to_sorted(c, VB, c->adj_vbar, nullptr));
     MD_TRY(to_sorted(c, CC, nullptr, c->adj_c));
+    // the positions are those of e_hi here
     for (int64_t e = e_hi; e >= s0; e--) {
-      MD_CUDA(cudaMemcpyAsync(c->x4, c->seg_x + (e - s0) * n, sizeof(double4_32a) * n,
-                              cudaMemcpyDeviceToDevice, c->stream));
-      MD_TRY(resplit(c));
       MD_TRY(launch_vjp(c));
       if (e == 0) break;
       const double mult = (e - 1 >= 1) ? 2.0 : 1.0;
       k_adj_step<<<(unsigned)md_blocks(n), MD_BLOCK, 0, c->stream>>>(
-          c->x4, c->adj_xbar, c->adj_vbar, c->adj_c, c->adj_cf, n, c->dt, mult, d);
+          e > s0 ? c->seg_x + (e - 1 - s0) * n : nullptr, c->x4, c->xs, c->xq, c->xgrid,
+          c->adj_xbar, c->adj_vbar, c->adj_c, c->adj_cf, n, c->dt, mult, d);
       c->launches++;
       MD_CUDA(cudaGetLastError());
     }
@@ -387,17 +419,23 @@ int md_traj_vjp(md_ctx* c, int64_t nsteps, int32_t every, const double* ckpt_x,
 
 int md_minimize(md_ctx* c, int64_t nsteps, double alpha) {
   if (!c || nsteps < 0 || !(alpha > 0.0) || !isfinite(alpha)) return MD_EINVAL;
-  if (!c->fmax_bits) MD_TRY(dalloc(&c->fmax_bits, 1));
+  if (!c->fmax_bits) MD_TRY(dalloc(&c->fmax_bits, 2));
   const unsigned nb = (unsigned)md_blocks(c->n);
+  const int fold = md_pair_fixed(c), zero = md_pair_accumulates(c);
+  if (nsteps > 0) {
+    MD_CUDA(cudaMemsetAsync(c->fmax_bits, 0, 2 * sizeof(unsigned long long), c->stream));
+    if (zero) MD_CUDA(cudaMemsetAsync(c->f, 0, sizeof(double) * 3 * c->n, c->stream));
+  }
   for (int64_t s = 0; s < nsteps; s++) {
     if (s > 0 && s % c->rebuild_every == 0) MD_TRY(md_rebuild(c));
-    MD_TRY(md_launch_pair(c, 0, c->tpa > 0 ? c->tpa : 1));
-    MD_CUDA(cudaMemsetAsync(c->fmax_bits, 0, sizeof(unsigned long long), c->stream));
-    k_fmax<<<nb, MD_BLOCK, 0, c->stream>>>(c->f, c->n, c->fmax_bits);
-    k_sd_update<<<nb, MD_BLOCK, 0, c->stream>>>(c->x4, c->f, c->n, alpha, c->fmax_bits);
+    MD_TRY(md_launch_pair_step(c));
+    k_fold_fmax<<<nb, MD_BLOCK, 0, c->stream>>>(c->f, fold ? c->fix : nullptr, c->n,
+                                                c->fmax_bits + (s & 1));
+    k_sd_step<<<nb, MD_BLOCK, 0, c->stream>>>(c->x4, c->f, c->n, alpha, c->fmax_bits + (s & 1),
+                                              c->fmax_bits + ((s + 1) & 1), zero, c->xs, c->xq,
+                                              c->xgrid);
     c->launches += 2;
     MD_CUDA(cudaGetLastError());
-    MD_TRY(resplit(c));  // the mixed form reads positions from the split
   }
   c->step = 0;
   return md_fresh_start(c);

@@ -266,6 +266,9 @@ struct md_ctx {
 
   // graphs
   std::map<GraphKey, std::pair<cudaGraphExec_t, int>>* graphs;
+  cudaGraphExec_t rebuild_graph;  // wrap, sort and build (run_rebuild), or NULL
+  int rebuild_kernels;            // kernels in it
+  int rebuilds;                   // rebuilds run without it
 
   // counters
   int64_t step, builds, dangerous, launches;

