@@ -464,7 +464,7 @@ void free_ctx(md_ctx* c) {
                   c->stage,  c->rep,     c->vcoef,    c->adj_c,    c->adj_xbar, c->adj_vbar,
                   c->adj_carry, c->seg_x, c->gbar,     c->fmax_bits, c->cut_hi_dev,
                   c->tile_ctr, c->fix,   c->xq,       c->evs,       c->fxt,
-                  c->adj_cf};
+                  c->adj_cf, c->dstep};
   for (void* b : bufs)
     if (b) cudaFree(b);
   if (c->pair_ev) {
@@ -553,6 +553,7 @@ PairArgs pair_args(md_ctx* c) {
   a.maxneigh = c->maxneigh;
   a.nslots = c->nsm;
   a.tile_ctr = nullptr;
+  a.stop = DispStop{nullptr, 0.f};
   return a;
 }
 
@@ -612,9 +613,42 @@ int run_segment_timed(md_ctx* c, int m, int last_k2) {
   return MD_OK;
 }
 
-int run_segment(md_ctx* c, int m, int last_k2) {
+// The displacement^2 above which check_disp rebuilds, as the largest FP32
+// value not above it (an FP32 d2 > limit iff d2 > that value).
+float disp_limit(const md_ctx* c) {
+  const double half = 0.5 * c->skin;
+  return round_down_f(half * half * (1.0 - 1e-5));
+}
+
+// The kernels of a checked segment (DispStop): every kernel looks at the
+// displacement after the drift before it; the words go to the host at the end.
+int enqueue_checked(md_ctx* c, int m, int last_k2) {
+  const int fold = md_pair_fixed(c), zero = md_pair_accumulates(c);
+  const float lim = disp_limit(c);
+  cudaStream_t s = c->stream;
+  MD_CUDA(cudaMemsetAsync(c->dstep, 0, sizeof(unsigned int) * (m + 1), s));
+  for (int k = 0; k < m; k++) {
+    const DispStop stop{k ? c->dstep + k : c->dmax, lim};
+    MD_TRY(md_launch_pair_step(c, &stop));
+    if (last_k2 && k == m - 1)
+      MD_TRY(md_launch_integrate(c, MD_K2, fold, 0, &stop));
+    else
+      MD_TRY(md_launch_integrate(c, MD_K21, fold, zero, &stop, c->dstep + k + 1));
+  }
+  MD_CUDA(cudaMemcpyAsync(c->h_pinned + 16, c->dmax, sizeof(unsigned int),
+                          cudaMemcpyDeviceToHost, s));
+  MD_CUDA(cudaMemcpyAsync((unsigned int*)(c->h_pinned + 16) + 1, c->dstep + 1,
+                          sizeof(unsigned int) * m, cudaMemcpyDeviceToHost, s));
+  const int w = last_k2 ? m - 1 : m;  // drifts of the segment
+  if (w > 0)
+    MD_CUDA(cudaMemcpyAsync(c->dmax, c->dstep + w, sizeof(unsigned int),
+                            cudaMemcpyDeviceToDevice, s));
+  return MD_OK;
+}
+
+int run_segment(md_ctx* c, int m, int last_k2, int check = 0) {
   if (c->time_pair) return run_segment_timed(c, m, last_k2);
-  GraphKey key{m, last_k2};
+  GraphKey key{m, last_k2, check};
   auto it = c->graphs->find(key);
   if (it == c->graphs->end()) {
     cudaGraph_t g = nullptr;
@@ -622,7 +656,9 @@ int run_segment(md_ctx* c, int m, int last_k2) {
     int rc = MD_OK;
     const int64_t saved = c->launches;
     const int fold = md_pair_fixed(c), zero = md_pair_accumulates(c);
-    if (md_step_fused_ok(c)) {
+    if (check) {
+      rc = enqueue_checked(c, m, last_k2);
+    } else if (md_step_fused_ok(c)) {
       // P, then (K21 + P) as one launch per step, then the closing kick:
       // m + 1 launches for m steps
       rc = md_launch_pair_step(c);
@@ -630,7 +666,7 @@ int run_segment(md_ctx* c, int m, int last_k2) {
       if (rc == MD_OK) rc = md_launch_integrate(c, last_k2 ? MD_K2 : MD_K21, fold,
                                                 last_k2 ? 0 : zero);
     }
-    for (int k = 0; k < m && rc == MD_OK && !md_step_fused_ok(c); k++) {
+    for (int k = 0; k < m && rc == MD_OK && !check && !md_step_fused_ok(c); k++) {
       rc = md_launch_pair_step(c);
       if (rc != MD_OK) break;
       if (last_k2 && k == m - 1)
@@ -774,10 +810,11 @@ int create_impl(const md_params* p, int nrep, const int64_t* rep_off, const doub
           cudaSuccess)
     rc = MD_ECUDA;
   if (rc == MD_OK) rc = dalloc(&c->dmax, 8);
+  if (rc == MD_OK) rc = dalloc(&c->dstep, MD_STOP_STEPS + 1);
   if (rc == MD_OK) rc = dalloc(&c->i64_tmp, 4);
-  if (rc == MD_OK && cudaMallocHost((void**)&c->h_pinned, 16 * sizeof(double)) != cudaSuccess)
+  if (rc == MD_OK && cudaMallocHost((void**)&c->h_pinned, 32 * sizeof(double)) != cudaSuccess)
     rc = MD_ENOMEM;
-  if (rc == MD_OK) memset(c->h_pinned, 0, 16 * sizeof(double));
+  if (rc == MD_OK) memset(c->h_pinned, 0, 32 * sizeof(double));
   if (rc == MD_OK && cudaMallocHost((void**)&c->ev_host,
                                     sizeof(double) * (size_t)nrep * MD_EV_STRIDE) != cudaSuccess)
     rc = MD_ENOMEM;
@@ -875,9 +912,11 @@ namespace {
 
 // ev: energy and virial too; the virial's sum over atoms needs the final
 // forces, so it is only asked for with the fold in this call.
-int launch_pair_impl(md_ctx* c, int ev, int tpa, int prezeroed, int defer_fold) {
+int launch_pair_impl(md_ctx* c, int ev, int tpa, int prezeroed, int defer_fold,
+                     const DispStop* stop = nullptr) {
   if (ev && defer_fold) return MD_EINVAL;
   PairArgs a = pair_args(c);
+  if (stop) a.stop = *stop;
   a.tile_ctr = c->persist ? c->tile_ctr : nullptr;
   if (c->persist)
     MD_CUDA(cudaMemsetAsync(c->tile_ctr, 0, sizeof(int) * c->nsm, c->stream));
@@ -933,7 +972,9 @@ int launch_pair_impl(md_ctx* c, int ev, int tpa, int prezeroed, int defer_fold) 
 // sums folded): the form every caller outside the step segments uses.
 int md_launch_pair(md_ctx* c, int ev, int tpa) { return launch_pair_impl(c, ev, tpa, 0, 0); }
 
-int md_launch_pair_step(md_ctx* c) { return launch_pair_impl(c, 0, c->tpa, 1, 1); }
+int md_launch_pair_step(md_ctx* c, const DispStop* stop) {
+  return launch_pair_impl(c, 0, c->tpa, 1, 1, stop);
+}
 
 // ---- C ABI ----------------------------------------------------------------------
 
@@ -1056,10 +1097,9 @@ int md_step(md_ctx* c, int64_t nsteps) {
   const int64_t every = c->rebuild_every;
   // the first pair launch of the step adds into f: K1 leaves it at zero
   MD_TRY(md_launch_integrate(c, MD_K1, 0, md_pair_accumulates(c)));
-  if (c->check_disp) {
+  if (c->check_disp && c->time_pair) {
     // one step per segment; after each drift the largest displacement since
     // the build decides whether the list is rebuilt before the next forces
-    const double half = 0.5 * c->skin;
     for (int64_t k = 0; k < nsteps; k++) {
       const int64_t s = c->step + k;
       bool rebuild = (s + 1) % every == 0;
@@ -1067,14 +1107,38 @@ int md_step(md_ctx* c, int64_t nsteps) {
         MD_CUDA(cudaMemcpyAsync(c->h_pinned + 13, c->dmax, sizeof(unsigned int),
                                 cudaMemcpyDeviceToHost, c->stream));
         MD_CUDA(cudaStreamSynchronize(c->stream));
-        unsigned int bits;
-        memcpy(&bits, (const char*)(c->h_pinned + 13), sizeof(bits));
         float d2;
-        memcpy(&d2, &bits, sizeof(d2));
-        rebuild = (double)d2 > half * half * (1.0 - 1e-5);
+        memcpy(&d2, (const char*)(c->h_pinned + 13), sizeof(d2));
+        rebuild = d2 > disp_limit(c);
       }
       if (rebuild) MD_TRY(md_rebuild(c));
       MD_TRY(run_segment(c, 1, k == nsteps - 1));
+    }
+    c->step += nsteps;
+    return MD_OK;
+  }
+  if (c->check_disp) {
+    // segments of several steps whose kernels stop by themselves once the
+    // displacement after a drift asks for a rebuild before the next forces:
+    // one synchronization per segment instead of one per step
+    const float lim = disp_limit(c);
+    int64_t k = 0;
+    while (k < nsteps) {
+      const int64_t r = (c->step + k + 1) % every;
+      if (r == 0) MD_TRY(md_rebuild(c));
+      int64_t m = r == 0 ? every : every - r;
+      if (m > nsteps - k) m = nsteps - k;
+      if (m > MD_STOP_STEPS) m = MD_STOP_STEPS;
+      MD_TRY(run_segment(c, (int)m, k + m == nsteps, 1));
+      MD_CUDA(cudaStreamSynchronize(c->stream));
+      float d2[MD_STOP_STEPS + 1];
+      memcpy(d2, (const char*)(c->h_pinned + 16), sizeof(float) * (m + 1));
+      // steps done before the first drift beyond the limit; the list is
+      // rebuilt there unless the cadence does it anyway
+      int64_t done = 0;
+      while (done < m && !(d2[done] > lim)) done++;
+      k += done;
+      if (k < nsteps && d2[done] > lim && (c->step + k + 1) % every != 0) MD_TRY(md_rebuild(c));
     }
     c->step += nsteps;
     return MD_OK;

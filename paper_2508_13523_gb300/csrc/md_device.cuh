@@ -12,6 +12,11 @@
 
 #include "md_internal.cuh"
 
+// Whether a checked segment has stopped (DispStop).
+__device__ __forceinline__ bool md_stopped(const DispStop& s) {
+  return s.disp && __uint_as_float(*s.disp) > s.lim;
+}
+
 // |d| > h for a finite double d and a positive double h, as an integer
 // compare of the bit patterns (IEEE doubles of one sign order like their
 // bit patterns).  Avoids a DSETP on the FP64 pipe.

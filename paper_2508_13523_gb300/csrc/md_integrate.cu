@@ -31,6 +31,11 @@ namespace {
 template <int MODE>
 __global__ void __launch_bounds__(MD_BLOCK) k_integrate(const IntArgs a) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (a.stop.disp) {
+    // the word after this drift is at least the one before it
+    if (MODE != MD_K2 && i == 0 && a.dmax != a.stop.disp) atomicMax(a.dmax, *a.stop.disp);
+    if (md_stopped(a.stop)) return;
+  }
   const float disp2 = i < a.n ? md_integrate_atom<MODE>(a, i) : 0.f;
   if (MODE != MD_K2) md_disp_max(disp2, a.dmax);
 }
@@ -247,14 +252,18 @@ IntArgs md_int_args(md_ctx* c, int fold, int zero) {
   a.gr = c->xgrid;
   a.xb = c->xb;
   a.dmax = c->dmax;
+  a.stop = DispStop{nullptr, 0.f};
   a.n = c->n;
   a.dt = c->dt;
   for (int t = 0; t < MD_MAX_TYPES; t++) a.dtf[t] = c->dtf[t];
   return a;
 }
 
-int md_launch_integrate(md_ctx* c, int mode, int fold, int zero) {
-  const IntArgs a = md_int_args(c, fold, zero);
+int md_launch_integrate(md_ctx* c, int mode, int fold, int zero, const DispStop* stop,
+                        unsigned int* disp_out) {
+  IntArgs a = md_int_args(c, fold, zero);
+  if (stop) a.stop = *stop;
+  if (disp_out) a.dmax = disp_out;
   const unsigned nb = (unsigned)md_blocks(c->n);
   if (mode == MD_K1)
     k_integrate<MD_K1><<<nb, MD_BLOCK, 0, c->stream>>>(a);

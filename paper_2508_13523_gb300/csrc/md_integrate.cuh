@@ -20,6 +20,8 @@ struct IntArgs {
   const XSplit* xb;
   XGrid gr;
   unsigned int* dmax;
+  DispStop stop;            // segments that check the displacement (no kernel of a step
+                            // runs once it is beyond the limit)
   int64_t n;
   double dt;
   double dtf[MD_MAX_TYPES];

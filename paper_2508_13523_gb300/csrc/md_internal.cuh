@@ -143,12 +143,23 @@ struct __align__(32) XFix {
   long long w;  // the atom's tag (as md_tag_of(x4)) | F << 32
 };
 
+// Segments of check_disp contexts: *disp holds the largest displacement^2
+// since the build (bits) after the step's drift; kernels that come after it
+// return at once where it is above lim, so that the host can rebuild the list
+// and go on from that drift.  disp NULL: no check.
+struct DispStop {
+  const unsigned int* disp;
+  float lim;
+};
+#define MD_STOP_STEPS 16  // steps per checked segment
+
 // ---- context -----------------------------------------------------------------
 struct GraphKey {
   int m;        // force/integrate pairs in the segment
   int last_k2;  // segment ends with the final half kick
+  int check;    // the segment checks the displacement (DispStop)
   bool operator<(const GraphKey& o) const {
-    return m != o.m ? m < o.m : last_k2 < o.last_k2;
+    return m != o.m ? m < o.m : last_k2 != o.last_k2 ? last_k2 < o.last_k2 : check < o.check;
   }
 };
 
@@ -247,7 +258,9 @@ struct md_ctx {
                        // [4] that state changed some position (0/1),
                        // [5] a fused step's grid barrier timed out (0/1),
                        // [6], [7] that barrier's arrivals and generation
-  double* h_pinned;    // small pinned host mirror (16 doubles)
+  unsigned int* dstep; // check_disp: the displacement word after each drift of a segment
+                       // (MD_STOP_STEPS + 1; [0] unused, dmax[0] takes its place)
+  double* h_pinned;    // small pinned host mirror (32 doubles; [16..] dstep)
   int64_t* i64_tmp;    // device int64 scratch (counts)
 
   // host staging for MD_MEM_HOST
@@ -290,7 +303,7 @@ void md_drop_graphs(md_ctx* c);
 int md_launch_pair(md_ctx* c, int ev, int tpa);
 // step-segment form: f (and the fixed-point sums) are already zero, and the
 // next integrator launch folds the fixed-point sums
-int md_launch_pair_step(md_ctx* c);
+int md_launch_pair_step(md_ctx* c, const DispStop* stop = nullptr);
 int md_pair_accumulates(const md_ctx* c);  // the pair launch adds into f (needs f = 0)
 int md_pair_fixed(const md_ctx* c);        // the pair launch leaves sums in fix
 int md_launch_fix_finalize(md_ctx* c);  // md_integrate.cu
@@ -312,7 +325,10 @@ int md_upload_coef(md_ctx* c);  // coefficients, FP32 filter bounds, single-type
 enum { MD_K1 = 0, MD_K21 = 1, MD_K2 = 2 };
 // fold: add the fixed-point sums into f first (and zero them); zero: K1/K21
 // leave f = 0 for a pair launch that accumulates
-int md_launch_integrate(md_ctx* c, int mode, int fold = 0, int zero = 0);
+// stop: see DispStop; disp_out: the word that receives the displacement after
+// the drift (default dmax[0]), at least stop's
+int md_launch_integrate(md_ctx* c, int mode, int fold = 0, int zero = 0,
+                        const DispStop* stop = nullptr, unsigned int* disp_out = nullptr);
 int md_launch_kinetic(md_ctx* c);
 int md_launch_virial_atoms(md_ctx* c);  // sum_a (x_a - c) (x) F_a into evs words 1..6
 int md_launch_ev_fold(md_ctx* c);       // ev += the sums of the evs rows; evs = 0

@@ -72,6 +72,7 @@ struct PairArgs {
   int* tile_ctr;         // per-SM tile counters (zeroed before each launch), or
                          // NULL: one tile per block
   int nslots;            // counters (= SMs)
+  DispStop stop;
   int64_t n;
   int nt;
   int maxneigh;
@@ -131,6 +132,7 @@ constexpr int md_pair_minb(int prec, bool half, bool ev) {
 template <int PREC, bool HALF, int TPA, bool EV, bool SINGLE, bool COUL = false>
 __global__ void __launch_bounds__(MD_BLOCK, md_pair_minb(PREC, HALF, EV)) k_pair(const PairArgs a) {
   static_assert(!COUL || PREC == MD_PREC_MIXED, "the FP64 Coulomb form is k_pair_q");
+  if (md_stopped(a.stop)) return;
   __shared__ PairCoef sc[SINGLE ? 1 : MD_MAX_TYPES * MD_MAX_TYPES];
   if (!SINGLE) {
     for (int k = threadIdx.x; k < a.nt * a.nt; k += blockDim.x) sc[k] = a.coef[k];

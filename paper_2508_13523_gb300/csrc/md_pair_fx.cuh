@@ -410,6 +410,7 @@ template <bool HALF, bool EV, bool SINGLE, bool COUL, int T, int U>
 __global__ void __launch_bounds__(MD_BLOCK, md_pair_fx_minb(HALF, EV))
     k_pair_fx(const __grid_constant__ PairArgs a, const float cut_hi1,
               const float* __restrict__ cut_hi_tab) {
+  if (md_stopped(a.stop)) return;
   md_pair_fx_tiles<HALF, EV, SINGLE, COUL, T, U>(a, cut_hi1, cut_hi_tab);
 }
 

@@ -296,6 +296,7 @@ constexpr int md_pair_q_minb(bool half, bool ev) { return ev ? (half ? 8 : 10) :
 template <bool HALF, bool EV, bool SINGLE, bool COUL>
 __global__ void __launch_bounds__(MD_BLOCK, md_pair_q_minb(HALF, EV))
     k_pair_q(const PairArgs a, const float cut_hi1, const float* __restrict__ cut_hi_tab) {
+  if (md_stopped(a.stop)) return;
   md_pair_q_tiles<HALF, EV, SINGLE, COUL>(a, cut_hi1, cut_hi_tab);
 }
 

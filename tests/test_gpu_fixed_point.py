@@ -193,3 +193,28 @@ def test_coulomb(case, kind):
     ec = (qqrd2e * np.abs(qt[t[i]] * qt[t[j]]) / np.sqrt(r2)).sum()
     assert abs(th.pe - E) <= 1e-12 * max(abs(E), np.abs(W).max(), ec) + noise
     assert np.abs(th.virial - W).max() <= 1e-12 * max(np.abs(W).max(), ec) + noise
+
+
+@pytest.mark.parametrize("prec", [md.MD_PREC_FP64, md.MD_PREC_MIXED])
+@pytest.mark.parametrize("every", [50, 7])
+def test_check_disp_segments(prec, every):
+    """check_disp runs several steps per launch and stops them on the device
+    where a displacement asks for a rebuild: the same builds and, bit for bit,
+    the same trajectory as one call per step (order-independent force sums)."""
+    x, box = lattice(6, 0.8442, 0.1, 91)
+    v = S.maxwell_boltzmann(np.ones(len(x)), 2.0, 92)
+    runs = []
+    for calls in ([61], [1] * 61, [20, 1, 40]):
+        with md.LJMD(x, v, None, box, 1.0, 1.0, 2.5, 1.0, precision=prec, check_disp=True,
+                     rebuild_every=every, threads_per_atom=1, list_kind=md.MD_LIST_HALF) as ctx:
+            ctx.set_kernel(1, -1, 2 if prec == md.MD_PREC_FP64 else 0, 0)
+            ctx.compute_forces(0)  # the initial forces with order-independent sums too
+            for k in calls:
+                ctx.step(k)
+            st = ctx.stats()
+            runs.append((st["builds"], st["max_disp"], [a.cpu().numpy() for a in ctx.get_state()]))
+    assert runs[0][0] > 61 // every + 2  # builds between the cadence's
+    for r in runs[1:]:
+        assert r[:2] == runs[0][:2]
+        for a, b in zip(r[2], runs[0][2]):
+            np.testing.assert_array_equal(a, b)
