@@ -464,7 +464,7 @@ void free_ctx(md_ctx* c) {
                   c->stage,  c->rep,     c->vcoef,    c->adj_c,    c->adj_xbar, c->adj_vbar,
                   c->adj_carry, c->seg_x, c->gbar,     c->fmax_bits, c->cut_hi_dev,
                   c->tile_ctr, c->fix,   c->xq,       c->evs,       c->fxt,
-                  c->adj_cf, c->dstep};
+                  c->adj_cf, c->dstep,   c->fmark};
   for (void* b : bufs)
     if (b) cudaFree(b);
   if (c->pair_ev) {
@@ -554,6 +554,7 @@ PairArgs pair_args(md_ctx* c) {
   a.nslots = c->nsm;
   a.tile_ctr = nullptr;
   a.stop = DispStop{nullptr, 0.f};
+  a.fmark = nullptr;
   return a;
 }
 
@@ -604,11 +605,11 @@ int run_segment_timed(md_ctx* c, int m, int last_k2) {
     return md_launch_integrate(c, last_k2 ? MD_K2 : MD_K21, fold, last_k2 ? 0 : zero);
   }
   for (int k = 0; k < m; k++) {
-    MD_TRY(timed([&] { return md_launch_pair_step(c); }));
+    MD_TRY(timed([&] { return md_launch_pair_step(c, nullptr, k); }));
     if (last_k2 && k == m - 1)
-      MD_TRY(md_launch_integrate(c, MD_K2, fold, 0));
+      MD_TRY(md_launch_integrate(c, MD_K2, fold, 0, nullptr, nullptr, k));
     else
-      MD_TRY(md_launch_integrate(c, MD_K21, fold, zero));
+      MD_TRY(md_launch_integrate(c, MD_K21, fold, zero, nullptr, nullptr, k));
   }
   return MD_OK;
 }
@@ -667,12 +668,12 @@ int run_segment(md_ctx* c, int m, int last_k2, int check = 0) {
                                                 last_k2 ? 0 : zero);
     }
     for (int k = 0; k < m && rc == MD_OK && !check && !md_step_fused_ok(c); k++) {
-      rc = md_launch_pair_step(c);
+      rc = md_launch_pair_step(c, nullptr, k);
       if (rc != MD_OK) break;
       if (last_k2 && k == m - 1)
-        rc = md_launch_integrate(c, MD_K2, fold, 0);
+        rc = md_launch_integrate(c, MD_K2, fold, 0, nullptr, nullptr, k);
       else
-        rc = md_launch_integrate(c, MD_K21, fold, zero);
+        rc = md_launch_integrate(c, MD_K21, fold, zero, nullptr, nullptr, k);
     }
     const int kernels = (int)(c->launches - saved);
     c->launches = saved;
@@ -772,8 +773,9 @@ int create_impl(const md_params* p, int nrep, const int64_t* rep_off, const doub
   if (rc == MD_OK) rc = dalloc(&c->f, 3 * n);
   if (rc == MD_OK) rc = dalloc(&c->fix, 3 * n);
   if (rc == MD_OK) rc = dalloc(&c->id, n);
-  if (rc == MD_OK) rc = dalloc(&c->xs, n);
-  if (rc == MD_OK) rc = dalloc(&c->xb, n);
+  const int64_t nhi = c->precision == MD_PREC_FP64 ? (n + 1) / 2 : n;  // md_ld_hi
+  if (rc == MD_OK) rc = dalloc(&c->xs, nhi);
+  if (rc == MD_OK) rc = dalloc(&c->xb, nhi);
   if (rc == MD_OK && c->precision == MD_PREC_FP64) rc = dalloc(&c->xq, n);
   if (rc == MD_OK) rc = dalloc(&c->cell, n);
   if (rc == MD_OK) rc = dalloc(&c->tag0, n);
@@ -811,6 +813,7 @@ int create_impl(const md_params* p, int nrep, const int64_t* rep_off, const doub
     rc = MD_ECUDA;
   if (rc == MD_OK) rc = dalloc(&c->dmax, 8);
   if (rc == MD_OK) rc = dalloc(&c->dstep, MD_STOP_STEPS + 1);
+  if (rc == MD_OK) rc = dalloc(&c->fmark, 3);
   if (rc == MD_OK) rc = dalloc(&c->i64_tmp, 4);
   if (rc == MD_OK && cudaMallocHost((void**)&c->h_pinned, 32 * sizeof(double)) != cudaSuccess)
     rc = MD_ENOMEM;
@@ -836,6 +839,7 @@ int create_impl(const md_params* p, int nrep, const int64_t* rep_off, const doub
         cudaMemcpyAsync(off_dev, rep_off, sizeof(int64_t) * (nrep + 1), cudaMemcpyHostToDevice,
                         s) == cudaSuccess &&
         cudaMemsetAsync(c->dmax, 0, 8 * sizeof(unsigned int), s) == cudaSuccess &&
+        cudaMemsetAsync(c->fmark, 0, 3 * sizeof(int), s) == cudaSuccess &&
         cudaMemsetAsync(c->f, 0, sizeof(double) * 3 * n, s) == cudaSuccess &&
         cudaMemsetAsync(c->fix, 0, sizeof(unsigned long long) * 3 * n, s) == cudaSuccess;
     if (ok) {
@@ -913,10 +917,11 @@ namespace {
 // ev: energy and virial too; the virial's sum over atoms needs the final
 // forces, so it is only asked for with the fold in this call.
 int launch_pair_impl(md_ctx* c, int ev, int tpa, int prezeroed, int defer_fold,
-                     const DispStop* stop = nullptr) {
+                     const DispStop* stop = nullptr, int mark = -1) {
   if (ev && defer_fold) return MD_EINVAL;
   PairArgs a = pair_args(c);
   if (stop) a.stop = *stop;
+  if (mark >= 0) a.fmark = c->fmark + mark % 3;
   a.tile_ctr = c->persist ? c->tile_ctr : nullptr;
   if (c->persist)
     MD_CUDA(cudaMemsetAsync(c->tile_ctr, 0, sizeof(int) * c->nsm, c->stream));
@@ -972,8 +977,8 @@ int launch_pair_impl(md_ctx* c, int ev, int tpa, int prezeroed, int defer_fold,
 // sums folded): the form every caller outside the step segments uses.
 int md_launch_pair(md_ctx* c, int ev, int tpa) { return launch_pair_impl(c, ev, tpa, 0, 0); }
 
-int md_launch_pair_step(md_ctx* c, const DispStop* stop) {
-  return launch_pair_impl(c, 0, c->tpa, 1, 1, stop);
+int md_launch_pair_step(md_ctx* c, const DispStop* stop, int mark) {
+  return launch_pair_impl(c, 0, c->tpa, 1, 1, stop, mark);
 }
 
 // ---- C ABI ----------------------------------------------------------------------

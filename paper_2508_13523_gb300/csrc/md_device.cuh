@@ -262,11 +262,18 @@ __device__ __forceinline__ bool md_xfix(double x, int F, long long& X) {
   return true;
 }
 
+// Hi parts and tag of atom i: FP64 contexts keep only them, 16 bytes an atom
+// (HS = 0: nothing there reads lo), mixed contexts whole XSplit records (HS = 1).
+template <int HS>
+__device__ __forceinline__ float4 md_ld_hi(const XSplit* xs, int64_t i) {
+  return __ldg(reinterpret_cast<const float4*>(xs) + (i << HS));
+}
+
 // Store the position p of atom i into its derived records: the double-float
 // split (md_split; tag in hi.w) and, where xq is given (FP64 contexts), the
 // fixed-point record, with MD_TAG_OFFGRID in its tag when some coordinate has
 // no fixed-point form.  FP64 contexts keep only the hi
-// parts of the split (lo = 0).  Returns the split.
+// parts of the split (md_ld_hi).  Returns the split.
 __device__ __forceinline__ XSplit md_store_pos(const double4_32a& p, const XGrid& gr,
                                                XSplit* __restrict__ xs, XFix* __restrict__ xq,
                                                int64_t i, XSplit* __restrict__ xb = nullptr);
@@ -332,8 +339,13 @@ __device__ __forceinline__ XSplit md_store_pos(const double4_32a& p, const XGrid
   }
   s.hi.w = __int_as_float(tag);
   s.lo.w = 0.f;
-  xs[i] = s;
-  if (xb) xb[i] = s;
+  if (xq) {
+    reinterpret_cast<float4*>(xs)[i] = s.hi;
+    if (xb) reinterpret_cast<float4*>(xb)[i] = s.hi;
+  } else {
+    xs[i] = s;
+    if (xb) xb[i] = s;
+  }
   return s;
 }
 

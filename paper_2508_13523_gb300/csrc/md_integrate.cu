@@ -36,6 +36,7 @@ __global__ void __launch_bounds__(MD_BLOCK) k_integrate(const IntArgs a) {
     if (MODE != MD_K2 && i == 0 && a.dmax != a.stop.disp) atomicMax(a.dmax, *a.stop.disp);
     if (md_stopped(a.stop)) return;
   }
+  if (MODE == MD_K21 && i == 0 && a.fclear) *a.fclear = 0;
   const float disp2 = i < a.n ? md_integrate_atom<MODE>(a, i) : 0.f;
   if (MODE != MD_K2) md_disp_max(disp2, a.dmax);
 }
@@ -187,7 +188,13 @@ __global__ void k_load_keep(const double* __restrict__ x, const double* __restri
     double4_32a q = x4[p];
     const double nx = x[3 * o], ny = x[3 * o + 1], nz = x[3 * o + 2];
     const double wx = v[3 * o], wy = v[3 * o + 1], wz = v[3 * o + 2];
-    const XSplit b = xb[p];  // every load before the stores
+    XSplit b;  // every load before the stores
+    if (xq) {
+      b.hi = md_ld_hi<0>(xb, p);
+      b.lo = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else {
+      b = xb[p];
+    }
     moved = (__double_as_longlong(nx) != __double_as_longlong(q.x)) |
             (__double_as_longlong(ny) != __double_as_longlong(q.y)) |
             (__double_as_longlong(nz) != __double_as_longlong(q.z));
@@ -247,6 +254,8 @@ IntArgs md_int_args(md_ctx* c, int fold, int zero) {
   a.f = c->f;
   a.fix = fold ? c->fix : nullptr;
   a.zero = zero;
+  a.fmark = nullptr;
+  a.fclear = nullptr;
   a.xs = c->xs;
   a.xq = c->xq;
   a.gr = c->xgrid;
@@ -260,8 +269,12 @@ IntArgs md_int_args(md_ctx* c, int fold, int zero) {
 }
 
 int md_launch_integrate(md_ctx* c, int mode, int fold, int zero, const DispStop* stop,
-                        unsigned int* disp_out) {
+                        unsigned int* disp_out, int mark) {
   IntArgs a = md_int_args(c, fold, zero);
+  if (mark >= 0 && fold) {
+    a.fmark = c->fmark + mark % 3;
+    a.fclear = c->fmark + (mark + 2) % 3;
+  }
   if (stop) a.stop = *stop;
   if (disp_out) a.dmax = disp_out;
   const unsigned nb = (unsigned)md_blocks(c->n);

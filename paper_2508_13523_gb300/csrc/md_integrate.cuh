@@ -15,6 +15,9 @@ struct IntArgs {
   double* f;
   unsigned long long* fix;  // fixed-point sums to fold into f (then zeroed), or NULL
   int zero;                 // K1/K21: leave f = 0 for the next pair launch's sums
+  const int* fmark;         // nonzero if the last pair launch added into f, or NULL
+                            // (unknown); with fix and zero only
+  int* fclear;              // K21: cleared for the pair launch after the next
   XSplit* xs;
   XFix* xq;
   const XSplit* xb;
@@ -37,7 +40,6 @@ __device__ __forceinline__ float md_integrate_atom(const IntArgs& a, int64_t i) 
   // of its loads, so all of an atom's are in flight at once
   double4_32a p = a.x4[i];
   double vx = a.v[i], vy = a.v[n + i], vz = a.v[2 * n + i];
-  double fx = a.f[i], fy = a.f[n + i], fz = a.f[2 * n + i];
   long long qx = 0, qy = 0, qz = 0;
   if (a.fix) {
     qx = (long long)a.fix[i];
@@ -45,7 +47,23 @@ __device__ __forceinline__ float md_integrate_atom(const IntArgs& a, int64_t i) 
     qz = (long long)a.fix[2 * n + i];
   }
   XSplit b;
-  if (MODE != MD_K2) b = a.xb[i];
+  if (MODE != MD_K2) {
+    if (a.xq) {
+      b.hi = reinterpret_cast<const float4*>(a.xb)[i];
+      b.lo = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else {
+      b = a.xb[i];
+    }
+  }
+  // f holds only what was beyond the fixed-point sums' range: +0 everywhere
+  // unless the pair launch has marked its word
+  const bool clean = MODE != MD_K1 && a.fmark && *a.fmark == 0;
+  double fx = 0.0, fy = 0.0, fz = 0.0;
+  if (!clean) {
+    fx = a.f[i];
+    fy = a.f[n + i];
+    fz = a.f[2 * n + i];
+  }
   const double h = a.dtf[md_type_of(p)];
   if (a.fix) {  // the last pair launch left its fixed-point sums unfolded
     fx = md_fold_add(fx, qx);
@@ -75,9 +93,11 @@ __device__ __forceinline__ float md_integrate_atom(const IntArgs& a, int64_t i) 
   a.v[n + i] = vy;
   a.v[2 * n + i] = vz;
   if (MODE != MD_K2 && a.zero) {
-    a.f[i] = 0.0;
-    a.f[n + i] = 0.0;
-    a.f[2 * n + i] = 0.0;
+    if (!clean) {
+      a.f[i] = 0.0;
+      a.f[n + i] = 0.0;
+      a.f[2 * n + i] = 0.0;
+    }
   } else if (a.fix) {
     a.f[i] = fx;
     a.f[n + i] = fy;

@@ -216,8 +216,9 @@ struct md_ctx {
   unsigned long long* fix;  // SoA 3n fixed-point force accumulators (FP64 compact == 2,
                             // and every mixed form); zero between pair launches
   int32_t* id;      // caller index of each sorted atom
-  XSplit* xs;       // double-float split of x4 (build filter, mixed gathers)
-  XSplit* xb;       // split of the positions at the last build (displacement)
+  XSplit* xs;       // double-float split of x4 (build filter, mixed gathers); FP64
+                    // contexts: the hi parts alone, one float4 an atom (md_ld_hi)
+  XSplit* xb;       // the same of the positions at the last build (displacement)
   XFix* xq;         // FP64 contexts: fixed-point positions (valid where xs's tag has no
                     // MD_TAG_OFFGRID); NULL for mixed precision
   int32_t* cell;    // global cell index of each sorted atom
@@ -258,6 +259,12 @@ struct md_ctx {
                        // [4] that state changed some position (0/1),
                        // [5] a fused step's grid barrier timed out (0/1),
                        // [6], [7] that barrier's arrivals and generation
+  // Step segments with fixed-point sums: word k % 3 is nonzero if the pair
+  // launch of step k added into f (contributions beyond the sums' range, rare);
+  // that step's integrator then reads f and zeroes it, and otherwise leaves it
+  // (48 of about 290 bytes an atom).  The integrator of step k clears the word
+  // of step k + 2; a word left set by an earlier segment costs one such pass.
+  int* fmark;
   unsigned int* dstep; // check_disp: the displacement word after each drift of a segment
                        // (MD_STOP_STEPS + 1; [0] unused, dmax[0] takes its place)
   double* h_pinned;    // small pinned host mirror (32 doubles; [16..] dstep)
@@ -303,7 +310,9 @@ void md_drop_graphs(md_ctx* c);
 int md_launch_pair(md_ctx* c, int ev, int tpa);
 // step-segment form: f (and the fixed-point sums) are already zero, and the
 // next integrator launch folds the fixed-point sums
-int md_launch_pair_step(md_ctx* c, const DispStop* stop = nullptr);
+// (mark: the step's number in its segment, whose word of fmark the launch sets
+// where it adds into f; -1: none)
+int md_launch_pair_step(md_ctx* c, const DispStop* stop = nullptr, int mark = -1);
 int md_pair_accumulates(const md_ctx* c);  // the pair launch adds into f (needs f = 0)
 int md_pair_fixed(const md_ctx* c);        // the pair launch leaves sums in fix
 int md_launch_fix_finalize(md_ctx* c);  // md_integrate.cu
@@ -326,9 +335,10 @@ enum { MD_K1 = 0, MD_K21 = 1, MD_K2 = 2 };
 // fold: add the fixed-point sums into f first (and zero them); zero: K1/K21
 // leave f = 0 for a pair launch that accumulates
 // stop: see DispStop; disp_out: the word that receives the displacement after
-// the drift (default dmax[0]), at least stop's
+// the drift (default dmax[0]), at least stop's; mark: as the pair launch before
 int md_launch_integrate(md_ctx* c, int mode, int fold = 0, int zero = 0,
-                        const DispStop* stop = nullptr, unsigned int* disp_out = nullptr);
+                        const DispStop* stop = nullptr, unsigned int* disp_out = nullptr,
+                        int mark = -1);
 int md_launch_kinetic(md_ctx* c);
 int md_launch_virial_atoms(md_ctx* c);  // sum_a (x_a - c) (x) F_a into evs words 1..6
 int md_launch_ev_fold(md_ctx* c);       // ev += the sums of the evs rows; evs = 0

@@ -217,6 +217,11 @@ __global__ void k_restore(const double4_32a* __restrict__ x4n, const double* __r
   md_store_pos(p, gr, xs, xq, i, xb);
 }
 
+// md_ld_hi with the records' kind (hs) at run time
+__device__ __forceinline__ float4 ld_hi(const XSplit* xs, int64_t i, int hs) {
+  return __ldg(reinterpret_cast<const float4*>(xs) + (i << hs));
+}
+
 // FP32 minimum image of one component (float positions in [0, L]).
 __device__ __forceinline__ float min_image_f(float d, float L, float halfL) {
   return fabsf(d) > halfL ? d - copysignf(L, d) : d;
@@ -234,13 +239,13 @@ __device__ __forceinline__ float min_image_f(float d, float L, float halfL) {
 // inner loop is almost branch-free and the skin loop mostly skips the force.
 template <bool HALF>
 __global__ void __launch_bounds__(MD_BLOCK)
-    k_build(const double4_32a* __restrict__ x4, const XSplit* __restrict__ xs,
+    k_build(const double4_32a* __restrict__ x4, const XSplit* __restrict__ xs, int hs,
             const int32_t* __restrict__ cell, const int32_t* __restrict__ start, int64_t n,
             Geo gg, const RepGeo* __restrict__ rep, int32_t* __restrict__ numneigh,
             int32_t* __restrict__ nbr, int maxneigh, unsigned int* __restrict__ maxcount) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const float4 hi = xs[i].hi;
+  const float4 hi = ld_hi(xs, i, hs);
   const int tag = __float_as_int(hi.w);
   const int ti = MD_TAG_TYPE(tag);
   const RepGeo& g = rep[MD_TAG_REP(tag)];  // fields read on use (fewer registers)
@@ -292,7 +297,7 @@ __global__ void __launch_bounds__(MD_BLOCK)
     // (md_owns), so each run is walked with stride 2 on the owned parity.
     auto run = [&](int b, int e, float sx, float sy, float sz) {
       auto visit = [&](int j) {
-        const float4 hj = __ldg(&xs[j].hi);
+        const float4 hj = ld_hi(xs, j, hs);
         consider(j, __fadd_rn(__fsub_rn(hj.x, hi.x), sx), __fadd_rn(__fsub_rn(hj.y, hi.y), sy),
                  __fadd_rn(__fsub_rn(hj.z, hi.z), sz), hj.w);
       };
@@ -363,7 +368,7 @@ __global__ void __launch_bounds__(MD_BLOCK)
           for (int j = b; j < e; j++) {
             if (j == ii) continue;
             if (HALF && !md_owns(ii, j)) continue;
-            const float4 hj = __ldg(&xs[j].hi);
+            const float4 hj = ld_hi(xs, j, hs);
             consider(j, min_image_f(hj.x - hi.x, g.Lf[0], g.halfLf[0]),
                      min_image_f(hj.y - hi.y, g.Lf[1], g.halfLf[1]),
                      min_image_f(hj.z - hi.z, g.Lf[2], g.halfLf[2]), hj.w);
@@ -401,7 +406,7 @@ constexpr int BC_OWN = 0;             // the own cell comes first among the 27
 
 template <bool HALF, bool SINGLE>
 __global__ void __launch_bounds__(MD_BLOCK)
-    k_build_cell(const double4_32a* __restrict__ x4, const XSplit* __restrict__ xs,
+    k_build_cell(const double4_32a* __restrict__ x4, const XSplit* __restrict__ xs, int hs,
                  const int32_t* __restrict__ start, int64_t n, const Geo gg,
                  const RepGeo* __restrict__ rep, int32_t* __restrict__ numneigh,
                  int32_t* __restrict__ nbr, int maxneigh, unsigned int* __restrict__ maxcount) {
@@ -419,7 +424,7 @@ __global__ void __launch_bounds__(MD_BLOCK)
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int ob = start[blockIdx.x], oe = start[blockIdx.x + 1];
   if (ob + (int)blockIdx.y * 32 >= oe) return;
-  const RepGeo& g = rep[MD_TAG_REP(__float_as_int(xs[ob].hi.w))];
+  const RepGeo& g = rep[MD_TAG_REP(__float_as_int(ld_hi(xs, ob, hs).w))];
   const bool img = g.nc[0] < 3 || g.nc[1] < 3 || g.nc[2] < 3;  // minimum image per pair
   if (threadIdx.x < gg.nt * gg.nt) scut[threadIdx.x] = gg.cutsqf[threadIdx.x];
   const float cut1 = gg.cutsqf[0];
@@ -484,14 +489,14 @@ __global__ void __launch_bounds__(MD_BLOCK)
     const int i = i0 + lane;
     int32_t* out = nbr + (int64_t)(i >> 5) * maxneigh * 32 + (i & 31);
     __syncthreads();
-    if (threadIdx.x < na) own[threadIdx.x] = xs[i0 + threadIdx.x].hi;
+    if (threadIdx.x < na) own[threadIdx.x] = ld_hi(xs, i0 + (int)threadIdx.x, hs);
     for (int p0 = 0; p0 < len; p0 += LCAP) {
       // stage the candidates of slots p0 .. p0 + LCAP - 1 of each list
       for (int c = w; c < 27; c += BC_WARPS) {
         const int b = s_b[c], e = s_e[c];
         const float s0 = s_sh[c][0], s1 = s_sh[c][1], s2 = s_sh[c][2];
         for (int j = b + lane; j < e; j += 32) {
-          float4 h = __ldg(&xs[j].hi);
+          float4 h = ld_hi(xs, j, hs);
           h.x += s0;
           h.y += s1;
           h.z += s2;
@@ -733,6 +738,7 @@ void md_drop_graphs(md_ctx* c) {
 static int launch_build(md_ctx* c) {
   unsigned nb = (unsigned)md_blocks(c->n);
   const bool half = c->list_kind == MD_LIST_HALF;
+  const int hs = c->xq ? 0 : 1;
   // sparse boxes (mostly empty cells) keep one thread per atom: a block per cell
   // would launch mostly empty blocks
   if (c->ncell <= c->n) {
@@ -744,14 +750,14 @@ static int launch_build(md_ctx* c) {
     const dim3 grid((unsigned)c->ncell, (unsigned)(gy < 64 ? gy : 64));
     auto kern = half ? (c->nt == 1 ? k_build_cell<true, true> : k_build_cell<true, false>)
                      : (c->nt == 1 ? k_build_cell<false, true> : k_build_cell<false, false>);
-    kern<<<grid, MD_BLOCK, 0, c->stream>>>(c->x4, c->xs, c->start, c->n, c->geo, c->rep,
+    kern<<<grid, MD_BLOCK, 0, c->stream>>>(c->x4, c->xs, hs, c->start, c->n, c->geo, c->rep,
                                            c->numneigh, c->nbr, c->maxneigh, c->dmax + 1);
   } else if (half) {
-    k_build<true><<<nb, MD_BLOCK, 0, c->stream>>>(c->x4, c->xs, c->cell, c->start, c->n,
+    k_build<true><<<nb, MD_BLOCK, 0, c->stream>>>(c->x4, c->xs, hs, c->cell, c->start, c->n,
                                                   c->geo, c->rep, c->numneigh, c->nbr,
                                                   c->maxneigh, c->dmax + 1);
   } else {
-    k_build<false><<<nb, MD_BLOCK, 0, c->stream>>>(c->x4, c->xs, c->cell, c->start, c->n,
+    k_build<false><<<nb, MD_BLOCK, 0, c->stream>>>(c->x4, c->xs, hs, c->cell, c->start, c->n,
                                                    c->geo, c->rep, c->numneigh, c->nbr,
                                                    c->maxneigh, c->dmax + 1);
   }

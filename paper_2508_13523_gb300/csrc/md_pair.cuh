@@ -73,6 +73,7 @@ struct PairArgs {
                          // NULL: one tile per block
   int nslots;            // counters (= SMs)
   DispStop stop;
+  int* fmark;            // set where a contribution goes to f, or NULL
   int64_t n;
   int nt;
   int maxneigh;
@@ -349,6 +350,7 @@ __global__ void __launch_bounds__(MD_BLOCK, md_pair_minb(PREC, HALF, EV)) k_pair
             az -= qz;
             if (HALF) atomicAdd(a.fix + 2 * n + j, (unsigned long long)qz);
           } else {  // beyond the fixed-point range (rare): FP64 reductions into f
+            if (a.fmark) *(volatile int*)a.fmark = 1;
             atomicAdd(a.f + ia, -(double)gx);
             atomicAdd(a.f + n + ia, -(double)gy);
             atomicAdd(a.f + 2 * n + ia, -(double)gz);

@@ -89,6 +89,7 @@ __device__ __noinline__ void md_pair_fx_slow(const PairArgs& a, const PairCoef* 
   const double gx = fpair * dx, gy = fpair * dy, gz = fpair * dz;
   if (!(md_fix(gx, ex_lim, o.q[0]) & md_fix(gy, ex_lim, o.q[1]) & md_fix(gz, ex_lim, o.q[2]))) {
     o.q[0] = o.q[1] = o.q[2] = 0;
+    if (a.fmark) *(volatile int*)a.fmark = 1;
     atomicAdd(a.f + i, md_neg(gx));
     atomicAdd(a.f + n + i, md_neg(gy));
     atomicAdd(a.f + 2 * n + i, md_neg(gz));
@@ -311,7 +312,7 @@ __device__ __forceinline__ void md_pair_fx_tiles(const PairArgs& a, const float 
     do {
       int nsv = 0;
       {
-        const float4 hi = __ldg(&a.xs[ia].hi);
+        const float4 hi = md_ld_hi<0>(a.xs, ia);
         const float Lf0 = g->Lf[0], Lf1 = g->Lf[1], Lf2 = g->Lf[2];
         const float hf0 = g->halfLf[0], hf1 = g->halfLf[1], hf2 = g->halfLf[2];
         auto test = [&](int j, const float4& hj) {
@@ -330,14 +331,14 @@ __device__ __forceinline__ void md_pair_fx_tiles(const PairArgs& a, const float 
         if (U == 2) {
           for (; q + T < nsk && nsv <= MD_FX_SLOTS - 2; q += 2 * T, ps -= 2 * T * 32) {
             const int j0 = __ldcs(ps), j1 = __ldcs(ps - T * 32);
-            const float4 h0 = __ldg(&a.xs[j0].hi), h1 = __ldg(&a.xs[j1].hi);
+            const float4 h0 = md_ld_hi<0>(a.xs, j0), h1 = md_ld_hi<0>(a.xs, j1);
             test(j0, h0);
             test(j1, h1);
           }
         }
         for (; q < nsk && (U == 1 || q + T >= nsk) && nsv < MD_FX_SLOTS; q += T, ps -= T * 32) {
           const int j = __ldcs(ps);
-          test(j, __ldg(&a.xs[j].hi));
+          test(j, md_ld_hi<0>(a.xs, j));
         }
       }
       const int own_in = left, tot = left + nsv;

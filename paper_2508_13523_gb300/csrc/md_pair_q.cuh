@@ -85,7 +85,7 @@ __device__ __forceinline__ void md_pair_q_tiles(const PairArgs& a, const float c
     const int ti = MD_TAG_TYPE(tag_i);
     const RepGeo* g = a.rep + MD_TAG_REP(tag_i);
     // FP32 view of the own position (phase 1)
-    const float4 hi = __ldg(&a.xs[ia].hi);
+    const float4 hi = md_ld_hi<0>(a.xs, ia);
     const float Lf0 = g->Lf[0], Lf1 = g->Lf[1], Lf2 = g->Lf[2];
     const float hf0 = g->halfLf[0], hf1 = g->halfLf[1], hf2 = g->halfLf[2];
     // routing bound (1 - 2^-12) L/2: the FP32 separation of the hi parts is
@@ -238,7 +238,7 @@ __device__ __forceinline__ void md_pair_q_tiles(const PairArgs& a, const float c
       int j = 0;
       if (q < cnt) {
         j = __ldcs(q < nin ? row + (int64_t)q * 32 : skin - (int64_t)(q - nin) * 32);
-        const float4 hj = __ldg(&a.xs[j].hi);
+        const float4 hj = md_ld_hi<0>(a.xs, j);
         float dx = hj.x - hi.x, dy = hj.y - hi.y, dz = hj.z - hi.z;
         wrap = (fabsf(dx) > hm0) | (fabsf(dy) > hm1) | (fabsf(dz) > hm2);
         dx = fabsf(dx) > hf0 ? dx - copysignf(Lf0, dx) : dx;

@@ -101,14 +101,14 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
   // code runs for lanes that almost all have a pair in range.
   __shared__ int sslot[MD_VJP_SLOTS][MD_BLOCK];
   auto walk = [&](const RepGeo* g, int type, auto take) {
-    const float4 hi = __ldg(&a.xs[ia].hi);
+    const float4 hi = md_ld_hi<MIX ? 1 : 0>(a.xs, ia);
     const float hf0 = g->halfLf[0], hf1 = g->halfLf[1], hf2 = g->halfLf[2];
     int left = nin, q = t;
     do {
       int nsv = 0;
       for (; q < nsk && nsv < MD_VJP_SLOTS; q += TPA) {
         const int j = __ldcs(skin - (int64_t)q * 32);
-        const float4 hj = __ldg(&a.xs[j].hi);
+        const float4 hj = md_ld_hi<MIX ? 1 : 0>(a.xs, j);
         float dx = hj.x - hi.x, dy = hj.y - hi.y, dz = hj.z - hi.z;
         dx = fabsf(dx) > hf0 ? dx - copysignf(g->Lf[0], dx) : dx;
         dy = fabsf(dy) > hf1 ? dy - copysignf(g->Lf[1], dy) : dy;
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
     // listed pair move continuously, unwrapped): its rows need no minimum
     // image.  The test is warp-uniform so that the other warps keep the
     // image code (which the compiler makes unconditional) off their pairs.
-    const float4 bh = __ldg(&a.xb[ia].hi);
+    const float4 bh = md_ld_hi<0>(a.xb, ia);
     const float r0 = a.rin + g->Lf[0] * 0x1p-20f, r1 = a.rin + g->Lf[1] * 0x1p-20f,
                 r2b = a.rin + g->Lf[2] * 0x1p-20f;
     const bool inner_atom = bh.x >= r0 && bh.x <= g->Lf[0] - r0 && bh.y >= r1 &&
