@@ -230,9 +230,23 @@ __device__ __forceinline__ float md_split_hi(double x, const XGrid& g) {
       eh == 0 ? 0u : ((unsigned int)(eh - 1023 + 127) << 23) | (unsigned int)((h >> 29) & 0x7fffff);
   return __uint_as_float((unsigned int)((unsigned long long)sign >> 32) | fb);
 }
+// lo without FP64 operations where hi's rounding dropped 29 .. 52 bits of x's
+// significand: x - hi is then the difference of the two bit patterns in units
+// of x's last place (also across a carry into the exponent), and its
+// conversion to FP32 rounds like that of the double.
 __device__ __forceinline__ void md_split(double x, const XGrid& g, float& hi, float& lo) {
   hi = md_split_hi(x, g);
-  lo = __double2float_rn(__dsub_rn(x, md_widen(hi)));
+  const long long b = __double_as_longlong(x);
+  const int e = (int)((b >> 52) & 0x7ff), d = g.k + 1075 - e;
+  // d >= 29: |x| < 2^24 2^k, so hi is the rounded value itself; e > 1000: the
+  // scale 2^(e - 1075) is a normal FP32 value
+  if (d >= 29 && d <= 52 && e > 1000) {
+    const long long m = b & 0x7fffffffffffffffLL, r = 1LL << (d - 1);
+    const long long l = m - ((m + r) & ~((r << 1) - 1));
+    lo = __fmul_rn(__ll2float_rn(b < 0 ? -l : l), __int_as_float((e - 1075 + 127) << 23));
+  } else {
+    lo = __double2float_rn(__dsub_rn(x, md_widen(hi)));
+  }
 }
 
 // x as a fixed-point count X = x 2^F, |x| < 2^(61 - F) (so |X| < 2^61); false
