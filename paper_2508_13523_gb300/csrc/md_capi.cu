@@ -872,10 +872,12 @@ double md_ev_trace_share(const md_ctx* c) {
              : 0.0;
 }
 
+int launch_pair_impl(md_ctx* c, int ev, int tpa, int prezeroed, int defer_fold,
+                     const DispStop* stop = nullptr, int mark = -1);
+
 // Pair energies/virials and kinetic energies per replica into ev_host.
 int thermo_per_replica(md_ctx* c) {
-  MD_TRY(md_launch_pair(c, 1, c->tpa));
-  MD_TRY(md_launch_kinetic(c));
+  MD_TRY(launch_pair_impl(c, 2, c->tpa, 0, 0));
   MD_CUDA(cudaMemcpyAsync(c->ev_host, c->ev, sizeof(double) * (size_t)c->nrep * MD_EV_STRIDE,
                           cudaMemcpyDeviceToHost, c->stream));
   MD_CUDA(cudaStreamSynchronize(c->stream));
@@ -914,10 +916,11 @@ int md_pair_fixed(const md_ctx* c) {
 
 namespace {
 
-// ev: energy and virial too; the virial's sum over atoms needs the final
-// forces, so it is only asked for with the fold in this call.
+// ev: 1 energy and virial too, 2 also the kinetic energy; the virial's sum over
+// atoms needs the final forces, so it is only asked for with the fold in this
+// call.
 int launch_pair_impl(md_ctx* c, int ev, int tpa, int prezeroed, int defer_fold,
-                     const DispStop* stop = nullptr, int mark = -1) {
+                     const DispStop* stop, int mark) {
   if (ev && defer_fold) return MD_EINVAL;
   PairArgs a = pair_args(c);
   if (stop) a.stop = *stop;
@@ -926,9 +929,6 @@ int launch_pair_impl(md_ctx* c, int ev, int tpa, int prezeroed, int defer_fold,
   if (c->persist)
     MD_CUDA(cudaMemsetAsync(c->tile_ctr, 0, sizeof(int) * c->nsm, c->stream));
   const unsigned blocks = (unsigned)md_blocks(c->n * (int64_t)tpa);
-  if (ev)
-    MD_CUDA(cudaMemsetAsync(c->ev, 0, sizeof(double) * (size_t)c->nrep * MD_EV_STRIDE,
-                            c->stream));
   const bool half = c->list_kind == MD_LIST_HALF;
   const bool compact = c->compact && c->precision == MD_PREC_FP64;
   if (md_pair_accumulates(c) && !prezeroed)  // sums by atomics start from zero
@@ -950,10 +950,8 @@ int launch_pair_impl(md_ctx* c, int ev, int tpa, int prezeroed, int defer_fold,
                    : md_pair_q_launch(a, half, ev != 0, single, cut1, cut, qb, s, c->carve));
     c->launches++;
     MD_CUDA(e);
-    if (fix && !defer_fold) MD_TRY(md_launch_fix_finalize(c));
-    if (ev) MD_TRY(md_launch_virial_atoms(c));
-    if (ev) MD_TRY(md_launch_ev_fold(c));
-    return MD_OK;
+    if (ev) return md_launch_ev_atoms(c, fix, ev == 2);
+    return fix && !defer_fold ? md_launch_fix_finalize(c) : MD_OK;
   }
   if (c->coul && c->precision == MD_PREC_FP64) return MD_EINVAL;  // FP64 Coulomb: k_pair_q
   cudaError_t e =
@@ -965,10 +963,8 @@ int launch_pair_impl(md_ctx* c, int ev, int tpa, int prezeroed, int defer_fold,
           : md_pair_launch_mixed(a, half, ev != 0, c->nt == 1, tpa, blocks, c->stream, c->carve);
   c->launches++;
   MD_CUDA(e);
-  if (md_pair_fixed(c) && !defer_fold) MD_TRY(md_launch_fix_finalize(c));
-  if (ev) MD_TRY(md_launch_virial_atoms(c));
-  if (ev) MD_TRY(md_launch_ev_fold(c));
-  return MD_OK;
+  if (ev) return md_launch_ev_atoms(c, md_pair_fixed(c), ev == 2);
+  return md_pair_fixed(c) && !defer_fold ? md_launch_fix_finalize(c) : MD_OK;
 }
 
 }  // namespace

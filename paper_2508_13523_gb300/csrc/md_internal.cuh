@@ -339,9 +339,10 @@ enum { MD_K1 = 0, MD_K21 = 1, MD_K2 = 2 };
 int md_launch_integrate(md_ctx* c, int mode, int fold = 0, int zero = 0,
                         const DispStop* stop = nullptr, unsigned int* disp_out = nullptr,
                         int mark = -1);
-int md_launch_kinetic(md_ctx* c);
-int md_launch_virial_atoms(md_ctx* c);  // sum_a (x_a - c) (x) F_a into evs words 1..6
-int md_launch_ev_fold(md_ctx* c);       // ev += the sums of the evs rows; evs = 0
+// after a pair launch with energy and virial: the sums folded into f (fold),
+// sum_a (x_a - c) (x) F_a and, if asked for, the kinetic energy; ev receives
+// the sums of the evs rows, which are left at zero
+int md_launch_ev_atoms(md_ctx* c, int fold, int kinetic);
 int md_launch_load_state(md_ctx* c, const double* x, const double* v);
 int md_launch_store_state(md_ctx* c, double* x, double* v, double* f);
 // caller order into the current sorted order, list kept; max displacement

@@ -12,7 +12,7 @@
 // shared-memory table).  With energy and virial the pair loop adds only the
 // energy, a pair count and, for pairs taken through a periodic image, the
 // virial's image terms; the rest of the virial is summed over atoms from the
-// final forces (k_virial_atoms), which costs one pass over x and f instead
+// final forces (k_ev_atoms), which costs one pass over x and f instead
 // of six FMAs per pair.
 //
 // FP64 form: separations, r^2, the cutoff test and all force arithmetic in
