@@ -442,6 +442,47 @@ __device__ __forceinline__ void md_warp_add_rep(double (&v)[NV], int rep, double
   }
 }
 
+// The pair kernels' energy and virial sums of a warp, weighted by evw, into row
+// `slot` of the lanes' replicas (as md_warp_add_rep): word 0 the energies, word
+// 7 the pair counts, words 1..6 the image terms m[k * MD_BLOCK] of the lanes
+// that have any (img, rare), which are cleared.  Only the energy costs FP64
+// additions in the common case (an FP64 instruction takes 64 cycles of its
+// pipe: eight sums through the shuffles took a third of an energy/virial
+// launch).  All 32 lanes must call it; lanes with rep < 0 contribute nothing.
+__device__ __forceinline__ void md_warp_add_ev(double e, int npair, bool img, double* m,
+                                               double evw, int rep, double* acc, int spread,
+                                               int slot) {
+  const int r0 = __shfl_sync(0xffffffffu, rep, 0);
+  const bool any_img = __any_sync(0xffffffffu, img);
+  if (__all_sync(0xffffffffu, rep == r0 || rep < 0)) {
+    const bool lead = (threadIdx.x & 31) == 0 && r0 >= 0;
+    double* row = acc + ((int64_t)r0 * spread + slot) * MD_EV_STRIDE;
+    const int np = __reduce_add_sync(0xffffffffu, npair);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) e += __shfl_xor_sync(0xffffffffu, e, off);
+    if (lead) {
+      atomicAdd(row, evw * e);
+      atomicAdd(row + 7, evw * (double)np);
+    }
+    if (any_img) {
+      for (int k = 0; k < 6; k++) {
+        double v = img ? m[k * MD_BLOCK] : 0.0;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+        if (lead) atomicAdd(row + 1 + k, evw * v);
+      }
+    }
+  } else if (rep >= 0) {
+    double* row = acc + ((int64_t)rep * spread + slot) * MD_EV_STRIDE;
+    atomicAdd(row, evw * e);
+    atomicAdd(row + 7, evw * (double)npair);
+    if (img)
+      for (int k = 0; k < 6; k++) atomicAdd(row + 1 + k, evw * m[k * MD_BLOCK]);
+  }
+  if (img)
+    for (int k = 0; k < 6; k++) m[k * MD_BLOCK] = 0.0;
+}
+
 // Block-wide sum of NV doubles into out[0..NV) of block's slot; all threads
 // of the block must call it.  blockDim.x == MD_BLOCK.
 template <int NV>

@@ -324,9 +324,13 @@ int md_launch_fix_finalize(md_ctx* c) {
 int md_launch_ev_atoms(md_ctx* c, int fold, int kinetic) {
   MassArgs ma;
   for (int t = 0; t < MD_MAX_TYPES; t++) ma.m[t] = c->mass[t];
-  // 16 blocks per SM, each a contiguous run of whole blocks' worth of atoms
-  const int64_t cap = 16 * (int64_t)(c->nsm > 0 ? c->nsm : 1);
-  const int64_t nb = md_blocks(c->n) < cap ? md_blocks(c->n) : cap;
+  // 4 to 16 blocks per SM, each a contiguous run of whole blocks' worth of
+  // atoms: 8 of them where there are enough, so that the sums' reductions (40
+  // FP64 additions a warp) do not outweigh the atoms
+  const int64_t sm = c->nsm > 0 ? c->nsm : 1, all = md_blocks(c->n);
+  int64_t nb = all / 8;
+  nb = nb < 4 * sm ? 4 * sm : nb > 16 * sm ? 16 * sm : nb;
+  if (nb > all) nb = all;
   const int64_t per = (md_blocks(c->n) + nb - 1) / nb;
   const int64_t blocks = (md_blocks(c->n) + per - 1) / per;
   k_ev_atoms<<<(unsigned)blocks, MD_BLOCK, 0, c->stream>>>(

@@ -170,6 +170,7 @@ __global__ void __launch_bounds__(MD_BLOCK, md_pair_minb(PREC, HALF, EV)) k_pair
     double fx = 0.0, fy = 0.0, fz = 0.0;
     double e0 = 0.0;  // energy (FP64, several types)
     int npair = 0;    // pairs within rc
+    bool img = false;  // this thread has image terms
     // the energy's partial sums: FP64, one type -- sum r^-6 alone, the
     // energy being trace(W) / 12 - (lj4 / 2) sum r^-6 (lj1 = 12 lj3, lj2 =
     // 6 lj4: a pair's energy is fpair r^2 / 12 - (lj4 / 2) r^-6), with the
@@ -234,6 +235,7 @@ __global__ void __launch_bounds__(MD_BLOCK, md_pair_minb(PREC, HALF, EV)) k_pair
             }
             npair++;
             if ((shx != 0.0) | (shy != 0.0) | (shz != 0.0)) {
+              img = true;
               const double gx = fpair * dx, gy = fpair * dy, gz = fpair * dz;
               double* m = &simg[0][threadIdx.x];
               m[0 * MD_BLOCK] = __fma_rn(-shx, gx, m[0 * MD_BLOCK]);
@@ -373,6 +375,7 @@ __global__ void __launch_bounds__(MD_BLOCK, md_pair_minb(PREC, HALF, EV)) k_pair
             }
             npair++;
             if (shf) {  // rare
+              img = true;
               auto sh = [&](int k) {
                 const int b = (shf >> (2 * k)) & 3;
                 return b == 1 ? g->L[k] : (b == 2 ? -g->L[k] : 0.0);
@@ -472,21 +475,12 @@ __global__ void __launch_bounds__(MD_BLOCK, md_pair_minb(PREC, HALF, EV)) k_pair
         a.f[2 * n + i] = fz;
       }
     }
-    if (EV) {
-      double ev[8];
-      ev[0] = PREC == MD_PREC_MIXED ? md_widen(es) + md_widen(ec)
-                                    : (SINGLE ? -0.5 * a.c1.lj4 * s6 : e0);
-  #pragma unroll
-      for (int k = 1; k < 7; k++) {
-        ev[k] = simg[k - 1][threadIdx.x];
-        simg[k - 1][threadIdx.x] = 0.0;
-      }
-  #pragma unroll
-      for (int k = 0; k < 7; k++) ev[k] *= evw;
-      ev[7] = evw * (double)npair;
-      md_warp_add_rep<8>(ev, active ? rep_i : -1, a.ev, a.ev_spread,
-                         (int)(((int64_t)blockIdx.x * MD_BLOCK + threadIdx.x) >> 5) % a.ev_spread);
-    }
+    if (EV)
+      md_warp_add_ev(PREC == MD_PREC_MIXED ? md_widen(es) + md_widen(ec)
+                                           : (SINGLE ? -0.5 * a.c1.lj4 * s6 : e0),
+                     npair, img, &simg[0][threadIdx.x], evw, active ? rep_i : -1, a.ev,
+                     a.ev_spread,
+                     (int)(((int64_t)blockIdx.x * MD_BLOCK + threadIdx.x) >> 5) % a.ev_spread);
   }
 }
 

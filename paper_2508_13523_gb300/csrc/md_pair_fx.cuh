@@ -171,6 +171,7 @@ __device__ __forceinline__ void md_pair_fx_tiles(const PairArgs& a, const float 
     unsigned long long s6 = 0;         // one type: sum x^3 2^(62 - ev_shift)
     double e0 = 0.0;                   // several types: energy; one type: r^-6 of FP64 pairs
     int npair = 0;
+    bool img = false;  // this thread has image terms
     auto slow = [&](int j) {
       FxSlow o;
       md_pair_fx_slow<HALF, EV, SINGLE, COUL>(a, SINGLE ? &a.c1 : sc, ia, j, o);
@@ -186,6 +187,7 @@ __device__ __forceinline__ void md_pair_fx_tiles(const PairArgs& a, const float 
         if (EV) {
           e0 += o.e;
           npair++;
+          img = true;
           double* m = &simg[0][threadIdx.x];
           m[0 * MD_BLOCK] = __fma_rn(-o.s[0], o.g[0], m[0 * MD_BLOCK]);
           m[1 * MD_BLOCK] = __fma_rn(-o.s[1], o.g[1], m[1 * MD_BLOCK]);
@@ -289,6 +291,7 @@ __device__ __forceinline__ void md_pair_fx_tiles(const PairArgs& a, const float 
                 __ull2double_rn(rho) *
                 __longlong_as_double((long long)(1023 - 60 + k - a.fxR) << 52);
         if (shf) {  // rare
+          img = true;
           auto shift = [&](int k3) {
             const int b = (shf >> (2 * k3)) & 3;
             return b == 1 ? g->L[k3] : (b == 2 ? -g->L[k3] : 0.0);
@@ -376,26 +379,19 @@ __device__ __forceinline__ void md_pair_fx_tiles(const PairArgs& a, const float 
     }
     if (EV) {
       const double evw = HALF ? 1.0 : 0.5;  // a full list visits each pair twice
-      double ev[8];
       // one type: -(lj4 / 2) sum r^-6, the rest of the energy is trace(W) / 12
       // (r^-6 = x^3 2^(3 B - 6 R))
-      ev[0] = SINGLE ? -0.5 * a.c1.lj4 *
-                           __fma_rn(__ull2double_rn(s6),
-                                    __longlong_as_double((long long)(1023 - 62 + a.ev_shift +
-                                                                     3 * a.fx1.B - 6 * a.fxR)
-                                                         << 52),
-                                    e0)
-                     : e0;
-#pragma unroll
-      for (int c = 1; c < 7; c++) {
-        ev[c] = simg[c - 1][threadIdx.x];
-        simg[c - 1][threadIdx.x] = 0.0;
-      }
-#pragma unroll
-      for (int c = 0; c < 7; c++) ev[c] *= evw;
-      ev[7] = evw * (double)npair;
-      md_warp_add_rep<8>(ev, active ? MD_TAG_REP(tag) : -1, a.ev, a.ev_spread,
-                         (int)(gid >> 5) % a.ev_spread);
+      const double e = SINGLE ? -0.5 * a.c1.lj4 *
+                                    __fma_rn(__ull2double_rn(s6),
+                                             __longlong_as_double(
+                                                 (long long)(1023 - 62 + a.ev_shift +
+                                                             3 * a.fx1.B - 6 * a.fxR)
+                                                 << 52),
+                                             e0)
+                              : e0;
+      md_warp_add_ev(e, npair, img, &simg[0][threadIdx.x], evw,
+                     active ? MD_TAG_REP(tag) : -1, a.ev, a.ev_spread,
+                     (int)(gid >> 5) % a.ev_spread);
     }
   }
 }
