@@ -28,33 +28,36 @@ int md_cuda_fail(cudaError_t e) {
   return e == cudaErrorMemoryAllocation ? MD_ENOMEM : MD_ECUDA;
 }
 
-cudaError_t md_prepare_kernel(const void* kernel, int carve, int* occ) {
-  // (kernel, device) -> (carveout applied, -1 none; resident blocks per SM)
+cudaError_t md_prepare_kernel(const void* kernel, int carve, size_t smem, int* occ) {
+  struct State {
+    int carve = -1;   // carveout applied, -1 none
+    int occ = 0;      // resident blocks per SM, 0: not known
+    size_t smem = 0;  // with that much dynamic shared memory
+  };
   static std::mutex mu;
-  static std::map<std::pair<const void*, int>, std::pair<int, int>> cache;
+  static std::map<std::pair<const void*, int>, State> cache;  // by (kernel, device)
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   std::lock_guard<std::mutex> lock(mu);
-  auto it = cache.find({kernel, dev});
-  if (it == cache.end()) it = cache.emplace(std::make_pair(kernel, dev), std::make_pair(-1, 0)).first;
-  std::pair<int, int>& st = it->second;
-  if (carve >= 0 && carve != st.first) {
+  State& st = cache[{kernel, dev}];
+  if (carve >= 0 && carve != st.carve) {
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, carve);
     if (e != cudaSuccess) return e;
-    st.first = carve;
-    st.second = 0;
+    st.carve = carve;
+    st.occ = 0;
   }
-  if (st.second == 0) {
+  if (st.occ == 0 || st.smem != smem) {
     int o = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kernel, MD_BLOCK, 0);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kernel, MD_BLOCK, smem);
     if (e != cudaSuccess) {
       cudaGetLastError();
       o = 1;
     }
-    st.second = o < 1 ? 1 : o;
+    st.occ = o < 1 ? 1 : o;
+    st.smem = smem;
   }
-  *occ = st.second;
+  *occ = st.occ;
   return cudaSuccess;
 }
 

@@ -51,6 +51,10 @@ struct PairCoef {
   int64_t cutmax_bits;      // the larger of the two: a pair has a force below it
 };
 
+// Entries of a shared table of nt * nt type pairs: room for any type below
+// MD_MAX_TYPES, also one that the parameters do not have.
+__host__ __device__ inline int md_tab_entries(int nt) { return (MD_MAX_TYPES - 1) * nt + MD_MAX_TYPES; }
+
 struct RepGeo;
 
 // Grid of the hi parts of split positions (md_split): step 2^k, with every

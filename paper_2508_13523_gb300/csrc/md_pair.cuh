@@ -128,13 +128,23 @@ constexpr int md_pair_minb(int prec, bool half, bool ev) {
                                : (ev ? 6 : 8);
 }
 
+// Dynamic shared memory of k_pair: the coefficient table of the types that
+// there are.  What a block does not take stays L1, which the gathers live on
+// (7.7 KB a block for MD_MAX_TYPES against 2.6 KB: 64,000 atoms of two types,
+// mixed half list 40.5 -> 40.0 us; the fixed-point kernel, which kept 14.6 KB
+// of tables, 297 -> 293 us for 500,000 charged atoms).
+inline size_t md_pair_smem(bool single, int nt) {
+  return single ? 0 : sizeof(PairCoef) * (size_t)md_tab_entries(nt);
+}
+
 // COUL (mixed precision only): the lj/cut/coul/cut style, Eq. 1 plus the
 // cut Coulomb term qq / r.
 template <int PREC, bool HALF, int TPA, bool EV, bool SINGLE, bool COUL = false>
 __global__ void __launch_bounds__(MD_BLOCK, md_pair_minb(PREC, HALF, EV)) k_pair(const PairArgs a) {
   static_assert(!COUL || PREC == MD_PREC_MIXED, "the FP64 Coulomb form is k_pair_q");
   if (md_stopped(a.stop)) return;
-  __shared__ PairCoef sc[SINGLE ? 1 : MD_MAX_TYPES * MD_MAX_TYPES];
+  extern __shared__ double s_tab[];  // md_pair_smem
+  PairCoef* sc = reinterpret_cast<PairCoef*>(s_tab);
   if (!SINGLE) {
     for (int k = threadIdx.x; k < a.nt * a.nt; k += blockDim.x) sc[k] = a.coef[k];
     __syncthreads();
@@ -487,37 +497,39 @@ __global__ void __launch_bounds__(MD_BLOCK, md_pair_minb(PREC, HALF, EV)) k_pair
 // Applies the preferred shared-memory carveout (percent; -1 leaves the
 // driver default) to a kernel on the current device, once per (kernel,
 // device, carveout), and returns in *occ its resident blocks per SM of
-// MD_BLOCK threads at that carveout.  Thread safe (md_capi.cu).
-cudaError_t md_prepare_kernel(const void* kernel, int carve, int* occ);
+// MD_BLOCK threads and smem bytes of dynamic shared memory at that carveout.
+// Thread safe (md_capi.cu).
+cudaError_t md_prepare_kernel(const void* kernel, int carve, size_t smem, int* occ);
 
 // Launch one instantiation; carve is the preferred shared-memory carveout in
 // percent (0: largest L1, the LJ kernel's cache -- Sec. 4.4 -- uses almost no
 // shared memory).  Returns cudaGetLastError().
 template <typename K>
 cudaError_t md_launch_carved(K kernel, const PairArgs& a, unsigned blocks, cudaStream_t s,
-                             int carve) {
+                             int carve, size_t smem) {
   int occ = 1;
-  cudaError_t e = md_prepare_kernel((const void*)kernel, carve, &occ);
+  cudaError_t e = md_prepare_kernel((const void*)kernel, carve, smem, &occ);
   if (e != cudaSuccess) return e;
   // persistent: as many blocks as can be resident at once
   if (a.tile_ctr) {
     const unsigned cap = (unsigned)(a.nslots * occ);
     if (blocks > cap) blocks = cap;
   }
-  kernel<<<blocks, MD_BLOCK, 0, s>>>(a);
+  kernel<<<blocks, MD_BLOCK, smem, s>>>(a);
   return cudaGetLastError();
 }
 
 template <int PREC, bool HALF, bool EV, bool SINGLE>
 cudaError_t md_pair_launch_tpa(const PairArgs& a, int tpa, unsigned blocks, cudaStream_t s,
                                int carve) {
+  const size_t smem = md_pair_smem(SINGLE, a.nt);
   switch (tpa) {
-    case 1: return md_launch_carved(k_pair<PREC, HALF, 1, EV, SINGLE>, a, blocks, s, carve);
-    case 2: return md_launch_carved(k_pair<PREC, HALF, 2, EV, SINGLE>, a, blocks, s, carve);
-    case 4: return md_launch_carved(k_pair<PREC, HALF, 4, EV, SINGLE>, a, blocks, s, carve);
-    case 8: return md_launch_carved(k_pair<PREC, HALF, 8, EV, SINGLE>, a, blocks, s, carve);
-    case 16: return md_launch_carved(k_pair<PREC, HALF, 16, EV, SINGLE>, a, blocks, s, carve);
-    case 32: return md_launch_carved(k_pair<PREC, HALF, 32, EV, SINGLE>, a, blocks, s, carve);
+    case 1: return md_launch_carved(k_pair<PREC, HALF, 1, EV, SINGLE>, a, blocks, s, carve, smem);
+    case 2: return md_launch_carved(k_pair<PREC, HALF, 2, EV, SINGLE>, a, blocks, s, carve, smem);
+    case 4: return md_launch_carved(k_pair<PREC, HALF, 4, EV, SINGLE>, a, blocks, s, carve, smem);
+    case 8: return md_launch_carved(k_pair<PREC, HALF, 8, EV, SINGLE>, a, blocks, s, carve, smem);
+    case 16: return md_launch_carved(k_pair<PREC, HALF, 16, EV, SINGLE>, a, blocks, s, carve, smem);
+    case 32: return md_launch_carved(k_pair<PREC, HALF, 32, EV, SINGLE>, a, blocks, s, carve, smem);
     default: return cudaErrorInvalidValue;
   }
 }

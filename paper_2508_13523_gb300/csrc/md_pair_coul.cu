@@ -28,13 +28,13 @@ static cudaError_t coul_tpa(const PairArgs& a, int tpa, unsigned blocks, cudaStr
   switch (tpa) {
     case 1:
       return md_launch_carved(k_pair<MD_PREC_MIXED, HALF, 1, EV, SINGLE, true>, a, blocks, s,
-                              carve);
+                              carve, md_pair_smem(SINGLE, a.nt));
     case 2:
       return md_launch_carved(k_pair<MD_PREC_MIXED, HALF, 2, EV, SINGLE, true>, a, blocks, s,
-                              carve);
+                              carve, md_pair_smem(SINGLE, a.nt));
     case 4:
       return md_launch_carved(k_pair<MD_PREC_MIXED, HALF, 4, EV, SINGLE, true>, a, blocks, s,
-                              carve);
+                              carve, md_pair_smem(SINGLE, a.nt));
     default: return cudaErrorInvalidValue;
   }
 }

@@ -111,6 +111,13 @@ __device__ __noinline__ void md_pair_fx_slow(const PairArgs& a, const PairCoef* 
   }
 }
 
+// Dynamic shared memory of the kernel: the tables of the types that there are
+// (what FP64 pairs and energies need of PairCoef is read from global memory).
+// What a block does not take stays L1, which the gathers live on.
+inline size_t md_pair_fx_smem(bool single, int nt) {
+  return single ? 0 : (sizeof(PairFx) + sizeof(float)) * (size_t)md_tab_entries(nt);
+}
+
 // The tile loop of the kernel: every block of the launch runs it (k_pair_fx,
 // and the pair phase of k_step_fused).  All threads of the block must call
 // it.  T lanes per atom; U: skin entries per round of the FP32 test, their
@@ -120,15 +127,14 @@ template <bool HALF, bool EV, bool SINGLE, bool COUL, int T, int U>
 __device__ __forceinline__ void md_pair_fx_tiles(const PairArgs& a, const float cut_hi1,
                                                  const float* __restrict__ cut_hi_tab) {
   static_assert(!(SINGLE && COUL), "the Coulomb style takes the general form");
-  __shared__ PairCoef sc[SINGLE ? 1 : MD_MAX_TYPES * MD_MAX_TYPES];
-  __shared__ PairFx sf[SINGLE ? 1 : MD_MAX_TYPES * MD_MAX_TYPES];
-  __shared__ float scut[SINGLE ? 1 : MD_MAX_TYPES * MD_MAX_TYPES];
+  extern __shared__ double s_tab[];  // md_pair_fx_smem
+  PairFx* sf = reinterpret_cast<PairFx*>(s_tab);
+  float* scut = reinterpret_cast<float*>(sf + md_tab_entries(a.nt));
   __shared__ int sslot[MD_FX_SLOTS][MD_BLOCK];
   __shared__ double simg[EV ? 6 : 1][MD_BLOCK];  // the virial's image terms, own column
   __shared__ int s_tile;
   if (!SINGLE) {
     for (int k = threadIdx.x; k < a.nt * a.nt; k += blockDim.x) {
-      sc[k] = a.coef[k];
       sf[k] = a.fxt[k];
       // atoms with very many partners: a smaller range per contribution (fx_dense)
       if (a.fx_dense)
@@ -174,7 +180,7 @@ __device__ __forceinline__ void md_pair_fx_tiles(const PairArgs& a, const float 
     bool img = false;  // this thread has image terms
     auto slow = [&](int j) {
       FxSlow o;
-      md_pair_fx_slow<HALF, EV, SINGLE, COUL>(a, SINGLE ? &a.c1 : sc, ia, j, o);
+      md_pair_fx_slow<HALF, EV, SINGLE, COUL>(a, SINGLE ? &a.c1 : a.coef, ia, j, o);
       if (o.in) {
         ax += o.q[0];
         ay += o.q[1];
@@ -287,7 +293,7 @@ __device__ __forceinline__ void md_pair_fx_tiles(const PairArgs& a, const float 
         else if (!COUL || in_lj)  // 4 eps (tau^6 - tau^3) = 2 eps (w - tau^3)
           e0 += c.e2 * 0x1p-57 * __ll2double_rn(fo.w - (long long)(fo.tau3 >> 2));
         if (COUL && in_co)  // qq / r = qq rho 2^(k - R)
-          e0 += sc[MD_TAG_TYPE(tag) * a.nt + MD_TAG_TYPE((int)o.w)].qq *
+          e0 += a.coef[MD_TAG_TYPE(tag) * a.nt + MD_TAG_TYPE((int)o.w)].qq *
                 __ull2double_rn(rho) *
                 __longlong_as_double((long long)(1023 - 60 + k - a.fxR) << 52);
         if (shf) {  // rare
@@ -415,15 +421,16 @@ template <bool HALF, bool EV, bool SINGLE, bool COUL, int T, int U>
 cudaError_t md_pair_fx_launch1(const PairArgs& a, float cut1, const float* cut_tab,
                                cudaStream_t s, int carve) {
   int occ = 1;
+  const size_t smem = md_pair_fx_smem(SINGLE, a.nt);
   cudaError_t e =
-      md_prepare_kernel((const void*)k_pair_fx<HALF, EV, SINGLE, COUL, T, U>, carve, &occ);
+      md_prepare_kernel((const void*)k_pair_fx<HALF, EV, SINGLE, COUL, T, U>, carve, smem, &occ);
   if (e != cudaSuccess) return e;
   unsigned blocks = (unsigned)md_blocks(a.n * T);
   if (a.tile_ctr) {
     const unsigned cap = (unsigned)(a.nslots * occ);
     if (blocks > cap) blocks = cap;
   }
-  k_pair_fx<HALF, EV, SINGLE, COUL, T, U><<<blocks, MD_BLOCK, 0, s>>>(a, cut1, cut_tab);
+  k_pair_fx<HALF, EV, SINGLE, COUL, T, U><<<blocks, MD_BLOCK, smem, s>>>(a, cut1, cut_tab);
   return cudaGetLastError();
 }
 

@@ -305,7 +305,7 @@ cudaError_t md_pair_q_launch5(const PairArgs& a, float cut1, const float* cut_ta
                               unsigned blocks, cudaStream_t s, int carve) {
   int occ = 1;
   cudaError_t e =
-      md_prepare_kernel((const void*)k_pair_q<HALF, EV, SINGLE, COUL>, carve, &occ);
+      md_prepare_kernel((const void*)k_pair_q<HALF, EV, SINGLE, COUL>, carve, 0, &occ);
   if (e != cudaSuccess) return e;
   if (a.tile_ctr) {
     const unsigned cap = (unsigned)(a.nslots * occ);

@@ -103,12 +103,13 @@ cudaError_t launch_fused(const IntArgs& ia, const PairArgs& a, float cut1, const
                          unsigned int* bar, unsigned int* err, cudaStream_t s) {
   auto kern = k_step_fused<MODE, HALF, SINGLE>;
   int occ = 1;
-  cudaError_t e = md_prepare_kernel((const void*)kern, -1, &occ);
+  const size_t smem = md_pair_fx_smem(SINGLE, a.nt);
+  cudaError_t e = md_prepare_kernel((const void*)kern, -1, smem, &occ);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(a.nslots * occ));
   cfg.blockDim = dim3(MD_BLOCK);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;

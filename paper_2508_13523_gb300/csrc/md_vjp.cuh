@@ -65,21 +65,23 @@ struct VjpArgs {
 
 template <int PREC, bool HALF, int TPA, bool SINGLE>
 __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
-  __shared__ PairCoef sc[SINGLE ? 1 : MD_MAX_TYPES * MD_MAX_TYPES];
-  __shared__ float scut[SINGLE ? 1 : MD_MAX_TYPES * MD_MAX_TYPES];
-  __shared__ VjpCoef sv[SINGLE ? 1 : MD_MAX_TYPES * MD_MAX_TYPES];
-  // parameter terms of each thread by partner type: [tj] eps, [MD_MAX_TYPES + tj]
-  // sigma; thread-private columns (no bank conflicts), reduced at the end
-  // (mixed: FP32 values with their rounding errors, md_acc2)
   constexpr bool MIX = PREC == MD_PREC_MIXED;
-  __shared__ double sg[SINGLE ? 1 : 2 * MD_MAX_TYPES][SINGLE ? 1 : MD_BLOCK];
+  // md_vjp_smem.  sg: parameter terms of each thread by partner type: [tj]
+  // eps, [nt + tj] sigma; thread-private columns (no bank conflicts), reduced
+  // at the end (mixed: FP32 values with their rounding errors, md_acc2).
+  // Types are clamped to those there are, as the columns end with them.
+  extern __shared__ double s_tab[];
+  double* sg = s_tab;
+  PairCoef* sc = reinterpret_cast<PairCoef*>(sg + 2 * a.nt * MD_BLOCK);
+  VjpCoef* sv = reinterpret_cast<VjpCoef*>(sc + a.nt * a.nt);
+  float* scut = reinterpret_cast<float*>(sv + a.nt * a.nt);
   if (!SINGLE) {
     for (int k = threadIdx.x; k < a.nt * a.nt; k += blockDim.x) {
       sc[k] = a.coef[k];
       sv[k] = a.vcoef[k];
       scut[k] = a.cut_tab[k];
     }
-    for (int k = 0; k < 2 * MD_MAX_TYPES; k++) sg[k][threadIdx.x] = 0.0;
+    for (int k = 0; k < 2 * a.nt; k++) sg[k * MD_BLOCK + threadIdx.x] = 0.0;
     __syncthreads();
   }
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -127,7 +129,7 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
 
   double bx = 0.0, by = 0.0, bz = 0.0;  // xbar_i
   double ge0 = 0.0, gs0 = 0.0;          // parameter terms when SINGLE
-  double* slot = SINGLE ? nullptr : &sg[0][threadIdx.x];
+  double* slot = SINGLE ? nullptr : sg + threadIdx.x;
   float2* slot2 = reinterpret_cast<float2*>(slot);
   float geh = 0.f, gel = 0.f, gsh = 0.f, gsl = 0.f;  // mixed: parameter terms when SINGLE
   int ti;
@@ -135,7 +137,7 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
   if (PREC == MD_PREC_FP64) {
     const double4_32a xi = md_ld4(a.x4 + ia);
     const int tag_i = md_tag_of(xi);
-    ti = MD_TAG_TYPE(tag_i);
+    ti = min((int)MD_TAG_TYPE(tag_i), a.nt - 1);
     const RepGeo* g = a.rep + MD_TAG_REP(tag_i);
     // An atom that was at least rlist from every face at the last build has
     // no pair across the boundary until the next build (both ends of a
@@ -163,7 +165,7 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
           dz = md_min_image(dz, L2, h2);
         }
         const double r2 = md_r2(dx, dy, dz);
-        const int tj = SINGLE ? 0 : md_type_of(xj);
+        const int tj = SINGLE ? 0 : min(md_type_of(xj), a.nt - 1);
         const PairCoef& cf = SINGLE ? a.c1 : sc[ti * a.nt + tj];
         if (md_lt_pos(r2, cf.cutsq_bits)) {
           // with t = r^-2 r^-6, A = lj1 r^-6 t, B = lj2 t:
@@ -200,7 +202,7 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
             gs0 += ds;
           } else {
             slot[tj * MD_BLOCK] += de;
-            slot[(MD_MAX_TYPES + tj) * MD_BLOCK] += ds;
+            slot[(a.nt + tj) * MD_BLOCK] += ds;
           }
         }
       });
@@ -212,7 +214,7 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
   } else {
     const XSplit si = md_ld_split(a.xs + ia);
     const int tag_i = __float_as_int(si.hi.w);
-    ti = MD_TAG_TYPE(tag_i);
+    ti = min((int)MD_TAG_TYPE(tag_i), a.nt - 1);
     const RepGeo* g = a.rep + MD_TAG_REP(tag_i);
     const float Lf0 = g->Lf[0], Lf1 = g->Lf[1], Lf2 = g->Lf[2];
     const float Ll0 = g->Llo[0], Ll1 = g->Llo[1], Ll2 = g->Llo[2];
@@ -242,7 +244,7 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
       }
       const float dx = hx + lx, dy = hy + ly, dz = hz + lz;
       const float r2 = __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, dx * dx));
-      const int tj = SINGLE ? 0 : MD_TAG_TYPE(__float_as_int(sj.hi.w));
+      const int tj = SINGLE ? 0 : min((int)MD_TAG_TYPE(__float_as_int(sj.hi.w)), a.nt - 1);
       const PairCoef& cf = SINGLE ? a.c1 : sc[ti * a.nt + tj];
       // the forward kernel's cutoff decision: FP64 r^2 inside the band
       bool in = r2 < cf.cutsqf;
@@ -278,11 +280,11 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
           md_acc2(geh, gel, de);
           md_acc2(gsh, gsl, ds);
         } else {
-          float2 e2 = slot2[tj * MD_BLOCK], s2 = slot2[(MD_MAX_TYPES + tj) * MD_BLOCK];
+          float2 e2 = slot2[tj * MD_BLOCK], s2 = slot2[(a.nt + tj) * MD_BLOCK];
           md_acc2(e2.x, e2.y, de);
           md_acc2(s2.x, s2.y, ds);
           slot2[tj * MD_BLOCK] = e2;
-          slot2[(MD_MAX_TYPES + tj) * MD_BLOCK] = s2;
+          slot2[(a.nt + tj) * MD_BLOCK] = s2;
         }
       }
     });
@@ -339,7 +341,7 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
           const int o = tt == ea ? eb : (tt == eb ? ea : -1);
           double v = 0.0;
           if (MIX) {  // FP32 pairs
-            float2 p = o >= 0 ? slot2[(w * MD_MAX_TYPES + o) * MD_BLOCK] : make_float2(0.f, 0.f);
+            float2 p = o >= 0 ? slot2[(w * a.nt + o) * MD_BLOCK] : make_float2(0.f, 0.f);
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) {
               const float h = __shfl_xor_sync(0xffffffffu, p.x, off);
@@ -348,7 +350,7 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
             }
             v = md_widen(p.x) + md_widen(p.y);
           } else {
-            if (o >= 0) v = slot[(w * MD_MAX_TYPES + o) * MD_BLOCK];
+            if (o >= 0) v = slot[(w * a.nt + o) * MD_BLOCK];
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
           }
@@ -360,12 +362,23 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
   }
 }
 
+// Dynamic shared memory: parameter terms and tables of the types that there are
+// (with room for MD_MAX_TYPES in every block, L1 was down to 28 KB: 64,000
+// atoms of two types, mixed half list 70 -> 65 us).
+inline size_t md_vjp_smem(bool single, int nt) {
+  return single ? 0
+                : sizeof(double) * 2 * nt * MD_BLOCK +
+                      (sizeof(PairCoef) + sizeof(VjpCoef)) * (size_t)(nt * nt) +
+                      sizeof(float) * (size_t)(nt * nt + MD_MAX_TYPES);
+}
+
 template <int PREC, bool HALF, bool SINGLE>
 cudaError_t md_vjp_launch_tpa(const VjpArgs& a, int tpa, unsigned blocks, cudaStream_t s) {
+  const size_t smem = md_vjp_smem(SINGLE, a.nt);
   switch (tpa) {
-    case 2: k_vjp<PREC, HALF, 2, SINGLE><<<blocks, MD_BLOCK, 0, s>>>(a); break;
-    case 4: k_vjp<PREC, HALF, 4, SINGLE><<<blocks, MD_BLOCK, 0, s>>>(a); break;
-    case 8: k_vjp<PREC, HALF, 8, SINGLE><<<blocks, MD_BLOCK, 0, s>>>(a); break;
+    case 2: k_vjp<PREC, HALF, 2, SINGLE><<<blocks, MD_BLOCK, smem, s>>>(a); break;
+    case 4: k_vjp<PREC, HALF, 4, SINGLE><<<blocks, MD_BLOCK, smem, s>>>(a); break;
+    case 8: k_vjp<PREC, HALF, 8, SINGLE><<<blocks, MD_BLOCK, smem, s>>>(a); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

@@ -218,3 +218,33 @@ def test_check_disp_segments(prec, every):
         assert r[:2] == runs[0][:2]
         for a, b in zip(r[2], runs[0][2]):
             np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("precision", [md.MD_PREC_FP64, md.MD_PREC_MIXED])
+@pytest.mark.parametrize("nt", [3, 8])
+def test_tables_of_many_types(nt, precision):
+    """The kernels' shared tables hold the types that there are: forces and
+    force VJP with an odd number of types and with the most, every pair of
+    types with coefficients of its own.  Bounds: 1e-11 (FP64) and 1e-3 (mixed)
+    of the largest component, as for two types."""
+    x, box = lattice(6, 0.8442, 0.2, 71)
+    t = np.arange(len(x), dtype=np.int32) % nt
+    u = S.uniform(72, 2 * nt * nt).reshape(2, nt, nt)
+    u = 0.5 * (u + u.transpose(0, 2, 1))
+    eps, sigma = 0.5 + u[0], 0.8 + 0.2 * u[1]
+    rc = 2.5 * sigma
+    tol = 1e-11 if precision == md.MD_PREC_FP64 else 1e-3
+    cot = S.normal(73, x.size).reshape(x.shape)
+    lj = O.LJ(eps, sigma, rc, ntypes=nt)
+    with md.LJMD(x, np.zeros_like(x), t, box, eps, sigma, rc, np.ones(nt), precision=precision,
+                 list_kind=md.MD_LIST_HALF, threads_per_atom=2) as ctx:
+        for compacted in ((0, 2) if precision == md.MD_PREC_FP64 else (0,)):
+            ctx.set_kernel(1 if compacted else 2, -1, compacted, 0)
+            ctx.compute_forces(0)
+            xw, _, f = (w.cpu().numpy() for w in ctx.get_state())
+            fref, _, _ = O.forces(xw, box, lj, type_=t, skin=0.3)
+            assert np.abs(f - fref).max() <= tol * np.abs(fref).max()
+        xbar, g = ctx.force_vjp(cot)
+    xref, gref = O.force_vjp(xw, box, lj, cot, type_=t, skin=0.3)
+    assert np.abs(xbar.cpu().numpy() - xref).max() <= tol * np.abs(xref).max()
+    assert np.abs(g - gref).max() <= tol * np.abs(gref).max()
