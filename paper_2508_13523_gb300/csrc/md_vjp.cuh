@@ -21,7 +21,7 @@
 // values with their rounding errors in the thread's own shared-memory column
 // (one row per thread put all lanes on the same banks), and the sums' atomics
 // are spread over rows.  62,500 atoms, half list, before and after: mixed 140 ->
-// 67 us, FP64 350 -> 272 us.
+// 59 us, FP64 350 -> 272 us.
 #pragma once
 
 #include <type_traits>
@@ -100,7 +100,10 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
   // The lane's entries in rounds (almost always one): an FP32 test of the hi
   // parts picks the skin entries that may be inside rc (few), then the inner
   // entries and the picked ones go through `take`, so that the derivative's
-  // code runs for lanes that almost all have a pair in range.
+  // code runs for lanes that almost all have a pair in range.  A lane waits for
+  // its gathers most of the time: two skin entries a round, the cotangent
+  // loaded with the position and the next entry's index before the pair
+  // (64,000 atoms of two types, mixed half list: 64 -> 59 us).
   __shared__ int sslot[MD_VJP_SLOTS][MD_BLOCK];
   auto walk = [&](const RepGeo* g, int type, auto take) {
     const float4 hi = md_ld_hi<MIX ? 1 : 0>(a.xs, ia);
@@ -108,9 +111,7 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
     int left = nin, q = t;
     do {
       int nsv = 0;
-      for (; q < nsk && nsv < MD_VJP_SLOTS; q += TPA) {
-        const int j = __ldcs(skin - (int64_t)q * 32);
-        const float4 hj = md_ld_hi<MIX ? 1 : 0>(a.xs, j);
+      auto test = [&](const float4& hj, int j) {
         float dx = hj.x - hi.x, dy = hj.y - hi.y, dz = hj.z - hi.z;
         dx = fabsf(dx) > hf0 ? dx - copysignf(g->Lf[0], dx) : dx;
         dy = fabsf(dy) > hf1 ? dy - copysignf(g->Lf[1], dy) : dy;
@@ -119,11 +120,31 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
         const float cut = SINGLE ? a.cut1
                                  : scut[type * a.nt + MD_TAG_TYPE(__float_as_int(hj.w))];
         if (r2f <= cut) sslot[nsv++][threadIdx.x] = j;
+      };
+      // two entries a round, their gathers in flight together
+      for (; q + TPA < nsk && nsv < MD_VJP_SLOTS - 1; q += 2 * TPA) {
+        const int j0 = __ldcs(skin - (int64_t)q * 32);
+        const int j1 = __ldcs(skin - (int64_t)(q + TPA) * 32);
+        const float4 h0 = md_ld_hi<MIX ? 1 : 0>(a.xs, j0), h1 = md_ld_hi<MIX ? 1 : 0>(a.xs, j1);
+        test(h0, j0);
+        test(h1, j1);
+      }
+      if (q + TPA >= nsk && q < nsk && nsv < MD_VJP_SLOTS) {
+        const int j = __ldcs(skin - (int64_t)q * 32);
+        test(md_ld_hi<MIX ? 1 : 0>(a.xs, j), j);
+        q += TPA;
       }
       const int own = left > t ? (left - t + TPA - 1) / TPA : 0;
       left = 0;
-      for (int k = 0; k < own + nsv; k++)
-        take(k < own ? __ldcs(row + (int64_t)(t + k * TPA) * 32) : sslot[k - own][threadIdx.x]);
+      auto entry = [&](int k) {
+        return k < own ? __ldcs(row + (int64_t)(t + k * TPA) * 32) : sslot[k - own][threadIdx.x];
+      };
+      int j = own + nsv > 0 ? entry(0) : 0;
+      for (int k = 0; k < own + nsv; k++) {
+        const int jn = k + 1 < own + nsv ? entry(k + 1) : 0;
+        take(j);
+        j = jn;
+      }
     } while (q < nsk);
   };
 
@@ -156,6 +177,7 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
       const long long h0 = g->halfL_bits[0], h1 = g->halfL_bits[1], h2 = g->halfL_bits[2];
       walk(g, ti, [&](int j) {
         const double4_32a xj = md_ld4(a.x4 + j);
+        const double4_32a cj = md_ld4(a.c + j);  // with the position: nearly every pair needs it
         double dx = __dsub_rn(xj.x, xi.x);
         double dy = __dsub_rn(xj.y, xi.y);
         double dz = __dsub_rn(xj.z, xi.z);
@@ -176,7 +198,6 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
           const double A = (cf.lj1 * r6inv) * tt;
           const double B = cf.lj2 * tt;
           const double gq = A - B;
-          const double4_32a cj = a.c[j];
           const double wx = ci.x - cj.x, wy = ci.y - cj.y, wz = ci.z - cj.z;
           const double dw = __fma_rn(dz, wz, __fma_rn(dy, wy, dx * wx));  // d . w = -(e . w)
           // J w = g w + 2 g' e (e . w) = g w + 2 g' (d . w) d
@@ -224,6 +245,7 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
     float axh = 0.f, axl = 0.f, ayh = 0.f, ayl = 0.f, azh = 0.f, azl = 0.f;
     walk(g, ti, [&](int j) {
       const XSplit sj = md_ld_split(a.xs + j);
+      const float4 cj = __ldg(a.cf + j);  // with the position: nearly every pair needs it
       float hx = sj.hi.x - si.hi.x, lx = sj.lo.x - si.lo.x;
       float hy = sj.hi.y - si.hi.y, ly = sj.lo.y - si.lo.y;
       float hz = sj.hi.z - si.hi.z, lz = sj.lo.z - si.lo.z;
@@ -256,7 +278,6 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
         const float r6inv = r2inv * r2inv * r2inv;
         const float gq = r6inv * (cf.lj1f * r6inv - cf.lj2f) * r2inv;
         const float gp = r2inv * r2inv * r6inv * (-7.0f * cf.lj1f * r6inv + 4.0f * cf.lj2f);
-        const float4 cj = __ldg(a.cf + j);
         const float wx = cix - cj.x, wy = ciy - cj.y, wz = ciz - cj.z;
         const float ew = -(dx * wx + dy * wy + dz * wz);
         const float s = -2.0f * gp * ew;
@@ -364,7 +385,7 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
 
 // Dynamic shared memory: parameter terms and tables of the types that there are
 // (with room for MD_MAX_TYPES in every block, L1 was down to 28 KB: 64,000
-// atoms of two types, mixed half list 70 -> 65 us).
+// atoms of two types, mixed half list 70 -> 64 us).
 inline size_t md_vjp_smem(bool single, int nt) {
   return single ? 0
                 : sizeof(double) * 2 * nt * MD_BLOCK +
