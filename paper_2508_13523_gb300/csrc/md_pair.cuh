@@ -54,7 +54,7 @@ struct PairArgs {
   const int32_t* numneigh;
   const int32_t* nbr;
   double* f;            // SoA fx[n], fy[n], fz[n]
-  unsigned long long* fix;   // SoA fixed-point accumulators (k_pair_q<FIX>, mixed
+  unsigned long long* fix;   // SoA fixed-point accumulators (k_pair_fx, mixed
                              // k_pair); zero at entry of a half-list launch
   const unsigned int* kmax;  // bound on the contributions one atom receives
   const PairCoef* coef;  // nt*nt table (multi-type)
@@ -123,9 +123,16 @@ __device__ __forceinline__ int md_next_tile(int* ctr, int nslots, int ntiles) {
 #ifndef MD_PAIR_MINB_EV_FULL
 #define MD_PAIR_MINB_EV_FULL 8
 #endif
-constexpr int md_pair_minb(int prec, bool half, bool ev) {
-  return prec == MD_PREC_MIXED ? (ev ? (half ? 9 : MD_PAIR_MINB_EV_FULL) : (half ? 9 : 10))
-                               : (ev ? 6 : 8);
+// Mixed force-only launches with several types hold more (the table's address,
+// the types): at 9 (half) and 10 blocks (full) they spill, one block less is
+// faster throughout -- two types, 1,048,576 atoms, best lanes: half list 472 ->
+// 461 us (7 blocks 475), full 565 -> 556 (8: 576), with the Coulomb term 363 ->
+// 353 and 413 -> 391 us; 64,000 atoms, half 45.0 -> 44.2 us (7: 42.9).
+constexpr int md_pair_minb(int prec, bool half, bool ev, bool single) {
+  return prec != MD_PREC_MIXED ? (ev ? 6 : 8)
+         : ev                  ? (half ? 9 : MD_PAIR_MINB_EV_FULL)
+         : single              ? (half ? 9 : 10)
+                               : (half ? 8 : 9);
 }
 
 // Dynamic shared memory of k_pair: the coefficient table of the types that
@@ -140,7 +147,8 @@ inline size_t md_pair_smem(bool single, int nt) {
 // COUL (mixed precision only): the lj/cut/coul/cut style, Eq. 1 plus the
 // cut Coulomb term qq / r.
 template <int PREC, bool HALF, int TPA, bool EV, bool SINGLE, bool COUL = false>
-__global__ void __launch_bounds__(MD_BLOCK, md_pair_minb(PREC, HALF, EV)) k_pair(const PairArgs a) {
+__global__ void __launch_bounds__(MD_BLOCK, md_pair_minb(PREC, HALF, EV, SINGLE))
+    k_pair(const PairArgs a) {
   static_assert(!COUL || PREC == MD_PREC_MIXED, "the FP64 Coulomb form is k_pair_q");
   if (md_stopped(a.stop)) return;
   extern __shared__ double s_tab[];  // md_pair_smem
