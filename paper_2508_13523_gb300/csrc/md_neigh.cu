@@ -823,9 +823,9 @@ static int run_rebuild(md_ctx* c) {
     }
     const cudaError_t ei = cudaGraphInstantiate(&c->rebuild_graph, g, 0);
     cudaGraphDestroy(g);
-    if (ei != cudaSuccess) {
+    if (ei != cudaSuccess) {  // no memory for a graph: without it
+      cudaGetLastError();
       c->rebuild_graph = nullptr;
-      return md_cuda_fail(ei);
     }
   }
   if (!c->rebuild_graph) return enqueue_rebuild(c);
