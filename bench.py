@@ -46,6 +46,8 @@ FP64_OPS_PER_CLK_SM = 2  # FP64 pipe lane-ops per clock per SM (1.25 TFLOP/s nom
 # for any other source or configuration the traffic is reported as null.
 PAIR_SOURCES = ("paper_2508_13523_gb300/csrc/md_pair.cuh",
                 "paper_2508_13523_gb300/csrc/md_pair_q.cuh",
+                "paper_2508_13523_gb300/csrc/md_pair_fx.cuh",
+                "paper_2508_13523_gb300/csrc/md_fx.cuh",
                 "paper_2508_13523_gb300/csrc/md_device.cuh")
 PAIR_TRAFFIC = {"349e1dd95a9eed30": {
     "fp64_half/2/1/2": (1422190336 + 92602112) / 4.0e6,
@@ -180,12 +182,12 @@ def fp64_ops_per_pair(compacted: int, coul: bool = False) -> int:
     With floating-point separations (per-atom kernel, compacted kernel with
     FP64 sums): separation 3, squared length 3, reciprocal refinement 3,
     r^-6 2, fpair 3, fpair * d 3 = 17 (the accumulations are reductions in
-    L2, off the pipe).  The compacted kernel with fixed-point sums forms the
-    separation, r^2 and fpair * d from exact fixed-point positions with
-    integer instructions, leaving reciprocal 3, r^-6 2, fpair 3 = 8.  The
-    lj/cut/coul/cut form takes 22 (reciprocal square root 5, r^-2 1, qq/r 1,
-    one FMA, instead of the reciprocal's 3) on the floating-point path,
-    which it always uses."""
+    L2, off the pipe).  With exact fixed-point separations, r^2 and fpair * d
+    the rest is reciprocal 3, r^-6 2, fpair 3 = 8: the count that the
+    fixed-point kernel (compacted 2) is rated with, although it evaluates these
+    with integer instructions too and leaves the FP64 pipe idle.  The
+    lj/cut/coul/cut form with FP64 arithmetic takes 22 (reciprocal square root
+    5, r^-2 1, qq/r 1, one FMA, instead of the reciprocal's 3)."""
     if coul:
         return 22
     return 8 if compacted == 2 else 17
@@ -797,13 +799,16 @@ def main():
     step_gbs = h["value"] / world * 1e6 * step_b / 1e9
     label = {0: f"k_pair<{prec},{kind},TPA={h['tpa']}>",
              1: f"k_pair_q<{kind}> (warp-compacted, FP64 force sums)",
-             2: f"k_pair_q<{kind}> (warp-compacted, fixed-point force sums)"}[h["compacted"]]
+             2: f"k_pair_fx<{kind}> (fixed-point pair force and sums)"}[h["compacted"]]
     if prec == "fp64":
         roofline = {"bound": "alu", "achieved": achieved_ops, "peak": fp64_peak,
                     "unit": "Gop/s (FP64 pipe)", "frac": achieved_ops / fp64_peak,
                     "peak_source": "2 FP64 lane-ops/clk/SM x 152 SMs x max SM clock (1.25 "
                                    "TFLOP/s nominal); DFMA measured at 628 Gop/s",
                     "ops_per_pair_visit": fp64_ops_per_pair(int(h["compacted"]))}
+        if int(h["compacted"]) == 2:
+            roofline["ops_note"] = ("the FP64 operations that the pair force needs beside exact "
+                                    "separations; k_pair_fx does them with integer instructions")
     else:  # the mixed form issues no FP64 operation per pair: HBM is its roof
         roofline = {"bound": "hbm", "achieved": achieved_gbs, "peak": hbm_peak, "unit": "GB/s",
                     "frac": achieved_gbs / hbm_peak, "peak_source": peak_src}

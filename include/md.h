@@ -120,8 +120,8 @@ typedef struct md_stats {
   int32_t carveout;         /* preferred shared-memory carveout of the pair
                                kernel in percent, -1 = driver default         */
   int32_t compacted;        /* FP64: 0 per-atom pair kernel, 1 warp-compacted
-                               kernel with FP64 reductions, 2 warp-compacted
-                               kernel with fixed-point reductions            */
+                               kernel with FP64 reductions, 2 fixed-point
+                               kernel                                        */
   int32_t persistent;       /* 1 if the pair kernel schedules tiles per SM; 2 if,
                                besides, each step is one cooperative launch   */
   double max_disp;          /* largest displacement since the last build (FP64
@@ -265,9 +265,9 @@ int md_get_neighbors(md_ctx* ctx, int64_t* offsets, int32_t* idx);
 /* Time the pair kernel for every allowed threads-per-atom value (Sec. 4.1:
  * parallelism over neighbors) and, in FP64, for the warp-compacted kernel
  * (in-range pairs queued per warp so that all 32 lanes do FP64 work; Sec.
- * 4.1's divergence) with either force summation (see md_set_kernel) on the
- * current list, the fixed-point one with one or two list entries per lane
- * per filter round (compacted 2 and 3), each with one block per tile and
+ * 4.1's divergence) with FP64 reductions on the current
+ * list, and for the fixed-point kernel with one or two list entries per
+ * lane per filter round (compacted 2 and 3), each with one block per tile and
  * with persistent per-SM tile scheduling (md_set_kernel's persistent 0 and
  * 1); keep the fastest.
  * The carveout keeps the driver's default and steps stay separate launches
@@ -283,8 +283,8 @@ int md_autotune(md_ctx* ctx);
  * qqrd2e q_a q_b (x_i - x_j) / r^3 (minimum image).  Charges are per type:
  * q (host, n_types doubles, copied).  rc_coul must be > 0 and at most the
  * largest rc (the lists are built at max rc + skin).  q == NULL turns the
- * term off.  The FP64 form runs the warp-compacted kernel (compacted 1 or 2;
- * compacted 0 becomes 2), the mixed form threads_per_atom 1, 2 or 4 (a
+ * term off.  The FP64 form runs compacted 1 or 2 of md_set_kernel (compacted 0
+ * becomes 2), the mixed form threads_per_atom 1, 2 or 4 (a
  * larger value becomes 2).  Forces are recomputed.  The adjoint entry points
  * return MD_EINVAL while the term is on (their derivative is of Eq. 1 only).
  * MD_EINVAL for a bad argument.  Synchronizes. */
@@ -294,11 +294,13 @@ int md_set_coulomb(md_ctx* ctx, const double* q, double rc_coul, double qqrd2e);
  * threads_per_atom in {1,2,4,8,16,32}; carveout -1 (driver default) or
  * 0..100 (% shared memory); compacted 1 selects the warp-compacted FP64
  * kernel (FP64 contexts, threads_per_atom 1) summing forces with FP64
- * atomics, compacted 2 the same kernel summing each force contribution,
- * rounded to a multiple of 2^-44, exactly in 64-bit integers (the result
- * does not depend on the order of the additions and lies within
- * contributions x 2^-45 of the exact FP64 sum; a contribution too large for
- * that range is added in FP64), compacted 3 the compacted 2 kernel whose
+ * atomics, compacted 2 the fixed-point kernel: positions, separations and
+ * Eq. 1's force in 64-bit integers, each force contribution rounded to a
+ * multiple of 2^-44 and summed exactly (the result does not depend on the
+ * order of the additions; every contribution lies within a count, 2^-44, and
+ * a few FP64 ulps of its exact value; pairs that the integers do not cover,
+ * among them contributions too large for the sums, are evaluated and added in
+ * FP64), compacted 3 the compacted 2 kernel whose
  * filter takes two list entries per lane per round, their loads in flight
  * together (Eq. 1 alone; md_get_stats then reports compacted 2 and
  * phase1_entries 2); persistent 1 launches one

@@ -500,7 +500,7 @@ int initial_capacity(const md_ctx* c) {
 }  // namespace
 
 // The step driver runs one cooperative launch per step (md_step_fused.cu):
-// persistent mode 2 on the compacted FP64 kernel with fixed-point sums.
+// persistent mode 2 on the fixed-point kernel.
 int md_step_fused_ok(const md_ctx* c) {
   return c->persist == 2 && c->precision == MD_PREC_FP64 && c->compact == 2 && !c->coul;
 }

@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(MD_BLOCK) k_integrate(const IntArgs a) {
 }
 
 // f += fix * 2^-MD_FIX_BITS and fix = 0, element by element (3n of each):
-// folds the fixed-point force sums of k_pair_q<FIX> into the FP64 forces
+// folds the fixed-point force sums of a pair launch into the FP64 forces
 // (which hold the contributions too large for the accumulators).  The fold
 // rounds once, in the final addition.
 // Two elements per thread with 16-byte accesses (both arrays are 256-byte

@@ -129,7 +129,7 @@ struct __align__(32) XSplit {
 #define MD_TAG_REP(tag) ((tag) >> 8)
 // Set in the tag of xs (XSplit hi.w) only: some coordinate of the atom is
 // not a multiple of 2^-F of its box (or too large), so its pairs take the
-// FP64 separation path of the compacted kernel (XFix).
+// FP64 path of the fixed-point kernel (XFix).
 #define MD_TAG_OFFGRID 0x80
 
 // Positions as fixed-point integers X = x 2^F with F = RepGeo::xfix of the
@@ -140,8 +140,8 @@ struct __align__(32) XSplit {
 // atom is flagged (MD_TAG_OFFGRID).  The difference X_j - X_i is then the
 // exact separation x_j - x_i (which the FP64 subtraction also yields
 // exactly here), below 2^60 in magnitude for pairs closer than half the
-// box: the compacted FP64 kernel forms separations, r^2 and force
-// contributions from it with integer instructions.
+// box: the fixed-point kernel (md_pair_fx.cuh) forms separations, r^2 and the
+// force from it with integer instructions.
 struct __align__(32) XFix {
   long long x, y, z;
   long long w;  // the atom's tag (as md_tag_of(x4)) | F << 32
@@ -175,8 +175,8 @@ struct md_ctx {
   int check_disp;  // also rebuild when some atom moved more than skin/2 (checked per step)
   int carve;    // preferred shared-memory carveout (%) of the pair kernel; -1 default
   int compact;  // FP64: 0 = per-atom loop (md_pair.cuh), 1 = warp-compacted kernel
-                // (md_pair_q.cuh) with FP64 reductions, 2 = warp-compacted with
-                // fixed-point reductions
+                // (md_pair_q.cuh) with FP64 reductions, 2 = fixed-point kernel
+                // (md_pair_fx.cuh)
   int time_pair;           // md_time_pair_kernel: segments without graphs, events
                            // around every pair launch
   cudaEvent_t* pair_ev;    // 2 * MD_PAIR_TIMING_MAX events (start, stop), or NULL

@@ -21,8 +21,9 @@
 // instructions per 32 pairs against 560 in the kernel it replaced (8 FP64
 // operations per pair, in-range pairs repacked through per-warp queues, owner
 // sums in shared memory).  Per launch inside a step, before and after: half
-// list 4,000,000 atoms 2.34 -> 1.46 ms, 32,000 atoms 63 -> 27 us; full list
-// 256,000 atoms 355 -> 188 us, 4,000,000 atoms 4.0 -> 2.40 ms.  Tried and left
+// list 4,000,000 atoms 2.34 -> 1.46 ms, 32,000 atoms 63 -> 23 us; full list
+// 256,000 atoms 355 -> 180 us; with energy and virial, half list, 4,000,000
+// atoms 2.95 -> 1.76 ms.  Tried and left
 // out: the next record's gather one pair ahead (8 more registers, 4 % slower),
 // and dealing the entries above the warp's mean row length to its idle lanes
 // (22 % fewer rounds, but the owner's position and box become variables: no
@@ -58,7 +59,7 @@ template <bool HALF, bool EV, bool SINGLE, bool COUL>
 __device__ __noinline__ void md_pair_fx_slow(const PairArgs& a, const PairCoef* coef, int64_t i,
                                              int j, FxSlow& o) {
   const int64_t n = a.n;
-  // range of the accumulators (as k_pair_q)
+  // range of the accumulators (MD_FIX_BITS)
   const int kb = 32 - __clz((int)min(*a.kmax, 0x7fffffffu));
   const int ex_lim = min(1023 + MD_FIX_EMAX + 1, 1023 + 63 - MD_FIX_BITS - kb);
   const double4_32a xi = md_ld4(a.x4 + i), xj = md_ld4(a.x4 + j);
@@ -405,7 +406,8 @@ __device__ __forceinline__ void md_pair_fx_tiles(const PairArgs& a, const float 
 // Resident blocks per SM the register allocation must allow (9: 56 registers).
 // 4,000,000 atoms, force-only half list: 8, 9 and 10 blocks measured 1.60,
 // 1.53 and 1.57 ms; energy/virial half list with 6, 7, 8, 9 and 10 blocks 2.49,
-// 2.35, 2.27, 2.42 and 2.76 ms, full list 8, 9 and 10 blocks 3.21, 3.14 and 3.53.
+// 2.35, 2.27, 2.42 and 2.76 ms, full list 8, 9 and 10 blocks 3.21, 3.14 and 3.53
+// (whole energy passes, with the passes over atoms of that time).
 #define MD_FX_MINB 9
 constexpr int md_pair_fx_minb(bool half, bool ev) { return ev && half ? 8 : MD_FX_MINB; }
 
