@@ -135,7 +135,8 @@ typedef struct md_stats {
                                force-only pair kernel's walk: 1 or 2 for the
                                FP64 compacted fixed-point kernel (picked by
                                md_autotune or md_set_kernel), 2 for the mixed
-                               kernel, 1 for the others                       */
+                               kernel (its half list; the full list's walk
+                               takes three), 1 for the others                 */
 } md_stats;
 
 /* ---- single box ---------------------------------------------------------- */

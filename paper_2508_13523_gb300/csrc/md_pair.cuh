@@ -102,16 +102,23 @@ __device__ __forceinline__ int md_next_tile(int* ctr, int nslots, int ntiles) {
 
 // Resident blocks per SM the register allocation must allow.  The mixed
 // kernels are bound by the latency of their position loads: registers buy
-// loads in flight (two entries a round), resident warps hide them.
+// loads in flight, resident warps hide them.
 // Mixed half-list energy/virial launches: at 4M atoms 7, 8, 9 and 10 blocks
 // measured 2.00, 1.89, 1.82 and 1.97 ms (TPA 2).
-// Mixed force-only launches walk their rows two entries a round (MD_PAIR_U),
-// both gathers in flight: at 4M atoms (TPA 2) against one entry at 10
-// blocks, 1.469 -> 1.440 ms (half list, 9 blocks: 56 registers) and 1.717 ->
-// 1.408 ms (full list, 10 blocks); the half list at 10 blocks spills (1.60
-// ms), the full list at 9 blocks measured 1.437 ms.
+// Mixed force-only launches walk a row as one sequence, inner entries then skin
+// entries, two (half list: MD_PAIR_U) or three (full: MD_PAIR_U_FULL) a round,
+// their gathers in flight together; what is left over goes one by one, which is
+// why inner and skin part are not walked separately.  4M atoms, one type (best
+// lanes), two a round with separate parts against this: half list 1.206 ->
+// 1.188 ms (9 blocks: 56 registers; three a round at 8: 1.201), full list 1.158
+// (10 blocks, spills) -> 1.114 ms (8 blocks; two a round at 10: 1.155, four at
+// 7: 1.156); 62,500 atoms half 33.7 -> 33.0, full 30.6 -> 28.5 us.  A last round
+// with predicated pairs instead of the leftovers: half 1.28 ms.
 #ifndef MD_PAIR_U
 #define MD_PAIR_U 2
+#endif
+#ifndef MD_PAIR_U_FULL
+#define MD_PAIR_U_FULL 3
 #endif
 // Mixed full-list energy/virial launches: two entries a round at 8 blocks
 // measured 2.13 ms at 4M atoms, one at 10 (spills) 2.26 ms, one at 9
@@ -123,16 +130,15 @@ __device__ __forceinline__ int md_next_tile(int* ctr, int nslots, int ntiles) {
 #ifndef MD_PAIR_MINB_EV_FULL
 #define MD_PAIR_MINB_EV_FULL 8
 #endif
-// Mixed force-only launches with several types hold more (the table's address,
-// the types): at 9 (half) and 10 blocks (full) they spill, one block less is
-// faster throughout -- two types, 1,048,576 atoms, best lanes: half list 472 ->
-// 461 us (7 blocks 475), full 565 -> 556 (8: 576), with the Coulomb term 363 ->
-// 353 and 413 -> 391 us; 64,000 atoms, half 45.0 -> 44.2 us (7: 42.9).
+// With several types the half-list launches hold more (the table's address, the
+// types) and run at 8 blocks: two types, 1,048,576 atoms, 9, 8 and 7 blocks 472,
+// 461 and 475 us with separate parts, 490 and 456 at 9 and 8 with this walk;
+// the full list 565 (10 blocks, separate parts) -> 489 us (8 blocks; 7: 515),
+// with the Coulomb term 413 -> 378 us.
 constexpr int md_pair_minb(int prec, bool half, bool ev, bool single) {
   return prec != MD_PREC_MIXED ? (ev ? 6 : 8)
          : ev                  ? (half ? 9 : MD_PAIR_MINB_EV_FULL)
-         : single              ? (half ? 9 : 10)
-                               : (half ? 8 : 9);
+                               : (half && single ? 9 : 8);
 }
 
 // Dynamic shared memory of k_pair: the coefficient table of the types that
@@ -411,38 +417,29 @@ __global__ void __launch_bounds__(MD_BLOCK, md_pair_minb(PREC, HALF, EV, SINGLE)
           }
         }
       };
-      // inner entries from the front of the row, skin entries from the back
-      // (force-only launches: PU entries a round, their gathers in flight
-      // together)
-      constexpr int PU = EV ? (HALF ? 1 : MD_PAIR_U_EV_FULL) : MD_PAIR_U;
+      // inner entries from the front of the row, skin entries from the back;
+      // PU entries a round, their gathers in flight together
+      constexpr int PU = EV ? (HALF ? 1 : MD_PAIR_U_EV_FULL)
+                            : (HALF ? MD_PAIR_U : MD_PAIR_U_FULL);
       auto walk = [&](auto second) {
-        const int32_t* p = row + (int64_t)t * 32;
+        const int tot = nin + nsk;
+        auto at = [&](int q) {
+          return __ldcs(q < nin ? row + (int64_t)q * 32 : skin - (int64_t)(q - nin) * 32);
+        };
         int q = t;
-        if (PU == 2) {
-          for (; q + TPA < nin; q += 2 * TPA, p += 2 * TPA * 32) {
-            const int j0 = __ldcs(p), j1 = __ldcs(p + TPA * 32);
-            const XSplit s0 = md_ld_split(a.xs + j0), s1 = md_ld_split(a.xs + j1);
-            pair(j0, s0, q, second);
-            pair(j1, s1, q + TPA, second);
-          }
+        for (; q + (PU - 1) * TPA < tot; q += PU * TPA) {
+          int j[PU];
+          XSplit s[PU];
+#pragma unroll
+          for (int u = 0; u < PU; u++) j[u] = at(q + u * TPA);
+#pragma unroll
+          for (int u = 0; u < PU; u++) s[u] = md_ld_split(a.xs + j[u]);
+#pragma unroll
+          for (int u = 0; u < PU; u++) pair(j[u], s[u], q + u * TPA, second);
         }
-        for (; q < nin; q += TPA, p += TPA * 32) {
-          const int j = __ldcs(p);
+        for (; q < tot; q += TPA) {
+          const int j = at(q);
           pair(j, md_ld_split(a.xs + j), q, second);
-        }
-        const int32_t* ps = skin - (int64_t)t * 32;
-        q = t;
-        if (PU == 2) {
-          for (; q + TPA < nsk; q += 2 * TPA, ps -= 2 * TPA * 32) {
-            const int j0 = __ldcs(ps), j1 = __ldcs(ps - TPA * 32);
-            const XSplit s0 = md_ld_split(a.xs + j0), s1 = md_ld_split(a.xs + j1);
-            pair(j0, s0, nin + q, second);
-            pair(j1, s1, nin + q + TPA, second);
-          }
-        }
-        for (; q < nsk; q += TPA, ps -= TPA * 32) {
-          const int j = __ldcs(ps);
-          pair(j, md_ld_split(a.xs + j), nin + q, second);
         }
       };
       walk(std::false_type{});
