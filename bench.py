@@ -49,11 +49,11 @@ PAIR_SOURCES = ("paper_2508_13523_gb300/csrc/md_pair.cuh",
                 "paper_2508_13523_gb300/csrc/md_pair_fx.cuh",
                 "paper_2508_13523_gb300/csrc/md_fx.cuh",
                 "paper_2508_13523_gb300/csrc/md_device.cuh")
-PAIR_TRAFFIC = {"349e1dd95a9eed30": {
-    "fp64_half/2/1/2": (1422190336 + 92602112) / 4.0e6,
-    "fp64_full/2/1/2": (1768076288 + 86858752) / 4.0e6,
-    "mixed_half/0/2/2": (1083237888 + 83930112) / 4.0e6,
-    "mixed_full/0/2/2": (1417269504 + 76367360) / 4.0e6}}
+PAIR_TRAFFIC = {"5f6b6b44cb86c0f0": {
+    "fp64_half/2/1/2": (1144426496 + 85809408) / 4.0e6,
+    "fp64_full/2/1/2": (1544429568 + 80557568) / 4.0e6,
+    "mixed_half/0/2/2": (1121923072 + 82675968) / 4.0e6,
+    "mixed_full/0/2/2": (1416501248 + 75228416) / 4.0e6}}
 
 
 def pair_source_hash() -> str:
