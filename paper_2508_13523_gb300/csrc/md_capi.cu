@@ -804,6 +804,7 @@ int create_impl(const md_params* p, int nrep, const int64_t* rep_off, const doub
   if (rc == MD_OK) rc = dalloc(&c->cell_alt, n);
   if (rc == MD_OK) rc = dalloc(&c->rank, n);
   if (rc == MD_OK) rc = dalloc(&c->perm, n);
+  if (rc == MD_OK) rc = md_scan_alloc(c);
   if (rc == MD_OK) rc = dalloc(&c->cnt, c->ncell);
   if (rc == MD_OK) rc = dalloc(&c->start, c->ncell + 1);
   if (rc == MD_OK) rc = dalloc(&c->numneigh, 2 * n);

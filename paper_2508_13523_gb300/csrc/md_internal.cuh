@@ -237,8 +237,7 @@ struct md_ctx {
   double* f_alt;
   int32_t* id_alt;
   int32_t *cnt, *start, *rank, *perm, *cell_alt;
-  int64_t* scan_tmp;  // tile sums of the scans
-  int64_t scan_tmp_n;
+  int64_t* scan_tmp;  // tile sums of the scans (md_scan_alloc; graphs hold its address)
 
   // neighbor list: tiles of 32 atoms, column-major inside a tile:
   // entry k of atom i at nbr[(i/32)*maxneigh*32 + k*32 + i%32].  A row holds
@@ -304,6 +303,7 @@ struct md_ctx {
 // ---- entry points of the translation units ---------------------------------
 // md_neigh.cu
 int md_rebuild(md_ctx* c);  // wrap, sort, build (+grow)
+int md_scan_alloc(md_ctx* c);  // once, before the first scan
 int md_scan_i32(md_ctx* c, const int32_t* in, int32_t* out, int64_t n);
 int md_scan_i64(md_ctx* c, const int32_t* in, int64_t* out, int64_t n);
 int md_list_entries(md_ctx* c, int64_t* total);

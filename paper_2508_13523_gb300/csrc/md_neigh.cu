@@ -674,20 +674,20 @@ __global__ void k_csr_fill(const int32_t* __restrict__ numneigh, const int32_t* 
 
 // ---- host side -----------------------------------------------------------------
 
-static int scan_tmp_reserve(md_ctx* c, int64_t n) {
-  int64_t tiles = (n + SCAN_TILE - 1) / SCAN_TILE + 1;
-  if (tiles <= c->scan_tmp_n) return MD_OK;
-  if (c->scan_tmp) cudaFree(c->scan_tmp);
+// Tile sums for every scan of the context: over its cells (the rebuild) and
+// over its atoms (the list export).  One buffer that stays where it is, because
+// the rebuild graph holds its address.
+int md_scan_alloc(md_ctx* c) {
+  const int64_t most = c->ncell > c->n ? c->ncell : c->n;
+  const int64_t tiles = (most + SCAN_TILE - 1) / SCAN_TILE + 1;
+  if (cudaMalloc(&c->scan_tmp, sizeof(int64_t) * tiles) == cudaSuccess) return MD_OK;
   c->scan_tmp = nullptr;
-  c->scan_tmp_n = 0;
-  if (cudaMalloc(&c->scan_tmp, sizeof(int64_t) * tiles) != cudaSuccess) return MD_ENOMEM;
-  c->scan_tmp_n = tiles;
-  return MD_OK;
+  cudaGetLastError();
+  return MD_ENOMEM;
 }
 
 template <typename TOUT>
 static int scan_impl(md_ctx* c, const int32_t* in, TOUT* out, int64_t n) {
-  MD_TRY(scan_tmp_reserve(c, n));
   int64_t tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
   if (tiles > 0) {
     k_scan_tiles<TOUT><<<(unsigned)tiles, SCAN_THREADS, 0, c->stream>>>(in, out, n, c->scan_tmp);
@@ -805,7 +805,6 @@ static int enqueue_rebuild(md_ctx* c) {
 // boxes: 32,000 atoms 70 -> 62 us a rebuild); the first two run directly, since
 // most contexts that only load states never need a third.
 static int run_rebuild(md_ctx* c) {
-  MD_TRY(scan_tmp_reserve(c, c->ncell));
   if (!c->rebuild_graph && c->rebuilds++ >= 2) {
     if (cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
       cudaGetLastError();  // a stream that cannot be captured

@@ -1,0 +1,59 @@
+"""The neighbor list over many rebuilds (needs a GPU): what other calls between
+rebuilds may not disturb.  Runs are compared bit for bit: fixed-point force sums
+and the stable sort do not depend on the order of additions.
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+import paper_2508_13523_gb300 as md  # noqa: E402
+from paper_2508_13523_gb300 import synth as S  # noqa: E402
+
+
+def context(n_cells, seed, **kw):
+    x, box, _ = S.fcc(n_cells, 0.8442)
+    x = x + 0.1 * (S.uniform(seed, x.size).reshape(x.shape) - 0.5)
+    v = S.maxwell_boltzmann(np.ones(len(x)), 1.44, seed + 1)
+    kw = dict(dict(rebuild_every=10, threads_per_atom=1), **kw)
+    ctx = md.LJMD(x, v, None, box, 1.0, 1.0, 2.5, 1.0, **kw)
+    if kw.get("precision", md.MD_PREC_FP64) == md.MD_PREC_FP64:
+        ctx.set_kernel(1, -1, 2, 0)
+    ctx.compute_forces(0)
+    return ctx
+
+
+def final(ctx):
+    off, idx = ctx.neighbors()
+    return [a.cpu().numpy() for a in (*ctx.get_state(), off, idx)]
+
+
+@pytest.mark.parametrize("prec", [md.MD_PREC_FP64, md.MD_PREC_MIXED])
+@pytest.mark.parametrize("kind", [md.MD_LIST_HALF, md.MD_LIST_FULL])
+def test_list_export_between_rebuilds(prec, kind):
+    """Exporting the list scans over the atoms, which takes more scratch than the
+    scan over the cells (10,976 atoms: 6 tiles against 1); the rebuilds after it
+    are one graph by then and keep the address they were captured with.  Other
+    contexts take device memory in between."""
+    runs = []
+    for export in (False, True):
+        with context(14, 3, precision=prec, list_kind=kind) as ctx:
+            ctx.step(35)  # three rebuilds after the first
+            others = []
+            if export:
+                ctx.neighbors()
+                others = [context(4, 7 + k, precision=prec, list_kind=kind) for k in range(4)]
+                before = [final(o) for o in others]
+            ctx.step(40)
+            runs.append(final(ctx))
+            for o, b in zip(others, before if export else ()):
+                o.compute_forces(0)
+                for p, q in zip(final(o), b):
+                    np.testing.assert_array_equal(p, q)
+                o.close()
+    for p, q in zip(*runs):
+        np.testing.assert_array_equal(p, q)
