@@ -524,9 +524,12 @@ __global__ void __launch_bounds__(MD_BLOCK)
         const int l = HALF ? ch / LCH : 0, c = ch - l * LCH;
         const int left = s_off[l][27] - p0 - 32 * c;  // candidates from this chunk on
         if (left <= 0) continue;
-        float4 h = cx[l * LCAP + 32 * c + lane];
-        const int j = cj[l * LCAP + 32 * c + lane];
-        if (lane >= left) h.x = 3.0e38f;  // no candidate
+        float4 h = make_float4(3.0e38f, 0.f, 0.f, 0.f);  // no candidate: beyond every cutoff, type 0
+        int j = -1;
+        if (lane < left) {  // (the slots from there on were never written)
+          h = cx[l * LCAP + 32 * c + lane];
+          j = cj[l * LCAP + 32 * c + lane];
+        }
         const int tj = MD_TAG_TYPE(__float_as_int(h.w));
         const int a0 = HALF ? ((i0 ^ l) & 1) : 0, da = HALF ? 2 : 1;
         // IMG: minimum image per pair; OWN: the chunk holds own-cell atoms (each

@@ -11,6 +11,7 @@ torch = pytest.importorskip("torch")
 if not torch.cuda.is_available():
     pytest.skip("needs a CUDA GPU", allow_module_level=True)
 
+import oracle as O  # noqa: E402
 import paper_2508_13523_gb300 as md  # noqa: E402
 from paper_2508_13523_gb300 import synth as S  # noqa: E402
 
@@ -57,3 +58,26 @@ def test_list_export_between_rebuilds(prec, kind):
                 o.close()
     for p, q in zip(*runs):
         np.testing.assert_array_equal(p, q)
+
+
+@pytest.mark.parametrize("nt", [2, 8])
+@pytest.mark.parametrize("kind", [md.MD_LIST_HALF, md.MD_LIST_FULL])
+@pytest.mark.parametrize("cells", [3, 5, 8])
+def test_partial_chunks_with_several_types(cells, kind, nt):
+    """The build tests 32 candidates at a time and looks up a cutoff for the
+    types of each; the last chunk of a cell's candidates is seldom full.  The list
+    against the oracle's pairs, with types that make every table entry in use."""
+    x, box, _ = S.fcc(cells, 0.8442)
+    x = (x + 0.2 * (S.uniform(60 + nt, x.size).reshape(x.shape) - 0.5)) % box
+    t = np.arange(len(x), dtype=np.int32) % nt
+    u = S.uniform(61, nt * nt).reshape(nt, nt)
+    rc = 1.5 + 0.25 * (u + u.T)
+    with md.LJMD(x, np.zeros_like(x), t, box, np.ones((nt, nt)), np.ones((nt, nt)), rc,
+                 np.ones(nt), list_kind=kind, threads_per_atom=1) as ctx:
+        off, idx = (a.cpu().numpy() for a in ctx.neighbors())
+    rlist = float(rc.max()) + 0.3
+    i, j = O.pairs_brute(x, box, rlist)
+    want = np.unique(np.minimum(i, j) * len(x) + np.maximum(i, j))
+    a = np.repeat(np.arange(len(x)), np.diff(off))
+    got = np.sort(np.minimum(a, idx) * len(x) + np.maximum(a, idx))
+    np.testing.assert_array_equal(got, want if kind == md.MD_LIST_HALF else np.repeat(want, 2))
