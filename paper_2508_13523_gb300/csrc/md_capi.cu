@@ -156,6 +156,7 @@ int setup_geometry(md_ctx* c, const double* boxes) {
     }
     const int64_t nr = c->rep_off_host[r + 1] - c->rep_off_host[r];
     const int64_t nc3 = (int64_t)g.nc[0] * g.nc[1] * g.nc[2];
+    c->cells_used += nc3;
     if (nr / nc3 > c->occ_max) c->occ_max = nr / nc3;
     if (cells + ncr > (int64_t)INT32_MAX - 1) return MD_EINVAL;
     g.cell_base = (int)cells;

@@ -207,7 +207,8 @@ struct md_ctx {
   RepGeo* rep;               // device, nrep
   RepGeo* rep_host;          // host copy
   int64_t* rep_off_host;     // host, nrep + 1 atom offsets
-  int64_t ncell;
+  int64_t ncell;             // cells, with those that pad each box to whole bricks
+  int64_t cells_used;        // without them
   int64_t occ_max;           // atoms per cell of the fullest box, on average
   cudaStream_t stream;
   int own_stream;  // the context created the stream (caller passed NULL)

@@ -742,15 +742,22 @@ static int launch_build(md_ctx* c) {
   unsigned nb = (unsigned)md_blocks(c->n);
   const bool half = c->list_kind == MD_LIST_HALF;
   const int hs = c->xq ? 0 : 1;
-  // sparse boxes (mostly empty cells) keep one thread per atom: a block per cell
-  // would launch mostly empty blocks
-  if (c->ncell <= c->n) {
-    // one block per cell and 32 of its atoms; further groups are looped over
-    // unless the grid is small (boxes with few, full cells)
-    const int64_t occ = c->occ_max < 1 ? 1 : c->occ_max;
-    int64_t gy = (occ + 31) / 32;
-    if (c->ncell * gy > 8192) gy = 1;
-    const dim3 grid((unsigned)c->ncell, (unsigned)(gy < 64 ? gy : 64));
+  // A block per cell costs 4 to 5 ns a cell whatever the cell holds (its set-up
+  // is a chain of latencies), a thread per atom 0.3 to 0.6 ns an atom, but at
+  // least 50 us.  So few atoms per cell keep one thread per atom, unless the
+  // cells are too few to fill the chip.  2,048,000 atoms with rlist 2.8, half
+  // list, per atom against per cell: 2.3 atoms a cell 656 against 4,263 us, 9.0
+  // 1,232 against 1,577 us, full list there 1,873 against 1,674 us; 256,000
+  // atoms, 14.6 a cell 261 against 199 us; 55,296 atoms, half list: 8,000 cells
+  // of 6.9 atoms 100 against 88 us, 12,167 cells of 4.5 81 against 103 us.
+  if (c->cells_used <= 8192 || c->n >= (half ? 12 : 8) * c->cells_used) {
+    // one block per cell and 32 of its atoms; where the fullest box's cells hold
+    // more than others' the blocks loop over the rest
+    int64_t gy = (c->occ_max + 31) / 32;
+    const int64_t most = (8192 + c->n / 8) / c->ncell;
+    gy = gy < most ? gy : most;
+    gy = gy < 1 ? 1 : gy > 65535 ? 65535 : gy;
+    const dim3 grid((unsigned)c->ncell, (unsigned)gy);
     auto kern = half ? (c->nt == 1 ? k_build_cell<true, true> : k_build_cell<true, false>)
                      : (c->nt == 1 ? k_build_cell<false, true> : k_build_cell<false, false>);
     kern<<<grid, MD_BLOCK, 0, c->stream>>>(c->x4, c->xs, hs, c->start, c->n, c->geo, c->rep,

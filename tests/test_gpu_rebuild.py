@@ -81,3 +81,26 @@ def test_partial_chunks_with_several_types(cells, kind, nt):
     a = np.repeat(np.arange(len(x)), np.diff(off))
     got = np.sort(np.minimum(a, idx) * len(x) + np.maximum(a, idx))
     np.testing.assert_array_equal(got, want if kind == md.MD_LIST_HALF else np.repeat(want, 2))
+
+
+@pytest.mark.parametrize("kind", [md.MD_LIST_HALF, md.MD_LIST_FULL])
+@pytest.mark.parametrize("cells, density, rc", [
+    (24, 0.2, 2.5),    # 12,167 cells of 4.5 atoms: one thread per atom
+    (24, 0.3, 2.5),    # 8,000 cells of 6.9: one block per cell
+    (9, 0.8442, 4.8),  # one cell of 2,916 atoms: many blocks for it
+    (4, 0.8442, 2.2),  # one cell of 256
+])
+def test_build_routes(cells, density, rc, kind):
+    """Both forms of the build on either side of the rule that picks one, and cells
+    that take many groups of 32 atoms: the list against the oracle's pairs."""
+    x, box, _ = S.fcc(cells, density)
+    x = (x + 0.3 * (S.uniform(70, x.size).reshape(x.shape) - 0.5)) % box
+    with md.LJMD(x, np.zeros_like(x), None, box, 1.0, 1.0, rc, 1.0, list_kind=kind,
+                 threads_per_atom=1) as ctx:
+        off, idx = (a.cpu().numpy() for a in ctx.neighbors())
+    i, j = O.pairs_cells(x, box, rc + 0.3) if len(x) > 4000 else O.pairs_brute(x, box, rc + 0.3)
+    i, j, idx = (q.astype(np.int64) for q in (i, j, idx))  # keys up to n^2
+    want = np.sort(np.minimum(i, j) * len(x) + np.maximum(i, j))
+    a = np.repeat(np.arange(len(x)), np.diff(off))
+    got = np.sort(np.minimum(a, idx) * len(x) + np.maximum(a, idx))
+    np.testing.assert_array_equal(got, want if kind == md.MD_LIST_HALF else np.repeat(want, 2))
