@@ -426,6 +426,7 @@ __global__ void __launch_bounds__(MD_BLOCK)
   if (ob + (int)blockIdx.y * 32 >= oe) return;
   const RepGeo& g = rep[MD_TAG_REP(__float_as_int(ld_hi(xs, ob, hs).w))];
   const bool img = g.nc[0] < 3 || g.nc[1] < 3 || g.nc[2] < 3;  // minimum image per pair
+  const bool one = g.nc[0] * g.nc[1] * g.nc[2] == 1;  // the box is one cell, its own stencil
   if (threadIdx.x < gg.nt * gg.nt) scut[threadIdx.x] = gg.cutsqf[threadIdx.x];
   const float cut1 = gg.cutsqf[0];
   // the stencil's cells: their atoms, image shifts and places in the lists
@@ -492,7 +493,17 @@ __global__ void __launch_bounds__(MD_BLOCK)
     if (threadIdx.x < na) own[threadIdx.x] = ld_hi(xs, i0 + (int)threadIdx.x, hs);
     for (int p0 = 0; p0 < len; p0 += LCAP) {
       // stage the candidates of slots p0 .. p0 + LCAP - 1 of each list
-      for (int c = w; c < 27; c += BC_WARPS) {
+      if (one) {  // (a warp per cell would leave one warp to stage the whole box)
+        for (int k = p0 + (int)threadIdx.x; k < min(oe - ob, p0 + LCAP); k += MD_BLOCK) {
+          const float4 h = ld_hi(xs, ob + k, hs);
+#pragma unroll
+          for (int l = 0; l < NL; l++) {
+            cx[l * LCAP + k - p0] = h;
+            cj[l * LCAP + k - p0] = ob + k;
+          }
+        }
+      }
+      for (int c = one ? 27 : w; c < 27; c += BC_WARPS) {
         const int b = s_b[c], e = s_e[c];
         const float s0 = s_sh[c][0], s1 = s_sh[c][1], s2 = s_sh[c][2];
         for (int j = b + lane; j < e; j += 32) {
