@@ -98,12 +98,8 @@ __device__ __forceinline__ double md_widen(float x) {
 // contributions are exact and independent of their order.  On GB300 integer
 // atomics in shared memory run at ~5 per clock per SM, while FP64 ones go
 // through the FP64 pipe (~1.6 per clock per SM) that the pair arithmetic
-// needs; in global memory (L2) both kinds run off the SM's pipes.
-#define MD_FIX_BITS 44
-// Largest binary exponent e of a contribution 2^e <= |g| that may go to a
-// fixed-point accumulator: |g| < 2^(MD_FIX_EMAX + 1) keeps the conversion a
-// right shift.
-#define MD_FIX_EMAX 7
+// needs; in global memory (L2) both kinds run off the SM's pipes.  MD_FIX_BITS
+// and MD_FIX_EMAX are in md_fx.cuh.
 
 // g rounded to the nearest multiple of 2^-MD_FIX_BITS (halves away from
 // zero), as an integer count, using integer instructions only.  Returns

@@ -31,7 +31,14 @@
 #define MD_HD inline
 #endif
 
-// Per type pair; built on the host (set_fx in md_capi.cu).
+// The force accumulators' unit is 2^-MD_FIX_BITS.
+#define MD_FIX_BITS 44
+// Largest binary exponent e of a contribution 2^e <= |g| that may go to a
+// fixed-point accumulator: |g| < 2^(MD_FIX_EMAX + 1) keeps the conversion a
+// right shift.
+#define MD_FIX_EMAX 7
+
+// Per type pair; built on the host (md_set_fx).
 struct PairFx {
   // high words of S: at or below smin FP64 path (r or the force out of range),
   // below cut_lo inside the cutoff, above cut_hi outside; between the last two

@@ -1,0 +1,47 @@
+"""The fixed-point pair kernel's coefficients, evaluated on the host over pair
+types of all kinds: every contribution that the rule takes in fixed point stays
+in the accumulators' range and within a count of the exact force (and 2^-46 of
+its magnitude).  No GPU: the number formats of the kernel are plain C++.
+"""
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_2508_13523_gb300", "csrc")
+
+
+@pytest.fixture(scope="module")
+def check(tmp_path_factory):
+    exe = str(tmp_path_factory.mktemp("fx") / "fx_coef_check")
+    subprocess.check_call(["g++", "-O2", "-std=gnu++17", "-I", CSRC, "-x", "c++",
+                           os.path.join(HERE, "fx_coef_check.cpp"), "-o", exe])
+
+    def run(rows):
+        """rows of (eps, sigma, rc, rcmax, lmax, qq, rc_coul, samples): an array of
+        (bad, in fixed point, in range, worst / bound, smallest r in fixed point)."""
+        text = "\n".join(" ".join(repr(float(v)) for v in r[:7]) + f" {r[7]}" for r in rows)
+        out = subprocess.run([exe], input=text, capture_output=True, text=True, check=True).stdout
+        return np.array([[float(v) for v in line.split()] for line in out.splitlines()])
+
+    return run
+
+
+def test_stiff_pairs_with_short_cutoffs(check):
+    """Forces beyond the accumulators' range at every separation in fixed point's
+    reach, cutoffs at and below a power of two: the FP64 path takes them all."""
+    rows = [(3850.0, 2.0 ** (-1 / 6), 1.0, 1.0, 20.0, 0.0, 0.0, 2000),
+            (2183.0, 1.0, 1.0, 1.0, 20.0, 0.0, 0.0, 2000),
+            (1e5, 0.95, 1.0, 1.0, 20.0, 0.0, 0.0, 2000),
+            (4e4, 1.99, 2.0, 2.0, 20.0, 0.0, 0.0, 2000)]
+    r = check(rows)
+    assert (r[:, 0] == 0).all(), r
+
+
+def test_lj_units_in_fixed_point(check):
+    """eps = sigma = 1: fixed point down to where the force reaches 256."""
+    r = check([(1.0, 1.0, 2.5, 2.5, 168.0, 0.0, 0.0, 20000)])
+    assert r[0, 0] == 0 and 0.8637 < r[0, 4] < 0.866
+    assert abs(r[0, 1] / r[0, 2] - (2.5 - 0.865) / 2.0) < 0.01  # r uniform in 0.5 .. 2.5
