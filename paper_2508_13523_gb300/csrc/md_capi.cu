@@ -241,7 +241,7 @@ int md_upload_coef(md_ctx* c) {
       const int k = a * nt + b;
       const double qq = c->coul ? c->qqrd2e * c->qtype[a] * c->qtype[b] : 0.0;
       md_set_coef(tab[k], c->eps[k], c->sigma[k], c->rc[k], qq, c->coul ? c->rc_coul : 0.0);
-      md_set_fx(fx[k], c->eps[k], c->sigma[k], c->rc[k], c->fxR, c->lmax, qq,
+      md_set_fx(fx[k], nt == 1 && !c->coul, c->eps[k], c->sigma[k], c->rc[k], c->fxR, c->lmax, qq,
                 c->coul ? c->rc_coul : 0.0);
     }
   c->coef1 = tab[0];

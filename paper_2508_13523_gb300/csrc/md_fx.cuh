@@ -49,10 +49,10 @@ struct PairFx {
   long long k1;               // 4 k2 q^3, below 2^63
   int B, zsh1, sh1;           // 4^R / r^2 < 2^B for S > smin, B <= MD_FX_BMAX
   // general form (S normalized per pair):
-  int zsh, sh;                // as zsh1, sh1
+  int zsh, sh;                // |w 2^(57 + zsh)| < 2^63; as sh1
   int tsh;                    // c - 62
   unsigned long long csign;   // sigma^2 / 4^R 2^c, in [2^62, 2^63)
-  long long cm;               // C = cm 2^-(p + 8 - zsh), in [2^61, 2^62)
+  long long cm;               // C = cm 2^-(p + 9 - zsh), in [2^62, 2^63)
   double e2;                  // 2 eps
   // lj/cut/coul/cut (general form): rc_coul's bounds as cut_lo, cut_hi, and
   // qq = cq 2^-x in 62 bits with csh = x - 9 + 3R - p
@@ -165,8 +165,9 @@ MD_HD long long md_fx_force1(unsigned long long T, const PairFx& c, unsigned lon
   return md_mulhi_s((long long)T, w << c.zsh1);
 }
 
-// The general form, from tau 2^62: tau^3 2^59, w = tau^3 (2 tau^3 - 1) 2^57
-// and P = cm tau w.
+// The general form, from tau 2^62: tau^3 2^59, w = tau^3 (2 tau^3 - 1) 2^57 and
+// P = cm tau w.  (w is shifted before the product with tau, not after it: its
+// error then counts for far pairs with their small tau.)
 struct FxForce {
   unsigned long long tau3;
   long long w;
@@ -178,8 +179,7 @@ MD_HD FxForce md_fx_force(unsigned long long tau, long long cm, int zsh) {
   r.tau3 = md_mulhi_u(tau2 << 1, tau);                   // 2^59
   const long long u = (long long)(r.tau3 << 2) - (1LL << 60);  // (2 tau^3 - 1) 2^60
   r.w = md_mulhi_s((long long)(r.tau3 << 2), u);               // 2^61 2^60 / 2^64
-  const long long z = md_mulhi_s((long long)tau, r.w << 1);    // 2^56
-  r.P = md_mulhi_s(cm, z << zsh);
+  r.P = md_mulhi_s(cm, md_mulhi_s((long long)tau, r.w << zsh));  // z 2^(55 + zsh)
   return r;
 }
 

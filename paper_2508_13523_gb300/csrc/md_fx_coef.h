@@ -32,9 +32,10 @@ inline long long md_dd_fixed(MdDd a, int s) {
 }
 
 // Eq. 1's fixed-point coefficients of one type pair (md_fx.cuh).
-// qq, rc_coul: the Coulomb term (rc_coul <= 0: none).
-inline void md_set_fx(PairFx& p, double eps, double sigma, double rc, int R, double lmax,
-                      double qq, double rc_coul) {
+// qq, rc_coul: the Coulomb term (rc_coul <= 0: none).  only: the context's only
+// pair type, without a Coulomb term (the one-type form where B allows it).
+inline void md_set_fx(PairFx& p, bool only, double eps, double sigma, double rc, int R,
+                      double lmax, double qq, double rc_coul) {
   memset(&p, 0, sizeof(p));
   // exact sigma^2 as m 2^e, m < 2^106
   int es = 0;
@@ -87,22 +88,21 @@ inline void md_set_fx(PairFx& p, double eps, double sigma, double rc, int R, dou
   double tl = lo * (1.0 - 1e-9);
   if (coul && fabs(qq) * tl > flim * sigma * sigma) tl = flim * sigma * sigma / fabs(qq);
   if (!(tl > 1e-3)) return;
-  // z = tau^4 (2 tau^3 - 1) over tau < tl: smallest -0.0806 at tau^3 = 2 / 7
-  const double tm = pow(2.0 / 7.0, 1.0 / 3.0);
-  auto zabs = [](double t) { return t * t * t * t * fabs(2.0 * t * t * t - 1.0); };
-  double zmax = zabs(tl);
-  if (tl > tm && zabs(tm) > zmax) zmax = zabs(tm);
-  int ze = 0;
-  frexp(zmax * 1.001, &ze);  // zmax < 2^ze
-  p.zsh = 7 - ze < 0 ? 0 : 7 - ze;
+  // general form: largest |w| over tau < tl, w = tau^3 (2 tau^3 - 1), at tl or, on
+  // the attractive branch, at tau^3 = 1/4 (-1/8); |w| < 2^we
+  const double tw = cbrt(0.25);
+  auto wabs = [](double t) { return t * t * t * fabs(2.0 * t * t * t - 1.0); };
+  int we = 0;
+  frexp(1.001 * (tl > tw && wabs(tw) > wabs(tl) ? wabs(tw) : wabs(tl)), &we);
+  p.zsh = 6 - we;
   const MdDd s2 = md_dd_mul({sigma, 0.0}, {sigma, 0.0}), s6 = md_dd_mul(s2, md_dd_mul(s2, s2));
   const MdDd c6 = md_dd_mul(md_dd_mul({24.0, 0.0}, {eps, 0.0}), s6);
   const MdDd cc = md_dd_div(md_dd_mul({24.0, 0.0}, {eps, 0.0}), s2);  // C
   int ce = 0;
   frexp(cc.h, &ce);
-  const int cx = 62 - ce;
+  const int cx = 63 - ce;
   p.cm = md_dd_fixed(cc, cx);
-  p.sh = cx - 8 + p.zsh - 45 - R;
+  p.sh = cx - 9 + p.zsh - 45 - R;
   if (p.sh > 12) {  // small forces: more bits than the counts can use
     const int d = p.sh - 12;
     p.cm = d < 62 ? p.cm >> d : 0;
@@ -127,9 +127,9 @@ inline void md_set_fx(PairFx& p, double eps, double sigma, double rc, int R, dou
   }
   if (p.sh < 1) return;
   p.B = 0;
-  while (ldexp(1.0, p.B) < 1.001 * MD_FX_TAU_MAX * ratio) p.B++;
+  while (ldexp(1.0, p.B) < 1.001 * tl * ratio) p.B++;  // tau's scale: tl, small for stiff pairs
   if (p.B <= MD_FX_BMAX) {
-    const double q = ldexp(1.0, p.B) / ratio;  // s 2^B, in (1.5, 3.1)
+    const double q = ldexp(1.0, p.B) / ratio;  // between tl and 2.1 tl where B > 0
     // C q^4 = 24 eps sigma^6 2^(4B - 8R) = kf 2^ke; k2 in [2^55, 2^56], k1 = 4 k2 q^3
     int ke = 0;
     frexp(ldexp(c6.h, 4 * p.B - 8 * R), &ke);
@@ -141,7 +141,6 @@ inline void md_set_fx(PairFx& p, double eps, double sigma, double rc, int R, dou
       const double t = tl * k / 256.0, x = t / q;
       wmax = fmax(wmax, x * x * x * fabs(2.0 * t * t * t - 1.0));
     }
-    int we = 0;
     frexp(wmax * 1.02, &we);
     p.zsh1 = 5 - we < 0 ? 0 : 5 - we;  // |w 2^zsh1| < 2^63
     p.sh1 = 57 + p.zsh1 - ke - 45 - R;  // P = fpair 2^(57 + zsh1 - ke)
@@ -153,6 +152,10 @@ inline void md_set_fx(PairFx& p, double eps, double sigma, double rc, int R, dou
     }
     if (p.sh1 < 1) p.B = MD_FX_BMAX + 1;  // the general form
   }
+  // The general form is exact to some units of 2^-57 on the scale of tau = 1,
+  // 24 eps / sigma of them in a contribution near sigma; beyond 2^9 eps / sigma
+  // that would pass a count (the one-type form's scale follows tl)
+  if (!(only && p.B <= MD_FX_BMAX) && eps > 512.0 * sigma) return;
   int c = 0;
   while (scaled(c + 1 - 2 * R) < (1ULL << 63)) c++;  // sigma^2 / 4^R 2^c in [2^62, 2^63)
   p.csign = scaled(c - 2 * R);

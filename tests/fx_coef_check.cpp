@@ -43,9 +43,10 @@ int main() {
                &samples) == 8) {
     int R;
     if (std::frexp(rcmax, &R) == 0.5) R--;
-    PairFx c;
-    md_set_fx(c, eps, sigma, rc, R, lmax, qq, rcc);
     const bool coul = rcc > 0.0;
+    PairFx forms[2];  // the only type, and one of several
+    for (int form = 0; form < 2; form++)
+      md_set_fx(forms[form], form == 0 && !coul, eps, sigma, rc, R, lmax, qq, rcc);
     int fixed = 0, bad = 0, in_range = 0;
     double worst = 0.0, rlow = 1e300;
     const double rmax = coul && rcc > rc ? rcc : rc;
@@ -55,6 +56,7 @@ int main() {
       const double st = std::sqrt(1.0 - ct * ct);
       const double d[3] = {r * st * std::cos(ph), r * st * std::sin(ph), r * ct};
       for (int form = 0; form < 2; form++) {
+        const PairFx& c = forms[form];
         const bool single = form == 0;  // the one-type form, or the general one
         if (single && (coul || c.B > MD_FX_BMAX)) continue;
         long long A[3];
@@ -118,7 +120,7 @@ int main() {
         }
       }
     }
-    printf("%d %d %d %.6g %.17g %u\n", bad, fixed, in_range, worst, rlow, c.smin);
+    printf("%d %d %d %.6g %.17g %u\n", bad, fixed, in_range, worst, rlow, forms[0].smin);
   }
   return 0;
 }

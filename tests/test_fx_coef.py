@@ -40,6 +40,29 @@ def test_stiff_pairs_with_short_cutoffs(check):
     assert (r[:, 0] == 0).all(), r
 
 
+@pytest.mark.parametrize("coul", [False, True])
+def test_sweep_of_pair_types(check, coul):
+    rng = np.random.RandomState(11 + coul)
+    rows = []
+    for _ in range(400):
+        rc = 2.0 ** rng.uniform(-3, 4)
+        if rng.rand() < 0.3:
+            rc = 2.0 ** rng.randint(-2, 4) * (1.0 if rng.rand() < 0.5 else 1.0 - 2.0 ** -rng.randint(3, 50))
+        sigma = rc / 10 ** rng.uniform(-0.05, 1.1)
+        eps = 10 ** rng.uniform(-6, 6) * sigma
+        rcmax = rc * (1.0 if rng.rand() < 0.6 else rng.uniform(1.0, 6.0))
+        lmax = max(4.0, 2.0 * rcmax) * rng.uniform(1.2, 40.0)
+        qq, rcc = 0.0, 0.0
+        if coul:
+            qq = 10 ** rng.uniform(-4, 4) * rng.choice([-1, 1]) * sigma * sigma
+            rcc = rcmax * rng.uniform(0.3, 1.0)
+        rows.append((eps, sigma, rc, rcmax, lmax, qq, rcc, 300))
+    r = check(rows)
+    bad = np.nonzero(r[:, 0])[0]
+    assert len(bad) == 0, [(rows[k], r[k]) for k in bad[:3]]
+    assert (r[:, 1] > 0).mean() > 0.3  # the sweep does reach the fixed-point path
+
+
 def test_lj_units_in_fixed_point(check):
     """eps = sigma = 1: fixed point down to where the force reaches 256."""
     r = check([(1.0, 1.0, 2.5, 2.5, 168.0, 0.0, 0.0, 20000)])
