@@ -226,6 +226,24 @@ void md_set_coef(PairCoef& pc, double eps, double sigma, double rc, double qq,
   pc.lj4f = (float)pc.lj4;
 }
 
+// The fixed-point kernel's table for the contributions that an atom may receive
+// (c->kmax).  Synchronizes, as below.
+int md_upload_fx(md_ctx* c) {
+  const int nt = c->nt;
+  c->fx_d = md_fx_dense(c->kmax);
+  PairFx fx[MD_MAX_TYPES * MD_MAX_TYPES];
+  memset(fx, 0, sizeof(fx));
+  for (int k = 0; k < nt * nt; k++) {
+    const double qq = c->coul ? c->qqrd2e * c->qtype[k / nt] * c->qtype[k % nt] : 0.0;
+    md_set_fx(fx[k], nt == 1 && !c->coul, c->fx_d, c->eps[k], c->sigma[k], c->rc[k], c->fxR,
+              c->lmax, qq, c->coul ? c->rc_coul : 0.0);
+  }
+  c->fx1 = fx[0];
+  MD_CUDA(cudaMemcpyAsync(c->fxt, fx, sizeof(fx), cudaMemcpyHostToDevice, c->stream));
+  MD_CUDA(cudaStreamSynchronize(c->stream));
+  return MD_OK;
+}
+
 // Coefficient table (device), the single-type copy, and the FP32 cutoff
 // bounds (device copy for the compacted kernel).  Synchronizes: the host
 // table must outlive the copies.
@@ -234,22 +252,17 @@ int md_upload_coef(md_ctx* c) {
   set_cut_bounds(c);
   PairCoef tab[MD_MAX_TYPES * MD_MAX_TYPES];
   memset(tab, 0, sizeof(tab));
-  PairFx fx[MD_MAX_TYPES * MD_MAX_TYPES];
-  memset(fx, 0, sizeof(fx));
   for (int a = 0; a < nt; a++)
     for (int b = 0; b < nt; b++) {
       const int k = a * nt + b;
       const double qq = c->coul ? c->qqrd2e * c->qtype[a] * c->qtype[b] : 0.0;
       md_set_coef(tab[k], c->eps[k], c->sigma[k], c->rc[k], qq, c->coul ? c->rc_coul : 0.0);
-      md_set_fx(fx[k], nt == 1 && !c->coul, c->eps[k], c->sigma[k], c->rc[k], c->fxR, c->lmax, qq,
-                c->coul ? c->rc_coul : 0.0);
     }
   c->coef1 = tab[0];
-  c->fx1 = fx[0];
-  MD_CUDA(cudaMemcpyAsync(c->fxt, fx, sizeof(fx), cudaMemcpyHostToDevice, c->stream));
   MD_CUDA(cudaMemcpyAsync(c->coef, tab, sizeof(tab), cudaMemcpyHostToDevice, c->stream));
   MD_CUDA(cudaMemcpyAsync(c->cut_hi_dev, c->geo.cut_hi, sizeof(c->geo.cut_hi),
                           cudaMemcpyHostToDevice, c->stream));
+  if (c->precision == MD_PREC_FP64) return md_upload_fx(c);
   MD_CUDA(cudaStreamSynchronize(c->stream));
   return MD_OK;
 }
@@ -360,17 +373,6 @@ int md_fresh_start(md_ctx* c) {
 
 namespace {
 
-// The fixed-point kernel keeps contributions below 2^(MD_FIX_EMAX + 1); an
-// atom that may receive k >= 2^11 of them needs contributions below 2^(63 -
-// MD_FIX_BITS) / k.  Returns log2 of the factor (the force falls at least as
-// r^-7, so a larger smin by that factor does it).
-int fx_dense(const md_ctx* c) {
-  int kb = 0;
-  while (kb < 31 && ((unsigned)c->kmax >> kb)) kb++;
-  const int d = kb - (63 - MD_FIX_BITS - (MD_FIX_EMAX + 1));
-  return d > 0 ? d : 0;
-}
-
 PairArgs pair_args(md_ctx* c) {
   PairArgs a;
   a.x4 = c->x4;
@@ -385,9 +387,6 @@ PairArgs pair_args(md_ctx* c) {
   a.fxt = c->fxt;
   a.fx1 = c->fx1;
   a.fxR = c->fxR;
-  a.fx_dense = fx_dense(c);
-  if (a.fx_dense)
-    a.fx1.smin = a.fx_dense < __builtin_clz(a.fx1.smin) ? a.fx1.smin << a.fx_dense : ~0u;
   a.nrep = c->nrep;
   // one type: at most maxneigh + 64 terms x^3 2^62 < 2^62 in 64 bits
   a.ev_shift = 0;
@@ -497,7 +496,7 @@ int enqueue_checked(md_ctx* c, int m, int last_k2) {
 
 int run_segment(md_ctx* c, int m, int last_k2, int check = 0) {
   if (c->time_pair) return run_segment_timed(c, m, last_k2);
-  GraphKey key{m, last_k2, check};
+  GraphKey key{m, last_k2, check, c->fx_d};
   auto it = c->graphs->find(key);
   if (it == c->graphs->end()) {
     cudaGraph_t g = nullptr;

@@ -31,10 +31,21 @@ inline long long md_dd_fixed(MdDd a, int s) {
   return (long long)f + llrint((h - f) + ldexp(a.l, s));
 }
 
+// An atom that may receive kmax contributions: its sums hold 2^11 of the largest,
+// 2^(MD_FIX_EMAX + 1) each, without overflow.  The power of two by which the
+// contributions have to be smaller where there may be more.
+inline int md_fx_dense(unsigned int kmax) {
+  int kb = 0;
+  while (kb < 31 && (kmax >> kb)) kb++;
+  const int d = kb - (63 - MD_FIX_BITS - (MD_FIX_EMAX + 1));
+  return d > 0 ? d : 0;
+}
+
 // Eq. 1's fixed-point coefficients of one type pair (md_fx.cuh).
 // qq, rc_coul: the Coulomb term (rc_coul <= 0: none).  only: the context's only
 // pair type, without a Coulomb term (the one-type form where B allows it).
-inline void md_set_fx(PairFx& p, bool only, double eps, double sigma, double rc, int R,
+// dense: see md_fx_dense.
+inline void md_set_fx(PairFx& p, bool only, int dense, double eps, double sigma, double rc, int R,
                       double lmax, double qq, double rc_coul) {
   memset(&p, 0, sizeof(p));
   // exact sigma^2 as m 2^e, m < 2^106
@@ -68,7 +79,7 @@ inline void md_set_fx(PairFx& p, bool only, double eps, double sigma, double rc,
   // largest tau with |F| below the accumulators' range for every smaller one
   // (|F| = 24 eps / sigma tau^3.5 |2 tau^3 - 1|, largest of the attractive
   // branch 2.397 eps / sigma at tau^3 = 7 / 26)
-  const double fs = 24.0 * eps / sigma, flim0 = ldexp(1.0 - ldexp(1.0, -10), MD_FIX_EMAX + 1);
+  const double fs = 24.0 * eps / sigma, flim0 = ldexp(1.0 - ldexp(1.0, -10), MD_FIX_EMAX + 1 - dense);
   const bool coul = rc_coul > 0.0 && qq != 0.0;  // each term then gets half the range
   const double flim = coul ? 0.5 * flim0 : flim0;
   auto force = [&](double t) { return fs * pow(t, 3.5) * fabs(2.0 * t * t * t - 1.0); };

@@ -162,8 +162,12 @@ struct GraphKey {
   int m;        // force/integrate pairs in the segment
   int last_k2;  // segment ends with the final half kick
   int check;    // the segment checks the displacement (DispStop)
+  int dense;    // the one-type coefficients in it are those of this md_fx_dense
   bool operator<(const GraphKey& o) const {
-    return m != o.m ? m < o.m : last_k2 != o.last_k2 ? last_k2 < o.last_k2 : check < o.check;
+    return m != o.m               ? m < o.m
+           : last_k2 != o.last_k2 ? last_k2 < o.last_k2
+           : check != o.check     ? check < o.check
+                                  : dense < o.dense;
   }
 };
 
@@ -201,6 +205,7 @@ struct md_ctx {
   PairFx fx1;                // fixed-point coefficients when nt == 1
   PairFx* fxt;               // nt*nt fixed-point coefficients (device)
   int fxR;                   // largest rc <= 2^fxR
+  int fx_d;                  // md_fx_dense that the coefficients are for
   double lmax;               // largest box edge
   Geo geo;
   int nrep;                  // replicas
@@ -333,6 +338,7 @@ static inline int md_barrier_status(const md_ctx* c) {
 // qq, rc_coul: the Coulomb term (rc_coul <= 0: none)
 void md_set_coef(PairCoef& pc, double eps, double sigma, double rc, double qq = 0.0,
                  double rc_coul = 0.0);
+int md_upload_fx(md_ctx* c);    // the fixed-point coefficients alone
 int md_upload_coef(md_ctx* c);  // coefficients, FP32 filter bounds, single-type copy
 
 // md_integrate.cu

@@ -27,6 +27,7 @@
 #include <type_traits>
 
 #include "md_device.cuh"
+#include "md_fx_coef.h"
 #include "md_internal.cuh"
 
 namespace {
@@ -868,10 +869,8 @@ int md_rebuild(md_ctx* c) {
     c->max_count = (int32_t)mc;
     uint32_t kmax;
     memcpy(&kmax, (const char*)(c->h_pinned + 9) + sizeof(mc), sizeof(kmax));
-    // captured graphs hold the range that follows from it (fx_dense)
-    if ((kmax | c->kmax) >= (1u << (63 - MD_FIX_BITS - (MD_FIX_EMAX + 1))) && kmax != c->kmax)
-      md_drop_graphs(c);
     c->kmax = kmax;
+    if (c->xq && md_fx_dense(kmax) != c->fx_d) MD_TRY(md_upload_fx(c));
     if ((int)mc <= c->maxneigh) {
       float disp2;
       memcpy(&disp2, &before[0], sizeof(disp2));

@@ -137,9 +137,6 @@ __device__ __forceinline__ void md_pair_fx_tiles(const PairArgs& a, const float 
   if (!SINGLE) {
     for (int k = threadIdx.x; k < a.nt * a.nt; k += blockDim.x) {
       sf[k] = a.fxt[k];
-      // atoms with very many partners: a smaller range per contribution (fx_dense)
-      if (a.fx_dense)
-        sf[k].smin = a.fx_dense < __clz((int)sf[k].smin) ? sf[k].smin << a.fx_dense : ~0u;
       scut[k] = cut_hi_tab[k];
     }
   }

@@ -3,7 +3,7 @@
 // separations read from stdin, and reports every contribution that is out of
 // the accumulators' range or off the exact force (128-bit floats).
 //
-// One line per pair type: eps sigma rc rcmax lmax qq rc_coul samples
+// One line per pair type: eps sigma rc rcmax lmax qq rc_coul samples dense
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -37,16 +37,16 @@ static double next_uniform(unsigned long long& s) {
 
 int main() {
   double eps, sigma, rc, rcmax, lmax, qq, rcc;
-  int samples;
+  int samples, dense;
   unsigned long long seed = 1;
-  while (scanf("%lf %lf %lf %lf %lf %lf %lf %d", &eps, &sigma, &rc, &rcmax, &lmax, &qq, &rcc,
-               &samples) == 8) {
+  while (scanf("%lf %lf %lf %lf %lf %lf %lf %d %d", &eps, &sigma, &rc, &rcmax, &lmax, &qq, &rcc,
+               &samples, &dense) == 9) {
     int R;
     if (std::frexp(rcmax, &R) == 0.5) R--;
     const bool coul = rcc > 0.0;
     PairFx forms[2];  // the only type, and one of several
     for (int form = 0; form < 2; form++)
-      md_set_fx(forms[form], form == 0 && !coul, eps, sigma, rc, R, lmax, qq, rcc);
+      md_set_fx(forms[form], form == 0 && !coul, dense, eps, sigma, rc, R, lmax, qq, rcc);
     int fixed = 0, bad = 0, in_range = 0;
     double worst = 0.0, rlow = 1e300;
     const double rmax = coul && rcc > rc ? rcc : rc;
@@ -116,7 +116,7 @@ int main() {
           const double tol = 1.0 + (double)q_scale(mag * (e[q] < 0 ? -e[q] : e[q]),
                                                    MD_FIX_BITS - 46);
           if (off / tol > worst) worst = off / tol;
-          if (!(off <= tol) || std::llabs(n) >= 1LL << (MD_FIX_BITS + MD_FIX_EMAX + 1)) bad++;
+          if (!(off <= tol) || std::llabs(n) >= 1LL << (MD_FIX_BITS + MD_FIX_EMAX + 1 - dense)) bad++;
         }
       }
     }

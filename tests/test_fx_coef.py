@@ -20,9 +20,10 @@ def check(tmp_path_factory):
                            os.path.join(HERE, "fx_coef_check.cpp"), "-o", exe])
 
     def run(rows):
-        """rows of (eps, sigma, rc, rcmax, lmax, qq, rc_coul, samples): an array of
-        (bad, in fixed point, in range, worst / bound, smallest r in fixed point)."""
-        text = "\n".join(" ".join(repr(float(v)) for v in r[:7]) + f" {r[7]}" for r in rows)
+        """rows of (eps, sigma, rc, rcmax, lmax, qq, rc_coul, samples[, dense]): an
+        array of (bad, in fixed point, in range, worst / bound, smallest r in fixed point)."""
+        text = "\n".join(" ".join(repr(float(v)) for v in r[:7]) + f" {r[7]} {r[8] if len(r) > 8 else 0}"
+                         for r in rows)
         out = subprocess.run([exe], input=text, capture_output=True, text=True, check=True).stdout
         return np.array([[float(v) for v in line.split()] for line in out.splitlines()])
 
@@ -56,7 +57,7 @@ def test_sweep_of_pair_types(check, coul):
         if coul:
             qq = 10 ** rng.uniform(-4, 4) * rng.choice([-1, 1]) * sigma * sigma
             rcc = rcmax * rng.uniform(0.3, 1.0)
-        rows.append((eps, sigma, rc, rcmax, lmax, qq, rcc, 300))
+        rows.append((eps, sigma, rc, rcmax, lmax, qq, rcc, 300, rng.choice([0, 0, 0, 1, 3, 6])))
     r = check(rows)
     bad = np.nonzero(r[:, 0])[0]
     assert len(bad) == 0, [(rows[k], r[k]) for k in bad[:3]]
@@ -68,3 +69,16 @@ def test_lj_units_in_fixed_point(check):
     r = check([(1.0, 1.0, 2.5, 2.5, 168.0, 0.0, 0.0, 20000)])
     assert r[0, 0] == 0 and 0.8637 < r[0, 4] < 0.866
     assert abs(r[0, 1] / r[0, 2] - (2.5 - 0.865) / 2.0) < 0.01  # r uniform in 0.5 .. 2.5
+
+
+@pytest.mark.parametrize("dense", [1, 2, 3, 6])
+def test_dense_lists_keep_their_pairs_in_fixed_point(check, dense):
+    """Atoms that may have 2^(11 + dense) partners: contributions have to be smaller
+    by 2^dense, and only the pairs whose force is not leave fixed point."""
+    r = check([(1.0, 1.0, 4.2, 4.2, 60.0, 0.0, 0.0, 20000, dense)])
+    f = lambda r: 24.0 * (2.0 * r ** -13 - r ** -7)
+    lo, hi = 0.8, 1.12  # (the samples start at 0.2 rc = 0.84)
+    for _ in range(60):
+        mid = 0.5 * (lo + hi)
+        lo, hi = (lo, mid) if f(mid) < 2.0 ** (8 - dense) else (mid, hi)
+    assert r[0, 0] == 0 and hi - 1e-3 < r[0, 4] < hi + 0.005
