@@ -314,7 +314,7 @@ int md_set_lj(md_ctx* c, const double* eps, const double* sigma) {
     c->sigma[k] = sigma[k];
   }
   MD_TRY(md_upload_coef(c));
-  md_drop_graphs(c);  // graphs hold the single-type coefficients by value
+  md_drop_segments(c);  // they hold the single-type coefficients by value
   if (c->vcoef) MD_TRY(upload_vcoef(c));
   return MD_OK;
 }

@@ -1108,7 +1108,7 @@ int md_autotune(md_ctx* c) {
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   MD_TRY(rc);
-  md_drop_graphs(c);
+  md_drop_segments(c);
   c->tpa = best_tpa;
   c->compact = best_compact;
   c->persist = best_persist;
@@ -1133,7 +1133,7 @@ int md_set_coulomb(md_ctx* c, const double* q, double rc_coul, double qqrd2e) {
   } else {
     c->coul = 0;
   }
-  md_drop_graphs(c);  // graphs hold the single-type coefficients and cutoff bound by value
+  md_drop_graphs(c);  // they hold the cutoffs, and the single-type coefficients, by value
   MD_TRY(md_upload_coef(c));
   return md_launch_pair(c, 0, c->tpa);
 }
@@ -1151,7 +1151,7 @@ int md_set_kernel(md_ctx* c, int32_t threads_per_atom, int32_t carveout, int32_t
   if (compacted && (c->precision != MD_PREC_FP64 || t != 1)) return MD_EINVAL;
   if (c->coul && c->precision == MD_PREC_FP64 && !compacted) return MD_EINVAL;
   if (c->coul && c->precision != MD_PREC_FP64 && t > 4) return MD_EINVAL;
-  md_drop_graphs(c);
+  md_drop_segments(c);
   c->tpa = t;
   c->carve = carveout;
   c->compact = compacted == 3 ? 2 : compacted;

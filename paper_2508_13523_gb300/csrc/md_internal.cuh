@@ -314,7 +314,8 @@ int md_scan_i32(md_ctx* c, const int32_t* in, int32_t* out, int64_t n);
 int md_scan_i64(md_ctx* c, const int32_t* in, int64_t* out, int64_t n);
 int md_list_entries(md_ctx* c, int64_t* total);
 int md_list_to_csr(md_ctx* c, int64_t* offsets, int32_t* idx);
-void md_drop_graphs(md_ctx* c);
+void md_drop_segments(md_ctx* c);  // the step segments: kernel choice, one-type coefficients
+void md_drop_graphs(md_ctx* c);    // and the rebuild: list buffers, cutoffs
 
 // md_capi.cu
 int md_launch_pair(md_ctx* c, int ev, int tpa);

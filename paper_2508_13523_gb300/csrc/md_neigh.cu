@@ -742,12 +742,16 @@ static int grow_list(md_ctx* c, int new_max) {
   return MD_OK;
 }
 
-void md_drop_graphs(md_ctx* c) {
-  if (c->rebuild_graph) cudaGraphExecDestroy(c->rebuild_graph);
-  c->rebuild_graph = nullptr;
+void md_drop_segments(md_ctx* c) {
   if (!c->graphs) return;
   for (auto& kv : *c->graphs) cudaGraphExecDestroy(kv.second.first);
   c->graphs->clear();
+}
+
+void md_drop_graphs(md_ctx* c) {
+  if (c->rebuild_graph) cudaGraphExecDestroy(c->rebuild_graph);
+  c->rebuild_graph = nullptr;
+  md_drop_segments(c);
 }
 
 static int launch_build(md_ctx* c) {

@@ -104,3 +104,28 @@ def test_build_routes(cells, density, rc, kind):
     a = np.repeat(np.arange(len(x)), np.diff(off))
     got = np.sort(np.minimum(a, idx) * len(x) + np.maximum(a, idx))
     np.testing.assert_array_equal(got, want if kind == md.MD_LIST_HALF else np.repeat(want, 2))
+
+
+@pytest.mark.parametrize("prec", [md.MD_PREC_FP64, md.MD_PREC_MIXED])
+@pytest.mark.parametrize("kind", [md.MD_LIST_HALF, md.MD_LIST_FULL])
+def test_new_coefficients_with_a_captured_rebuild(prec, kind):
+    """set_lj and set_kernel keep the captured rebuild (it depends on neither):
+    a run with new coefficients is, bit for bit, that of a context created with
+    them."""
+    with context(10, 21, precision=prec, list_kind=kind) as ctx:
+        ctx.step(45)  # four rebuilds: captured by then
+        x, v, _ = ctx.get_state()
+        ctx.set_lj(1.25, 0.97)
+        ctx.set_kernel(2 if prec else 1, -1, 0 if prec else 3, 0)
+        ctx.set_state(x, v)
+        ctx.step(45)
+        got = final(ctx)
+    _, box, _ = S.fcc(10, 0.8442)
+    with md.LJMD(x, v, None, box, 1.25, 0.97, 2.5, 1.0, precision=prec, list_kind=kind,
+                 rebuild_every=10, threads_per_atom=1) as ctx:
+        ctx.set_kernel(2 if prec else 1, -1, 0 if prec else 3, 0)
+        ctx.set_state(x, v)
+        ctx.step(45)
+        want = final(ctx)
+    for p, q in zip(got, want):
+        np.testing.assert_array_equal(p, q)
