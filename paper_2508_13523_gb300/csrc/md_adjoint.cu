@@ -173,6 +173,20 @@ __global__ void k_sd_step(double4_32a* __restrict__ x4, double* __restrict__ f, 
   md_store_pos(p, gr, xs, xq, i);
 }
 
+// Row 0 of gbar = the sum of its rows.  One block per entry, one thread per row.
+__global__ void __launch_bounds__(MD_GBAR_ROWS) k_gbar_fold(double* __restrict__ gbar, int entries) {
+  __shared__ double part[MD_GBAR_ROWS / 32];
+  double v = gbar[(int64_t)threadIdx.x * entries + blockIdx.x];
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < MD_GBAR_ROWS / 32; w++) v += part[w];
+    gbar[blockIdx.x] = v;
+  }
+}
+
 int upload_vcoef(md_ctx* c) {
   VjpCoef tab[MD_MAX_TYPES * MD_MAX_TYPES];
   memset(tab, 0, sizeof(tab));
@@ -216,6 +230,13 @@ int vjp_lanes(const md_ctx* c) {
   return c->precision == MD_PREC_FP64 && c->n < 160000 ? 4 : 2;
 }
 
+// Rows of gbar: a few blocks' atomics queue for less time than the launch that
+// sums the rows takes (864 atoms, 54 blocks: one row saves 4 us of a call).
+int gbar_rows(const md_ctx* c) {
+  return md_blocks(c->n * (int64_t)vjp_lanes(c)) <= 64 ? 1 : MD_GBAR_ROWS;
+}
+size_t gbar_bytes(const md_ctx* c) { return sizeof(double) * gbar_rows(c) * 2 * c->nt * c->nt; }
+
 int launch_vjp(md_ctx* c) {
   VjpArgs a;
   a.x4 = c->x4;
@@ -228,6 +249,7 @@ int launch_vjp(md_ctx* c) {
   a.nbr = c->nbr;
   a.xbar = c->adj_xbar;
   a.gbar = c->gbar;
+  a.rows = gbar_rows(c);
   a.coef = c->coef;
   a.vcoef = (const VjpCoef*)c->vcoef;
   a.c1 = c->coef1;
@@ -253,15 +275,19 @@ int launch_vjp(md_ctx* c) {
 }
 
 // gbar (device rows, entry [min][max]) -> host, both entries of each pair.
+// The rows are summed on the device (all of them to pageable host memory took
+// 10 us more of a 90 us call: 864 atoms).
 int gbar_to_host(md_ctx* c, double* out) {
   const int nt = c->nt, nt2 = nt * nt;
-  double rows[MD_GBAR_ROWS * 2 * MD_MAX_TYPES * MD_MAX_TYPES];  // 128 KB
-  MD_CUDA(cudaMemcpyAsync(rows, c->gbar, sizeof(double) * MD_GBAR_ROWS * 2 * nt2,
-                          cudaMemcpyDeviceToHost, c->stream));
+  double* h = c->h_pinned + MD_PIN_GBAR;
+  if (gbar_rows(c) > 1) {
+    k_gbar_fold<<<2 * nt2, MD_GBAR_ROWS, 0, c->stream>>>(c->gbar, 2 * nt2);
+    c->launches++;
+    MD_CUDA(cudaGetLastError());
+  }
+  MD_CUDA(cudaMemcpyAsync(h, c->gbar, sizeof(double) * 2 * nt2, cudaMemcpyDeviceToHost,
+                          c->stream));
   MD_CUDA(cudaStreamSynchronize(c->stream));
-  double h[2 * MD_MAX_TYPES * MD_MAX_TYPES] = {0};
-  for (int r = 0; r < MD_GBAR_ROWS; r++)
-    for (int k = 0; k < 2 * nt2; k++) h[k] += rows[r * 2 * nt2 + k];
   for (int w = 0; w < 2; w++)
     for (int a = 0; a < nt; a++)
       for (int b = 0; b < nt; b++) {
@@ -325,8 +351,7 @@ int md_force_vjp(md_ctx* c, const double* cot, double* xbar, double* gbar) {
   MD_TRY(adj_reserve(c, 0));
   MD_TRY(to_sorted(c, cot, nullptr, c->adj_c));
   MD_CUDA(cudaMemsetAsync(c->adj_xbar, 0, sizeof(double) * 3 * c->n, c->stream));
-  MD_CUDA(cudaMemsetAsync(c->gbar, 0, sizeof(double) * MD_GBAR_ROWS * 2 * c->nt * c->nt,
-                          c->stream));
+  MD_CUDA(cudaMemsetAsync(c->gbar, 0, gbar_bytes(c), c->stream));
   MD_TRY(launch_vjp(c));
   MD_TRY(to_caller(c, c->adj_xbar, nullptr, xbar));
   return gbar_to_host(c, gbar);
@@ -366,8 +391,7 @@ int md_traj_vjp(md_ctx* c, int64_t nsteps, int32_t every, const double* ckpt_x,
   MD_CUDA(cudaMemsetAsync(XB, 0, sizeof(double) * 2 * n3, c->stream));
   MD_CUDA(cudaMemcpyAsync(CC, cot_final, sizeof(double) * n3, cudaMemcpyDeviceToDevice,
                           c->stream));
-  MD_CUDA(cudaMemsetAsync(c->gbar, 0, sizeof(double) * MD_GBAR_ROWS * 2 * c->nt * c->nt,
-                          c->stream));
+  MD_CUDA(cudaMemsetAsync(c->gbar, 0, gbar_bytes(c), c->stream));
   DtfArgs d;
   for (int t = 0; t < MD_MAX_TYPES; t++) d.dtf[t] = c->dtf[t];
   for (int64_t j = J; j >= 0; j--) {

@@ -663,9 +663,9 @@ int create_impl(const md_params* p, int nrep, const int64_t* rep_off, const doub
   if (rc == MD_OK) rc = dalloc(&c->dstep, MD_STOP_STEPS + 1);
   if (rc == MD_OK) rc = dalloc(&c->fmark, 3);
   if (rc == MD_OK) rc = dalloc(&c->i64_tmp, 4);
-  if (rc == MD_OK && cudaMallocHost((void**)&c->h_pinned, 32 * sizeof(double)) != cudaSuccess)
+  if (rc == MD_OK && cudaMallocHost((void**)&c->h_pinned, MD_PIN * sizeof(double)) != cudaSuccess)
     rc = MD_ENOMEM;
-  if (rc == MD_OK) memset(c->h_pinned, 0, 32 * sizeof(double));
+  if (rc == MD_OK) memset(c->h_pinned, 0, MD_PIN * sizeof(double));
   if (rc == MD_OK && cudaMallocHost((void**)&c->ev_host,
                                     sizeof(double) * (size_t)nrep * MD_EV_STRIDE) != cudaSuccess)
     rc = MD_ENOMEM;

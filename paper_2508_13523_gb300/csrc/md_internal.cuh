@@ -157,6 +157,10 @@ struct DispStop {
 };
 #define MD_STOP_STEPS 16  // steps per checked segment
 
+// Doubles of md_ctx::h_pinned; the parameter derivatives of a VJP start at MD_PIN_GBAR.
+#define MD_PIN_GBAR 32
+#define MD_PIN (MD_PIN_GBAR + 2 * MD_MAX_TYPES * MD_MAX_TYPES)
+
 // ---- context -----------------------------------------------------------------
 struct GraphKey {
   int m;        // force/integrate pairs in the segment
@@ -276,7 +280,7 @@ struct md_ctx {
   int* fmark;
   unsigned int* dstep; // check_disp: the displacement word after each drift of a segment
                        // (MD_STOP_STEPS + 1; [0] unused, dmax[0] takes its place)
-  double* h_pinned;    // small pinned host mirror (32 doubles; [16..] dstep)
+  double* h_pinned;    // small pinned host mirror (MD_PIN doubles; [16..] dstep)
   int64_t* i64_tmp;    // device int64 scratch (counts)
 
   // host staging for MD_MEM_HOST

@@ -46,9 +46,10 @@ struct VjpArgs {
   const int32_t* numneigh;
   const int32_t* nbr;
   double* xbar;          // SoA per sorted atom, accumulated (+=)
-  double* gbar;          // MD_GBAR_ROWS rows of 2 nt^2: dL/deps then dL/dsigma, entry
-                         // [min][max]; the blocks' sums are spread over the rows so
-                         // that their atomics do not queue on the same addresses
+  double* gbar;          // rows of 2 nt^2: dL/deps then dL/dsigma, entry [min][max]; the
+                         // blocks' sums are spread over the rows so that their atomics
+                         // do not queue on the same addresses
+  int rows;              // 1 or MD_GBAR_ROWS
   const PairCoef* coef;
   const VjpCoef* vcoef;
   PairCoef c1;
@@ -339,7 +340,7 @@ __global__ void __launch_bounds__(MD_BLOCK) k_vjp(const VjpArgs a) {
   }
   // parameter terms: entry [min(ti,tj)][max(ti,tj)] of each table
   const int nt2 = a.nt * a.nt;
-  double* grow = a.gbar + (int64_t)(blockIdx.x % MD_GBAR_ROWS) * 2 * nt2;
+  double* grow = a.gbar + (int64_t)(blockIdx.x % (unsigned)a.rows) * 2 * nt2;
   if (SINGLE) {
     double v[2] = {ge0, gs0};
 #pragma unroll
