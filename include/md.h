@@ -214,7 +214,10 @@ int md_get_state(md_ctx* ctx, double* x, double* v, double* f, int32_t mem);
 
 /* Wrap positions, sort atoms by cell and rebuild the neighbor list now
  * (Sec. 4: the list is periodically updated).  Grows the capacity and
- * rebuilds if an atom has more neighbors than fit.  Synchronizes. */
+ * rebuilds if an atom has more neighbors than fit.  Where that fails
+ * (MD_ENOMEM), here or in another call that rebuilds, there is no list: calls
+ * that need one return the same error until a rebuild succeeds (this call, or
+ * md_set_state).  Synchronizes. */
 int md_build_neighbors(md_ctx* ctx);
 
 /* Compute forces on the current list (Eq. 1 derivative, Sec. 4; half or full

@@ -238,6 +238,7 @@ int gbar_rows(const md_ctx* c) {
 size_t gbar_bytes(const md_ctx* c) { return sizeof(double) * gbar_rows(c) * 2 * c->nt * c->nt; }
 
 int launch_vjp(md_ctx* c) {
+  MD_TRY(c->list_rc);
   VjpArgs a;
   a.x4 = c->x4;
   a.xs = c->xs;

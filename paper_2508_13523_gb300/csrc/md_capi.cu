@@ -770,6 +770,7 @@ namespace {
 int launch_pair_impl(md_ctx* c, int ev, int tpa, int prezeroed, int defer_fold,
                      const DispStop* stop, int mark) {
   if (ev && defer_fold) return MD_EINVAL;
+  MD_TRY(c->list_rc);
   PairArgs a = pair_args(c);
   if (stop) a.stop = *stop;
   if (mark >= 0) a.fmark = c->fmark + mark % 3;
@@ -877,7 +878,7 @@ int md_set_state(md_ctx* c, const double* x, const double* v, int32_t mem) {
     x = c->stage;
     v = c->stage + 3 * n;
   }
-  if (keep) {
+  if (keep && c->list_rc == MD_OK) {
     // the list stays valid while no atom moved more than skin/2 since the
     // build (a pair can then have closed in by at most skin); the FP32
     // displacement is within 1e-6 relative of the exact one
@@ -943,6 +944,7 @@ int md_compute_forces(md_ctx* c, int32_t flags) {
 int md_step(md_ctx* c, int64_t nsteps) {
   if (!c || nsteps < 0) return MD_EINVAL;
   if (nsteps == 0) return MD_OK;
+  MD_TRY(c->list_rc);
   const int64_t every = c->rebuild_every;
   // the first pair launch of the step adds into f: K1 leaves it at zero
   MD_TRY(md_launch_integrate(c, MD_K1, 0, md_pair_accumulates(c)));
@@ -1198,7 +1200,7 @@ int md_get_stats(md_ctx* c, md_stats* out) {
   if (!c || !out) return MD_EINVAL;
   memset(out, 0, sizeof(*out));
   int64_t total = 0;
-  MD_TRY(md_list_entries(c, &total));
+  if (c->list_rc == MD_OK) MD_TRY(md_list_entries(c, &total));
   MD_CUDA(cudaMemcpyAsync(c->h_pinned + 11, c->dmax, sizeof(unsigned int), cudaMemcpyDeviceToHost,
                           c->stream));
   MD_CUDA(cudaStreamSynchronize(c->stream));

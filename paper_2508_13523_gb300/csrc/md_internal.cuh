@@ -306,6 +306,7 @@ struct md_ctx {
   // counters
   int64_t step, builds, dangerous, launches;
   int32_t max_count;
+  int list_rc;             // what the last rebuild returned: MD_OK, or there is no list
   uint32_t kmax;           // dmax[2] of the last build
   int64_t pairs_in_range;  // at the last md_energy
 };

@@ -635,8 +635,8 @@ __global__ void __launch_bounds__(MD_BLOCK)
       }
       __syncthreads();
     }
-    // on overflow the rows are incomplete (but in bounds); the host sees
-    // total > maxneigh, grows the list and rebuilds
+    // on overflow rows are left as they were; the host sees a count above
+    // maxneigh, grows the list and rebuilds, or lets nothing read them (list_rc)
     if (w == 0 && lane < na) {
       const int a = min(nin, maxneigh);
       numneigh[i] = a;
@@ -730,15 +730,19 @@ int md_scan_i64(md_ctx* c, const int32_t* in, int64_t* out, int64_t n) {
 static int grow_list(md_ctx* c, int new_max) {
   int64_t tiles = (c->n + 31) / 32;
   int64_t need = tiles * 32 * (int64_t)new_max;
+  md_drop_graphs(c);  // captured graphs hold the old pointer and capacity
   if (need > c->nbr_alloc) {
     if (c->nbr) cudaFree(c->nbr);
     c->nbr = nullptr;
     c->nbr_alloc = 0;
-    if (cudaMalloc(&c->nbr, sizeof(int32_t) * need) != cudaSuccess) return MD_ENOMEM;
+    if (cudaMalloc(&c->nbr, sizeof(int32_t) * need) != cudaSuccess) {
+      c->nbr = nullptr;
+      cudaGetLastError();
+      return MD_ENOMEM;
+    }
     c->nbr_alloc = need;
   }
   c->maxneigh = new_max;
-  md_drop_graphs(c);  // captured graphs hold the old pointer and capacity
   return MD_OK;
 }
 
@@ -859,8 +863,9 @@ static int run_rebuild(md_ctx* c) {
   return MD_OK;
 }
 
-int md_rebuild(md_ctx* c) {
+static int rebuild(md_ctx* c) {
   cudaStream_t s = c->stream;
+  if (!c->nbr) MD_TRY(grow_list(c, c->maxneigh));  // (an earlier growth found no memory)
   MD_TRY(run_rebuild(c));
   for (int attempt = 0; attempt < 4; attempt++) {
     if (attempt > 0) MD_TRY(enqueue_build(c));
@@ -892,7 +897,16 @@ int md_rebuild(md_ctx* c) {
   return MD_ENEIGH;
 }
 
+// Until a rebuild succeeds again, rows hold stale entries or there are none:
+// list_rc keeps them from being read.
+int md_rebuild(md_ctx* c) {
+  c->list_rc = MD_OK;
+  c->list_rc = rebuild(c);
+  return c->list_rc;
+}
+
 int md_list_entries(md_ctx* c, int64_t* total) {
+  MD_TRY(c->list_rc);
   unsigned long long* d = reinterpret_cast<unsigned long long*>(c->i64_tmp);
   MD_CUDA(cudaMemsetAsync(d, 0, sizeof(unsigned long long), c->stream));
   k_sum_counts<<<(unsigned)md_blocks(2 * c->n), MD_BLOCK, 0, c->stream>>>(c->numneigh, 2 * c->n, d);
@@ -908,6 +922,7 @@ int md_list_entries(md_ctx* c, int64_t* total) {
 }
 
 int md_list_to_csr(md_ctx* c, int64_t* offsets, int32_t* idx) {
+  MD_TRY(c->list_rc);
   const unsigned nb = (unsigned)md_blocks(c->n);
   int32_t* cnt_orig = c->rank;  // rebuild scratch, free between rebuilds
   k_csr_counts<<<nb, MD_BLOCK, 0, c->stream>>>(c->numneigh, c->id, c->n, cnt_orig);

@@ -129,3 +129,38 @@ def test_new_coefficients_with_a_captured_rebuild(prec, kind):
         want = final(ctx)
     for p, q in zip(got, want):
         np.testing.assert_array_equal(p, q)
+
+
+@pytest.mark.parametrize("kind", [md.MD_LIST_HALF, md.MD_LIST_FULL])
+def test_list_without_memory(kind):
+    """A list that has to grow and finds no device memory: the call says so, calls
+    that would read the list say so until a rebuild succeeds, and the context then
+    gives the forces of a new one."""
+    with context(20, 9, list_kind=kind) as ctx:
+        ctx.step(35)  # with captured segments and rebuild
+        x, v, f = ctx.get_state()
+        ctx.set_state(x, v)
+        want = ctx.get_state()
+        dense = 0.25 * x  # rows of thousands of entries: 350 MB and more
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        free, _ = torch.cuda.mem_get_info()
+        hold = torch.empty(free - (200 << 20), dtype=torch.uint8, device="cuda")
+        try:
+            with pytest.raises(md.MDError) as e:
+                ctx.set_state(dense, v)
+            assert e.value.code == md.MD_ENOMEM
+            for call in (lambda: ctx.compute_forces(0), lambda: ctx.step(5), ctx.energy,
+                         ctx.neighbor_count, lambda: ctx.force_vjp(v), ctx.build_neighbors,
+                         lambda: ctx.set_state(dense, v, keep_list=True)):
+                with pytest.raises(md.MDError) as e:
+                    call()
+                assert e.value.code == md.MD_ENOMEM
+            assert ctx.stats()["list_entries"] == 0
+        finally:
+            del hold
+            torch.cuda.empty_cache()
+        ctx.set_state(x, v)
+        for a, b in zip(ctx.get_state(), want):
+            assert torch.equal(a, b)
+        ctx.step(25)
