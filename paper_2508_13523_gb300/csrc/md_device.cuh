@@ -245,31 +245,37 @@ __device__ __forceinline__ void md_split(double x, const XGrid& g, float& hi, fl
   }
 }
 
-// x as a fixed-point count X = x 2^F, |x| < 2^(61 - F) (so |X| < 2^61); false
+// x as a fixed-point count X = x 2^F, |x| < 2^(63 - F) (so |X| < 2^63); false
 // beyond that range (and for infinities and NaNs).  Integer instructions only.
 // x = M 2^(e - 1075) with M the 53-bit significand: X = M 2^(e - 1075 + F),
 // an integer for |x| >= 2^(52 - F).  Smaller x are rounded to the nearest
 // multiple of 2^-F where F >= MD_XFIX_ROUND_F (an error of at most 2^-53, no
 // more than FP64's own rounding of a separation above 1); with a coarser
-// grid (boxes of more than 409 length units) they must be exact, else false.
-#define MD_XFIX_ROUND_F 52
+// grid they must be exact, else false.
 __device__ __forceinline__ bool md_xfix(double x, int F, long long& X) {
   const long long b = __double_as_longlong(x);
   const int e = (int)((b >> 52) & 0x7ff);
   X = 0;
   if (e == 0) return true;  // zero (or subnormal: rounds to it)
-  if (e - 1023 >= 61 - F) return false;  // |x| >= 2^(61 - F)
+  if (e - 1023 >= 63 - F) return false;  // |x| >= 2^(63 - F)
   const long long M = (b & 0xfffffffffffffLL) | (1LL << 52);
   const int sh = 1075 - F - e;
   long long m;
   if (sh <= 0) {
-    m = M << (-sh);  // -sh <= 8: |x| < 2^(61 - F)
+    m = M << (-sh);  // -sh <= 10: |x| < 2^(63 - F)
   } else {
     if (F < MD_XFIX_ROUND_F && (sh > 52 || (M & ((1LL << sh) - 1)) != 0)) return false;
     m = sh > 53 ? 0 : (M + (1LL << (sh - 1))) >> sh;
   }
   X = b < 0 ? -m : m;
   return true;
+}
+// The same counted from the box's centre, h = L 2^(F-1) above 0; false farther
+// than MD_XFIX_MAX from it.
+__device__ __forceinline__ bool md_xfix_centred(double x, int F, long long h, long long& X) {
+  const bool on = md_xfix(x, F, X) & (X > h - MD_XFIX_MAX);
+  X -= on ? h : 0;
+  return on & (X < MD_XFIX_MAX);
 }
 
 // Hi parts and tag of atom i: FP64 contexts keep only them, 16 bytes an atom
@@ -341,9 +347,11 @@ __device__ __forceinline__ XSplit md_store_pos(const double4_32a& p, const XGrid
   const int tag = md_tag_of(p);
   if (xq) {  // FP64 contexts: the fixed-point kernel's record
     XFix q;
-    const int F = gr.rep[MD_TAG_REP(tag)].xfix;
-    const bool on = md_xfix(p.x, F, q.x) & md_xfix(p.y, F, q.y) & md_xfix(p.z, F, q.z);
-    if (!on) q.x = q.y = q.z = 1LL << 62;  // farther than 2^61 from every position
+    const RepGeo& g = gr.rep[MD_TAG_REP(tag)];
+    const int F = g.xfix;
+    const bool on = md_xfix_centred(p.x, F, g.hx[0], q.x) & md_xfix_centred(p.y, F, g.hx[1], q.y) &
+                    md_xfix_centred(p.z, F, g.hx[2], q.z);
+    if (!on) q.x = q.y = q.z = MD_XFIX_OFF;
     q.w = (long long)(unsigned int)(on ? tag : tag | MD_TAG_OFFGRID) | ((long long)F << 32);
     xq[i] = q;
   }

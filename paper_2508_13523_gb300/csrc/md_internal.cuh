@@ -75,8 +75,7 @@ struct RepGeo {
   int nb[3];                // 4x4x4-cell bricks along each axis: ceil(nc / 4)
   int lo[3], hi[3];         // stencil offsets along each axis (-1..1 or 0..0)
   int cell_base;            // first global cell of this replica
-  int xfix;                 // fixed-point scale F of its positions (XFix): 61 - E
-                            // with 2^E >= 1.25 x the largest edge
+  int xfix;                 // fixed-point scale F of its positions (XFix)
   // fixed-point kernel (md_pair_fx.cuh), all in units of 2^-xfix:
   long long Lx[3], hx[3];   // L and L / 2, rounded down
   int gh;                   // min(2^R, L / 2 over the axes) >> 32: separations whose
@@ -127,21 +126,24 @@ struct __align__(32) XSplit {
 #define MD_TAG(type, rep) ((int)(type) | ((int)(rep) << 8))
 #define MD_TAG_TYPE(tag) ((tag) & 0x7f)
 #define MD_TAG_REP(tag) ((tag) >> 8)
-// Set in the tag of xs (XSplit hi.w) only: some coordinate of the atom is
-// not a multiple of 2^-F of its box (or too large), so its pairs take the
-// FP64 path of the fixed-point kernel (XFix).
+// Set in the tag of an XFix record (XFix::w) only: some coordinate of the atom
+// has no fixed-point form, so its pairs take the FP64 path of the fixed-point
+// kernel.
 #define MD_TAG_OFFGRID 0x80
 
-// Positions as fixed-point integers X = x 2^F with F = RepGeo::xfix of the
-// atom's box (F = 61 - E, 2^E >= 1.25 x the box's largest edge: 53 for a
-// 168-wide box).  X is exact for every double with 2^(52 - F) <= |x| < 2^E
-// (all of them are multiples of 2^-F: from 0.5 up in a 168-wide box), and
-// for smaller x whose low significand bits happen to be zero; any other
-// atom is flagged (MD_TAG_OFFGRID).  The difference X_j - X_i is then the
-// exact separation x_j - x_i (which the FP64 subtraction also yields
-// exactly here), below 2^60 in magnitude for pairs closer than half the
-// box: the fixed-point kernel (md_pair_fx.cuh) forms separations, r^2 and the
-// force from it with integer instructions.
+// Positions as fixed-point integers, counted from the box's centre: X = x 2^F -
+// L 2^(F-1) with F = RepGeo::xfix of the atom's box (54 for a 168-wide one).
+// x 2^F is exact for |x| >= 2^(52 - F) (from 0.25 up in a 168-wide box).  Smaller x
+// are rounded to the nearest multiple of 2^-F, an error of at most 2^-(F + 1), where
+// F >= MD_XFIX_ROUND_F (edges up to 1,173); with a coarser grid an atom with a
+// coordinate that is no multiple of it is flagged (MD_TAG_OFFGRID), as is one
+// farther than MD_XFIX_MAX from the centre.  The difference of two X is the
+// separation x_j - x_i, exact but for those roundings (FP64's own subtraction
+// rounds separations by as much): the fixed-point kernel (md_pair_fx.cuh) forms
+// separations, r^2 and the force from it with integer instructions.
+#define MD_XFIX_ROUND_F 52
+#define MD_XFIX_MAX (11LL << 58)
+#define MD_XFIX_OFF (21LL << 58)  // an atom without X: farther from every X than half a box
 struct __align__(32) XFix {
   long long x, y, z;
   long long w;  // the atom's tag (as md_tag_of(x4)) | F << 32
@@ -233,8 +235,8 @@ struct md_ctx {
   XSplit* xs;       // double-float split of x4 (build filter, mixed gathers); FP64
                     // contexts: the hi parts alone, one float4 an atom (md_ld_hi)
   XSplit* xb;       // the same of the positions at the last build (displacement)
-  XFix* xq;         // FP64 contexts: fixed-point positions (valid where xs's tag has no
-                    // MD_TAG_OFFGRID); NULL for mixed precision
+  XFix* xq;         // FP64 contexts: fixed-point positions (valid where the record's tag
+                    // has no MD_TAG_OFFGRID); NULL for mixed precision
   int32_t* cell;    // global cell index of each sorted atom
   int32_t* tag0;    // tags in the caller's order
   PairCoef* coef;   // nt*nt coefficients (device)

@@ -2,7 +2,7 @@
 // 2508.13523, Eq. 1 and Sec. 4; Sec. 4.1: half list with reductions, full
 // list, T threads per atom).
 //
-// Positions are 64-bit fixed-point numbers (XFix), separations their exact
+// Positions are 64-bit fixed-point numbers (XFix), separations their
 // differences, Eq. 1's force is evaluated in 64-bit fixed point (md_fx.cuh)
 // and every contribution is a 2^-44 count summed exactly in 64-bit integers:
 // the owner's share in registers, f_j's (half list) by global integer
@@ -170,7 +170,7 @@ __device__ __forceinline__ void md_pair_fx_tiles(const PairArgs& a, const float 
     const int tag = (int)own.w;
     const RepGeo* g = a.rep + MD_TAG_REP(tag);
     const int sh0 = 63 - a.fxR - (int)(own.w >> 32);  // D to A
-    const int gh = g->gh;
+    const unsigned gh = (unsigned)g->gh;
     long long ax = 0, ay = 0, az = 0;  // counts for the partners (owner: minus)
     unsigned long long s6 = 0;         // one type: sum x^3 2^(62 - ev_shift)
     double e0 = 0.0;                   // several types: energy; one type: r^-6 of FP64 pairs
@@ -208,9 +208,8 @@ __device__ __forceinline__ void md_pair_fx_tiles(const PairArgs& a, const float 
       int shf = 0;  // EV: image shifts taken off d, 2 bits per axis (+L: 1, -L: 2)
       // |D| beyond 2^(R + F) or half the box on some axis: a periodic image
       // may be nearer (rare: only pairs across the boundary)
-      if (((unsigned)((int)(Dx >> 32) + gh) >= 2u * gh) |
-          ((unsigned)((int)(Dy >> 32) + gh) >= 2u * gh) |
-          ((unsigned)((int)(Dz >> 32) + gh) >= 2u * gh)) {
+      auto far = [&](long long D) { return (unsigned)(int)(D >> 32) + gh >= 2u * gh; };
+      if (far(Dx) | far(Dy) | far(Dz)) {
         // (x_j - x_i is rounded to FP64's 53 bits before the edge is taken
         // off, as the FP64 separation is)
         auto image = [&](long long& D, int k) {
