@@ -37,6 +37,7 @@ N_CELLS = 100  # 4 * 100^3 = 4,000,000 atoms
 HBM_PEAK_FALLBACK = 6800.0
 SM_COUNT = 152
 FP64_OPS_PER_CLK_SM = 2  # FP64 pipe lane-ops per clock per SM (1.25 TFLOP/s nominal)
+MADD_PER_CLK_SM = 64  # 32 x 32 + 64-bit multiply-adds (a loop of independent ones: 57)
 
 # DRAM bytes (read + write) per atom of one pair-kernel launch from 1-pass
 # ncu captures at 4,000,000 atoms (commands and figures under profiles/),
@@ -182,15 +183,22 @@ def fp64_ops_per_pair(compacted: int, coul: bool = False) -> int:
     With floating-point separations (per-atom kernel, compacted kernel with
     FP64 sums): separation 3, squared length 3, reciprocal refinement 3,
     r^-6 2, fpair 3, fpair * d 3 = 17 (the accumulations are reductions in
-    L2, off the pipe).  With exact fixed-point separations, r^2 and fpair * d
-    the rest is reciprocal 3, r^-6 2, fpair 3 = 8: the count that the
-    fixed-point kernel (compacted 2) is rated with, although it evaluates these
-    with integer instructions too and leaves the FP64 pipe idle.  The
+    L2, off the pipe).  The fixed-point kernel (compacted 2) has none; its count,
+    8, is the force's own (reciprocal 3, r^-6 2, fpair 3), for comparison with
+    the others at equal work (madds_per_pair is what it does).  The
     lj/cut/coul/cut form with FP64 arithmetic takes 22 (reciprocal square root
     5, r^-2 1, qq/r 1, one FMA, instead of the reciprocal's 3)."""
     if coul:
         return 22
     return 8 if compacted == 2 else 17
+
+
+def madds_per_pair(coul: bool = False) -> int:
+    """32 x 32 + 64-bit multiply-adds of the fixed-point kernel (compacted 2) per
+    visit of a pair inside rc, one type: r^2 6, reciprocal 4, five 64-bit high
+    products of 3, three counts of 3.  lj/cut/coul/cut: r^2 6, reciprocal square
+    root 6, its square 3, tau 3, the force 15, the Coulomb term 6, counts 9."""
+    return 48 if coul else 34
 
 
 def pair_work(kind: str, prec: str, n: int, entries: int, pairs: int, compacted: int = 0,
@@ -729,6 +737,7 @@ def main():
     md.load(build_if_missing=False)
     hbm_peak, sm_max, peak_src = peaks()
     fp64_peak = FP64_OPS_PER_CLK_SM * SM_COUNT * sm_max * 1e6 / 1e9  # Gop/s
+    madd_peak = MADD_PER_CLK_SM * SM_COUNT * sm_max * 1e6 / 1e9
 
     sysm = S.fcc_liquid(args.cells)
     n = sysm.n
@@ -800,15 +809,23 @@ def main():
     label = {0: f"k_pair<{prec},{kind},TPA={h['tpa']}>",
              1: f"k_pair_q<{kind}> (warp-compacted, FP64 force sums)",
              2: f"k_pair_fx<{kind}> (fixed-point pair force and sums)"}[h["compacted"]]
-    if prec == "fp64":
+    if prec == "fp64" and int(h["compacted"]) == 2:  # no FP64 operation per pair
+        achieved = madds_per_pair() * (1 if kind == "half" else 2) * h["pairs"] / (kern_ms * 1e6)
+        roofline = {"bound": "alu", "achieved": achieved, "peak": madd_peak,
+                    "unit": "Gop/s (32 x 32 + 64-bit multiply-adds)",
+                    "frac": achieved / madd_peak,
+                    "peak_source": "64 multiply-adds/clk/SM x 152 SMs x max SM clock; a loop of "
+                                   "independent ones measured at 17,840 Gop/s",
+                    "ops_per_pair_visit": madds_per_pair(),
+                    "ops_note": "the products of the pair force alone: shifts, adds and "
+                                "address arithmetic share their pipe, and issue and L1 are "
+                                "as busy (no unit binds alone)"}
+    elif prec == "fp64":
         roofline = {"bound": "alu", "achieved": achieved_ops, "peak": fp64_peak,
                     "unit": "Gop/s (FP64 pipe)", "frac": achieved_ops / fp64_peak,
                     "peak_source": "2 FP64 lane-ops/clk/SM x 152 SMs x max SM clock (1.25 "
                                    "TFLOP/s nominal); DFMA measured at 628 Gop/s",
                     "ops_per_pair_visit": fp64_ops_per_pair(int(h["compacted"]))}
-        if int(h["compacted"]) == 2:
-            roofline["ops_note"] = ("the FP64 operations that the pair force needs beside exact "
-                                    "separations; k_pair_fx does them with integer instructions")
     else:  # the mixed form issues no FP64 operation per pair: HBM is its roof
         roofline = {"bound": "hbm", "achieved": achieved_gbs, "peak": hbm_peak, "unit": "GB/s",
                     "frac": achieved_gbs / hbm_peak, "peak_source": peak_src}
@@ -861,11 +878,16 @@ def main():
              "energy_drift_per_atom_step": r["energy_drift"]}
         if p == "mixed":
             f["force_err_vs_fp64"] = mixed_force_error(md, r["ctx"], style == ["coul"])
-        if p == "fp64":
+        coul = style == ["coul"]
+        if p == "fp64" and r["compacted"] == 2:
+            f["madds_per_pair_visit"] = madds_per_pair(coul)
+            f["pair_kernel_madd_frac"] = (madds_per_pair(coul) * (1 if k == "half" else 2)
+                                          * r["pairs"] / (r["pair_ms"] * 1e6) / madd_peak)
+        elif p == "fp64":
             f["pair_kernel_fp64_gops"] = o / (r["pair_ms"] * 1e-3) / 1e9
-        if style == ["coul"]:
+            f["ops_per_pair_visit"] = fp64_ops_per_pair(int(r["compacted"]), coul)
+        if coul:
             f["pair_style"] = "lj/cut/coul/cut, charges +-0.5 by fcc site, rc_coul 2.5"
-            f["ops_per_pair_visit"] = 22
         forms_out[name] = f
 
     if drift is not None:
