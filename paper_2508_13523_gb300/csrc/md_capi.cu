@@ -388,7 +388,6 @@ PairArgs pair_args(md_ctx* c) {
   a.fxt = c->fxt;
   a.fx1 = c->fx1;
   a.fxR = c->fxR;
-  a.nrep = c->nrep;
   // one type: at most maxneigh + 64 terms x^3 2^62 < 2^62 in 64 bits
   a.ev_shift = 0;
   while (a.ev_shift < 32 && (int64_t)c->maxneigh + 64 > (4LL << a.ev_shift)) a.ev_shift++;
@@ -792,7 +791,7 @@ int launch_pair_impl(md_ctx* c, int ev, int tpa, int prezeroed, int defer_fold,
     cudaStream_t s = c->stream;
     const int t = fx_lanes(c);
     cudaError_t e =
-        fix ? (c->coul ? md_pair_fx_coul_launch(a, half, ev != 0, t, 2, cut1, cut, s, c->carve)
+        fix ? (c->coul ? md_pair_fx_coul_launch(a, half, ev != 0, t, cut1, cut, s, c->carve)
                        : md_pair_fx_launch(a, half, ev != 0, fx_single(c), t, c->qu, cut1, cut, s,
                                            c->carve))
             : (c->coul

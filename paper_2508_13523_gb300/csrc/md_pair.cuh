@@ -61,7 +61,6 @@ struct PairArgs {
   const PairFx* fxt;     // the fixed-point kernel's nt*nt table
   PairFx fx1;            // and its only entry when nt == 1
   int fxR;               // largest cutoff <= 2^fxR
-  int nrep;
   int ev_shift;          // one type: sums of x^3 (md_fx_force1) in units of 2^(ev_shift - 62)
   PairCoef c1;           // the only coefficients when nt == 1
   const RepGeo* rep;     // box of each replica

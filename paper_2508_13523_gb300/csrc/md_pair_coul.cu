@@ -13,13 +13,13 @@ cudaError_t md_pair_q_coul_launch(const PairArgs& a, bool half, bool ev, bool si
   return md_pair_q_launch_t<true>(a, half, ev, single, cut1, cut_tab, blocks, s, carve);
 }
 
-cudaError_t md_pair_fx_coul_launch(const PairArgs& a, bool half, bool ev, int t, int u,
-                                   float cut1, const float* cut_tab, cudaStream_t s, int carve) {
+cudaError_t md_pair_fx_coul_launch(const PairArgs& a, bool half, bool ev, int t, float cut1,
+                                   const float* cut_tab, cudaStream_t s, int carve) {
   if (half)
-    return ev ? md_pair_fx_launch_t<true, true, false, true>(a, t, u, cut1, cut_tab, s, carve)
-              : md_pair_fx_launch_t<true, false, false, true>(a, t, u, cut1, cut_tab, s, carve);
-  return ev ? md_pair_fx_launch_t<false, true, false, true>(a, t, u, cut1, cut_tab, s, carve)
-            : md_pair_fx_launch_t<false, false, false, true>(a, t, u, cut1, cut_tab, s, carve);
+    return ev ? md_pair_fx_launch_u<true, true, false, true, 2>(a, t, cut1, cut_tab, s, carve)
+              : md_pair_fx_launch_u<true, false, false, true, 2>(a, t, cut1, cut_tab, s, carve);
+  return ev ? md_pair_fx_launch_u<false, true, false, true, 2>(a, t, cut1, cut_tab, s, carve)
+            : md_pair_fx_launch_u<false, false, false, true, 2>(a, t, cut1, cut_tab, s, carve);
 }
 
 template <bool HALF, bool EV, bool SINGLE>

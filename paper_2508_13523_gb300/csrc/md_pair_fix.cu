@@ -5,16 +5,9 @@
 
 cudaError_t md_pair_fx_launch(const PairArgs& a, bool half, bool ev, bool single, int t, int u,
                               float cut1, const float* cut_tab, cudaStream_t s, int carve) {
-  if (half) {
-    if (ev)
-      return single ? md_pair_fx_launch_t<true, true, true, false>(a, t, u, cut1, cut_tab, s, carve)
-                    : md_pair_fx_launch_t<true, true, false, false>(a, t, u, cut1, cut_tab, s, carve);
-    return single ? md_pair_fx_launch_t<true, false, true, false>(a, t, u, cut1, cut_tab, s, carve)
-                  : md_pair_fx_launch_t<true, false, false, false>(a, t, u, cut1, cut_tab, s, carve);
-  }
-  if (ev)
-    return single ? md_pair_fx_launch_t<false, true, true, false>(a, t, u, cut1, cut_tab, s, carve)
-                  : md_pair_fx_launch_t<false, true, false, false>(a, t, u, cut1, cut_tab, s, carve);
-  return single ? md_pair_fx_launch_t<false, false, true, false>(a, t, u, cut1, cut_tab, s, carve)
-                : md_pair_fx_launch_t<false, false, false, false>(a, t, u, cut1, cut_tab, s, carve);
+  if (half)
+    return single ? md_pair_fx_launch_t<true, true>(a, ev, t, u, cut1, cut_tab, s, carve)
+                  : md_pair_fx_launch_t<true, false>(a, ev, t, u, cut1, cut_tab, s, carve);
+  return single ? md_pair_fx_launch_t<false, true>(a, ev, t, u, cut1, cut_tab, s, carve)
+                : md_pair_fx_launch_t<false, false>(a, ev, t, u, cut1, cut_tab, s, carve);
 }

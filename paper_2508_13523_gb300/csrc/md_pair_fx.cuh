@@ -432,32 +432,29 @@ cudaError_t md_pair_fx_launch1(const PairArgs& a, float cut1, const float* cut_t
   return cudaGetLastError();
 }
 
-template <bool HALF, bool EV, bool SINGLE, bool COUL>
-cudaError_t md_pair_fx_launch_t(const PairArgs& a, int t, int u, float cut1,
-                                const float* cut_tab, cudaStream_t s, int carve) {
-  constexpr int U1 = EV ? 2 : 1;
-  if (u == 1) {
-    switch (t) {
-      case 1: return md_pair_fx_launch1<HALF, EV, SINGLE, COUL, 1, U1>(a, cut1, cut_tab, s, carve);
-      case 2: return md_pair_fx_launch1<HALF, EV, SINGLE, COUL, 2, U1>(a, cut1, cut_tab, s, carve);
-      case 4: return md_pair_fx_launch1<HALF, EV, SINGLE, COUL, 4, U1>(a, cut1, cut_tab, s, carve);
-      case 8: return md_pair_fx_launch1<HALF, EV, SINGLE, COUL, 8, U1>(a, cut1, cut_tab, s, carve);
-      default: return cudaErrorInvalidValue;
-    }
-  }
+template <bool HALF, bool EV, bool SINGLE, bool COUL, int U>
+cudaError_t md_pair_fx_launch_u(const PairArgs& a, int t, float cut1, const float* cut_tab,
+                                cudaStream_t s, int carve) {
   switch (t) {
-    case 1: return md_pair_fx_launch1<HALF, EV, SINGLE, COUL, 1, 2>(a, cut1, cut_tab, s, carve);
-    case 2: return md_pair_fx_launch1<HALF, EV, SINGLE, COUL, 2, 2>(a, cut1, cut_tab, s, carve);
-    case 4: return md_pair_fx_launch1<HALF, EV, SINGLE, COUL, 4, 2>(a, cut1, cut_tab, s, carve);
-    case 8: return md_pair_fx_launch1<HALF, EV, SINGLE, COUL, 8, 2>(a, cut1, cut_tab, s, carve);
+    case 2: return md_pair_fx_launch1<HALF, EV, SINGLE, COUL, 2, U>(a, cut1, cut_tab, s, carve);
+    case 4: return md_pair_fx_launch1<HALF, EV, SINGLE, COUL, 4, U>(a, cut1, cut_tab, s, carve);
+    case 8: return md_pair_fx_launch1<HALF, EV, SINGLE, COUL, 8, U>(a, cut1, cut_tab, s, carve);
     default: return cudaErrorInvalidValue;
   }
 }
 
-// t: lanes per atom (1, 2, 4 or 8); u: skin entries per round (1 or 2; 2 with
-// energy and virial)
+template <bool HALF, bool SINGLE>
+cudaError_t md_pair_fx_launch_t(const PairArgs& a, bool ev, int t, int u, float cut1,
+                                const float* cut_tab, cudaStream_t s, int carve) {
+  if (ev) return md_pair_fx_launch_u<HALF, true, SINGLE, false, 2>(a, t, cut1, cut_tab, s, carve);
+  return u == 1 ? md_pair_fx_launch_u<HALF, false, SINGLE, false, 1>(a, t, cut1, cut_tab, s, carve)
+                : md_pair_fx_launch_u<HALF, false, SINGLE, false, 2>(a, t, cut1, cut_tab, s, carve);
+}
+
+// t: lanes per atom (2, 4 or 8); u: skin entries per round of a force-only
+// launch (1 or 2; 2 with energy and virial)
 cudaError_t md_pair_fx_launch(const PairArgs& a, bool half, bool ev, bool single, int t, int u,
                               float cut1, const float* cut_tab, cudaStream_t s, int carve);
-// lj/cut/coul/cut (md_pair_coul.cu)
-cudaError_t md_pair_fx_coul_launch(const PairArgs& a, bool half, bool ev, int t, int u,
-                                   float cut1, const float* cut_tab, cudaStream_t s, int carve);
+// lj/cut/coul/cut (md_pair_coul.cu): two skin entries per round
+cudaError_t md_pair_fx_coul_launch(const PairArgs& a, bool half, bool ev, int t, float cut1,
+                                   const float* cut_tab, cudaStream_t s, int carve);

@@ -399,7 +399,12 @@ cudaError_t md_vjp_launch_tpa(const VjpArgs& a, int tpa, unsigned blocks, cudaSt
   const size_t smem = md_vjp_smem(SINGLE, a.nt);
   switch (tpa) {
     case 2: k_vjp<PREC, HALF, 2, SINGLE><<<blocks, MD_BLOCK, smem, s>>>(a); break;
-    case 4: k_vjp<PREC, HALF, 4, SINGLE><<<blocks, MD_BLOCK, smem, s>>>(a); break;
+    case 4:  // FP64 alone (vjp_lanes)
+      if constexpr (PREC == MD_PREC_FP64)
+        k_vjp<PREC, HALF, 4, SINGLE><<<blocks, MD_BLOCK, smem, s>>>(a);
+      else
+        return cudaErrorInvalidValue;
+      break;
     case 8: k_vjp<PREC, HALF, 8, SINGLE><<<blocks, MD_BLOCK, smem, s>>>(a); break;
     default: return cudaErrorInvalidValue;
   }
