@@ -96,8 +96,9 @@ typedef struct md_params {
                                displacement check is reported, as "dangerous
                                builds"); 1: also rebuild before any step at
                                which some atom has moved more than skin/2
-                               since the last build (checked after every
-                               drift; one host synchronization per step)      */
+                               since the last build (checked on the device
+                               after every drift; one host synchronization
+                               per 16 steps or rebuild)                       */
 } md_params;
 
 typedef struct md_ctx md_ctx;
@@ -116,7 +117,9 @@ typedef struct md_stats {
   int32_t max_neigh;        /* current capacity per atom                       */
   int32_t max_count;        /* largest per-atom count at the last build        */
   int32_t cells[3];         /* cell grid (1 along an axis too short for 3)     */
-  int32_t threads_per_atom; /* in use                                          */
+  int32_t threads_per_atom; /* of the per-atom kernel, as tuned or set; 1 with
+                               compacted (the fixed-point kernel takes 2, 4 or
+                               8 lanes per atom by the number of atoms)       */
   int32_t carveout;         /* preferred shared-memory carveout of the pair
                                kernel in percent, -1 = driver default         */
   int32_t compacted;        /* FP64: 0 per-atom pair kernel, 1 warp-compacted
@@ -133,10 +136,10 @@ typedef struct md_stats {
   int32_t coulomb;          /* 1 if the lj/cut/coul/cut style is on (md_set_coulomb) */
   int32_t phase1_entries;   /* list entries each lane takes per round of the
                                force-only pair kernel's walk: 1 or 2 for the
-                               FP64 compacted fixed-point kernel (picked by
-                               md_autotune or md_set_kernel), 2 for the mixed
-                               kernel (its half list; the full list's walk
-                               takes three), 1 for the others                 */
+                               FP64 fixed-point kernel (picked by md_autotune
+                               or md_set_kernel; the Coulomb style always
+                               takes 2), 2 for the mixed kernel (its half list;
+                               the full list's walk takes 3), 1 for the others */
 } md_stats;
 
 /* ---- single box ---------------------------------------------------------- */
@@ -302,9 +305,11 @@ int md_set_coulomb(md_ctx* ctx, const double* q, double rc_coul, double qqrd2e);
  * Eq. 1's force in 64-bit integers, each force contribution rounded to a
  * multiple of 2^-44 and summed exactly (the result does not depend on the
  * order of the additions; every contribution lies within a count, 2^-44, and
- * a few FP64 ulps of its exact value; pairs that the integers do not cover,
- * among them contributions too large for the sums, are evaluated and added in
- * FP64), compacted 3 the compacted 2 kernel whose
+ * a few FP64 ulps of its exact value; coordinates below 2^-2 to 1, by the box's
+ * size up to an edge of 1,173, are rounded by at most 2^-53, as an FP64
+ * separation above 1 is; pairs that the integers do not cover, among them
+ * contributions too large for the sums, 2^8 or less on very dense lists, and
+ * atoms in longer boxes near a face, are evaluated and added in FP64), compacted 3 the compacted 2 kernel whose
  * filter takes two list entries per lane per round, their loads in flight
  * together (Eq. 1 alone; md_get_stats then reports compacted 2 and
  * phase1_entries 2); persistent 1 launches one
@@ -366,7 +371,9 @@ int md_set_lj(md_ctx* ctx, const double* eps, const double* sigma);
  *   gbar: host, 2 n_types^2, receives dL/deps then dL/dsigma as symmetric
  *         tables: entries (a,b) and (b,a) both hold the derivative with
  *         respect to the one parameter of the unordered type pair {a,b}.
- * The cutoffs are constants.  FP64 or mixed precision as the context.
+ * The cutoffs are constants.  FP64 or mixed precision as the context (mixed:
+ * pair terms in FP32, the cotangent rounded to it; each thread's parameter
+ * terms summed as FP32 value and rounding error, everything else in FP64).
  * Synchronizes. */
 int md_force_vjp(md_ctx* ctx, const double* cot, double* xbar, double* gbar);
 

@@ -441,9 +441,8 @@ class LJMD:
 
     def set_kernel(self, threads_per_atom=1, carveout=-1, compacted=0, persistent=1):
         """md_set_kernel: fix the pair kernel's configuration (compacted: 0
-        per-atom loop, 1 warp-compacted with FP64 force sums, 2 warp-compacted
-        with exact fixed-point force sums, 3 the same with two list entries per
-        lane per filter round)."""
+        per-atom loop, 1 warp-compacted with FP64 force sums, 2 the fixed-point
+        kernel, 3 the same with two list entries per lane per filter round)."""
         _check(self._lib.md_set_kernel(self._ctx, int(threads_per_atom), int(carveout),
                                        int(compacted), int(persistent)), "md_set_kernel")
 

@@ -150,9 +150,10 @@ int setup_geometry(md_ctx* c, const double* boxes) {
       g.hi[a] = g.nc[a] >= 3 ? 1 : 0;
       ncr *= 4 * g.nb[a];  // brick order pads each axis to a multiple of 4
       // |(|d_f| - |d|)| per component: position rounding (|x - hi| <= u P
-      // for each of the two atoms; the subtraction of hi parts and the image
-      // shift are exact), and a different image choice near |d| = L/2
-      // (<= 5 u L); u (2 P + 10 L) covers them.
+      // for each of the two atoms; the subtraction of hi parts is exact), the
+      // image shift (Lf for L: u L; where it is added to a position first,
+      // k_build_cell, the sum below 2 L rounds by u 2 L) and a different image
+      // choice near |d| = L/2 (<= 5 u L); u (2 P + 10 L) covers them.
       const double ea = u * (2.0 * P + 10.0 * L);
       e2 += ea * ea;
     }
@@ -182,8 +183,8 @@ int setup_geometry(md_ctx* c, const double* boxes) {
 }  // namespace
 
 // The force cutoff of each type pair (the larger of rc and, with the
-// Coulomb term, rc_coul): the build's inner/skin split and the compacted
-// kernel's certified FP32 upper bound of it.
+// Coulomb term, rc_coul): the build's inner/skin split and the FP64
+// kernels' certified FP32 upper bound of it.
 static void set_cut_bounds(md_ctx* c) {
   const double u = ldexp(1.0, -24), e = c->filt_e;
   Geo& gg = c->geo;
@@ -246,7 +247,7 @@ int md_upload_fx(md_ctx* c) {
 }
 
 // Coefficient table (device), the single-type copy, and the FP32 cutoff
-// bounds (device copy for the compacted kernel).  Synchronizes: the host
+// bounds (device copy for the FP64 kernels).  Synchronizes: the host
 // table must outlive the copies.
 int md_upload_coef(md_ctx* c) {
   const int nt = c->nt;
@@ -410,7 +411,8 @@ bool fx_single(const md_ctx* c) { return c->nt == 1 && c->fx1.B <= MD_FX_BMAX; }
 
 // Lanes per atom of the fixed-point kernel.  Few atoms: more lanes shorten
 // each lane's chain of dependent loads and fill the SMs; many atoms: two lanes
-// share a row's tail (1, 2, 4 and 8 lanes, force-only half list: 4,000 atoms
+// share a row's tail (1, 2, 4 and 8 lanes, force-only half list, md_compute_forces
+// alone, with its fold: 4,000 atoms
 // 38, 24, 17 and 14 us; 32,000 atoms 42, 31, 27 and 27 us; 108,000 atoms 68,
 // 62, 60 and 64 us; 256,000 atoms 134, 117, 122 and 138 us; 4,000,000 atoms
 // 1.470, 1.464, 1.70 and 2.00 ms).
@@ -1054,12 +1056,12 @@ int md_get_neighbors(md_ctx* c, int64_t* offsets, int32_t* idx) {
 int md_autotune(md_ctx* c) {
   if (!c) return MD_EINVAL;
   // threads per atom (Sec. 4.1: parallelism over neighbors) and, in FP64,
-  // the warp-compacted kernel with FP64 or fixed-point reductions, each with
-  // one block per tile and then with persistent per-SM tile scheduling, and
-  // for the fixed-point kernel (Eq. 1 alone) one or two list entries per
-  // lane per round of its filter; driver-default carveout (a largest-L1 carveout was measured slower or
-  // equal for every configuration on GB300 and stays available through
-  // md_set_kernel, as does the one-launch-per-step schedule)
+  // the warp-compacted kernel and the fixed-point kernel, each with one block
+  // per tile and then with persistent per-SM tile scheduling, and for the
+  // fixed-point kernel (Eq. 1 alone) one or two list entries per lane per round
+  // of its filter; driver-default carveout (a largest-L1 carveout was measured
+  // slower or equal for every configuration on GB300 and stays available
+  // through md_set_kernel, as does the one-launch-per-step schedule)
   static const int cand[] = {1, 2, 4, 8, 16, 32};
   cudaEvent_t e0, e1;
   MD_CUDA(cudaEventCreate(&e0));
@@ -1070,7 +1072,7 @@ int md_autotune(md_ctx* c) {
   int rc = MD_OK;
   c->carve = -1;
   const int ncompact = c->precision == MD_PREC_FP64 ? 3 : 1;
-  // the Coulomb style exists as the compacted FP64 kernel and as the mixed
+  // the Coulomb style exists as the compacted and fixed-point kernels and as the mixed
   // kernel at 1, 2 or 4 threads per atom
   const int cp0 = (c->coul && c->precision == MD_PREC_FP64) ? 1 : 0;
   const int ntpa = c->coul ? 3 : 6;

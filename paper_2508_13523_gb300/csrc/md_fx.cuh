@@ -19,7 +19,7 @@
 // same formula in FP64 (rms over r uniform in 0.82 .. 2.5, random directions:
 // 0.58 against 0.82 units of 2^-44).
 // Pairs outside these ranges (closer than 0.816 sigma, forces beyond the
-// accumulators' range, within a band around a cutoff, positions without a
+// accumulators' range, md_fx_dense, within a band around a cutoff, positions without a
 // fixed-point form) are evaluated in FP64 by the caller.
 #pragma once
 

@@ -191,8 +191,8 @@ struct md_ctx {
                            // around every pair launch
   cudaEvent_t* pair_ev;    // 2 * MD_PAIR_TIMING_MAX events (start, stop), or NULL
   int pair_ev_used;        // event pairs recorded since the last enable
-  int qu;       // list entries per phase-1 round of the force-only compacted
-                // fixed-point kernel (1 or 2; md_autotune picks it)
+  int qu;       // skin entries per round of the force-only fixed-point kernel
+                // (1 or 2; md_autotune picks it)
   int persist;  // 1 = persistent per-SM tile scheduling of the pair kernel;
                 // 2 = the same, and one cooperative launch per step (kick,
                 // drift and forces; md_step_fused.cu)
