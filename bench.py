@@ -50,11 +50,11 @@ PAIR_SOURCES = ("paper_2508_13523_gb300/csrc/md_pair.cuh",
                 "paper_2508_13523_gb300/csrc/md_pair_fx.cuh",
                 "paper_2508_13523_gb300/csrc/md_fx.cuh",
                 "paper_2508_13523_gb300/csrc/md_device.cuh")
-PAIR_TRAFFIC = {"5f6b6b44cb86c0f0": {
-    "fp64_half/2/1/2": (1144426496 + 85809408) / 4.0e6,
-    "fp64_full/2/1/2": (1544429568 + 80557568) / 4.0e6,
-    "mixed_half/0/2/2": (1121923072 + 82675968) / 4.0e6,
-    "mixed_full/0/2/2": (1416501248 + 75228416) / 4.0e6}}
+PAIR_TRAFFIC = {"c804166656110a0e": {
+    "fp64_half/2/1/2": (1144646656 + 85815040) / 4.0e6,
+    "fp64_full/2/1/2": (1544428288 + 80500480) / 4.0e6,
+    "mixed_half/0/2/2": (1123662336 + 82505472) / 4.0e6,
+    "mixed_full/0/2/2": (1417366784 + 75100928) / 4.0e6}}
 
 
 def pair_source_hash() -> str:
