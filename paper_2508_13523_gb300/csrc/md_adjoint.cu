@@ -395,20 +395,26 @@ int md_traj_vjp(md_ctx* c, int64_t nsteps, int32_t every, const double* ckpt_x,
   MD_CUDA(cudaMemsetAsync(c->gbar, 0, gbar_bytes(c), c->stream));
   DtfArgs d;
   for (int t = 0; t < MD_MAX_TYPES; t++) d.dtf[t] = c->dtf[t];
-  for (int64_t j = J; j >= 0; j--) {
+  // Segments in reverse; one whose list a displacement rebuilds on the way
+  // (check_disp) goes in parts, each with the list and order of its positions:
+  // hi is the last evaluation not yet differentiated
+  int64_t hi = nsteps;
+  for (int64_t j = J; j >= 0;) {
     const int64_t s0 = j * every < nsteps ? j * every : nsteps;
-    const int64_t e_hi = (j == J) ? nsteps : ((j + 1) * every < nsteps ? (j + 1) * every : nsteps) - 1;
     // recompute the segment's positions from its checkpoint
     MD_TRY(md_set_state(c, ckpt_x + j * n3, ckpt_v + j * n3, MD_MEM_DEVICE));
-    const int64_t npos = e_hi - s0 + 1;
+    const int64_t npos = hi - s0 + 1;
     MD_CUDA(cudaMemcpyAsync(c->seg_x, c->x4, sizeof(double4_32a) * n, cudaMemcpyDeviceToDevice,
                             c->stream));
-    // (no rebuild falls inside: the segment is shorter than the cadence; the
+    // (no other rebuild falls inside: the segment is shorter than the cadence; the
     // forces at its last position are not needed)
     const int fold = md_pair_fixed(c), zero = md_pair_accumulates(c);
+    int64_t lo = s0;  // the first position in the current list's order
     for (int64_t k = 1; k < npos; k++) {
       if (c->check_disp) {
+        const int64_t builds = c->builds;
         MD_TRY(md_step(c, 1));
+        if (c->builds != builds) lo = s0 + k;
       } else {
         if (k > 1) MD_TRY(md_launch_pair_step(c));
         MD_TRY(md_launch_integrate(c, k > 1 ? MD_K21 : MD_K1, k > 1 ? fold : 0, zero));
@@ -420,13 +426,13 @@ int md_traj_vjp(md_ctx* c, int64_t nsteps, int32_t every, const double* ckpt_x,
     MD_TRY(to_sorted(c, XB, c->adj_xbar, nullptr));
     MD_TRY(to_sorted(c, VB, c->adj_vbar, nullptr));
     MD_TRY(to_sorted(c, CC, nullptr, c->adj_c));
-    // the positions are those of e_hi here
-    for (int64_t e = e_hi; e >= s0; e--) {
+    // the positions are those of hi here
+    for (int64_t e = hi; e >= lo; e--) {
       MD_TRY(launch_vjp(c));
       if (e == 0) break;
       const double mult = (e - 1 >= 1) ? 2.0 : 1.0;
       k_adj_step<<<(unsigned)md_blocks(n), MD_BLOCK, 0, c->stream>>>(
-          e > s0 ? c->seg_x + (e - 1 - s0) * n : nullptr, c->x4, c->xs, c->xq, c->xgrid,
+          e > lo ? c->seg_x + (e - 1 - s0) * n : nullptr, c->x4, c->xs, c->xq, c->xgrid,
           c->adj_xbar, c->adj_vbar, c->adj_c, c->adj_cf, n, c->dt, mult, d);
       c->launches++;
       MD_CUDA(cudaGetLastError());
@@ -434,6 +440,8 @@ int md_traj_vjp(md_ctx* c, int64_t nsteps, int32_t every, const double* ckpt_x,
     MD_TRY(to_caller(c, c->adj_xbar, nullptr, XB));
     MD_TRY(to_caller(c, c->adj_vbar, nullptr, VB));
     MD_TRY(to_caller(c, nullptr, c->adj_c, CC));
+    hi = lo - 1;
+    if (lo == s0) j--;
   }
   MD_CUDA(cudaMemcpyAsync(x0bar, XB, sizeof(double) * n3, cudaMemcpyDeviceToDevice, c->stream));
   MD_CUDA(cudaMemcpyAsync(v0bar, VB, sizeof(double) * n3, cudaMemcpyDeviceToDevice, c->stream));
